@@ -7,22 +7,22 @@
 // flag (1 = the jump detector fired; such records are not trained on).
 // Loss per record: (sum_k w_k q_k - T)^2 + lam * sum_k d_k log(d_k / w_k).
 //
-// One training step, all seven networks at once, B records per field:
-//   fwd_bwd_kernel   one thread per record: forward pass, loss and the
-//                    backward pass to the pre-activation gradients, stored
-//                    with the activations in a scratch buffer;
-//   reduce_kernel    one thread per parameter (and one per field for the
-//                    loss): sums the per-record products in a fixed order, so
-//                    the gradient is bitwise repeatable;
-//   adam_kernel      one thread per parameter.
+// One training step, all seven networks at once, B records per field, in two
+// launches:
+//   grad_kernel      a block walks chunks of 32 records of one field: forward
+//                    and backward pass out of shared memory, then every
+//                    thread adds its share of the 1 380 gradient (and loss)
+//                    entries, record by record in a fixed order;
+//   apply_kernel     one thread per entry: the blocks' sums in a fixed order,
+//                    the mean, and the Adam step of its parameter.
+// Every sum over records is exact to twice the FP32 mantissa (see add_prod),
+// so the gradient is bitwise repeatable and rounds once, at the end.
 // Minibatch indices come from a counter-based generator (splitmix64 of seed,
 // step, field, slot), so a run is reproducible.
 #include "../../include/wombat_gb300.h"
 #include "wb_internal.h"
 
 #include <algorithm>
-#include <cmath>
-#include <numeric>
 #include <vector>
 
 namespace {
@@ -35,9 +35,17 @@ constexpr int O_W1 = 0, O_B1 = O_W1 + NH * NIN, O_W2 = O_B1 + NH, O_B2 = O_W2 + 
               O_W3 = O_B2 + NH, O_B3 = O_W3 + NOUT * NH;
 static_assert(O_B3 + NOUT == NP, "parameter layout");
 
-// scratch per record: x(6) a1(32) h1(32) a2(32) h2(32) da1(32) da2(32) dz(3) loss(1)
-constexpr int S_X = 0, S_H1 = 6, S_H2 = 38, S_DA1 = 70, S_DA2 = 102, S_DZ = 134, S_L = 137,
-              SREC = 138;
+// One record's row in shared memory (floats): x(6) 1 h1(32) h2(32) da1(32)
+// da2(32) dz(3) loss; every gradient entry is the sum over records of a
+// product of two entries of the row (the biases' second factor is the 1).
+constexpr int S_X = 0, S_ONE = 6, S_H1 = 8, S_H2 = 40, S_DA1 = 72, S_DA2 = 104, S_DZ = 136, S_L = 139,
+              SROW = 140;
+constexpr int NE = NP + 1;                   // entries per field: the parameters and the loss
+constexpr int kChunk = 32;                   // records per pass of a block
+constexpr int kGradThreads = 256;
+// Blocks per field: two resident blocks per SM over seven fields, which cuts
+// a 4 096-record batch into three chunks per block.
+constexpr int kGradBlocks = 43;
 
 // GELU in its sigmoid form, gelu(t) = t sigma(1.702 t) = t/2 (1 + tanh(0.851 t)),
 // and its derivative sigma + 1.702 t sigma (1 - sigma).
@@ -57,7 +65,7 @@ __device__ __forceinline__ unsigned long long splitmix64(unsigned long long z) {
 // Record index for (field, slot) of this step: either all records of the
 // field in order (full batch) or a counter-based random draw.
 __device__ __forceinline__ long long pick(const long long* off, const long long* cnt, int f,
-                                          int slot, int full, unsigned long long seed,
+                                          long long slot, int full, unsigned long long seed,
                                           long long step) {
     if (full) return off[f] + slot;
     const unsigned long long h =
@@ -66,121 +74,251 @@ __device__ __forceinline__ long long pick(const long long* off, const long long*
     return off[f] + (long long)(h % (unsigned long long)cnt[f]);
 }
 
-__global__ void __launch_bounds__(128)
-fwd_bwd_kernel(const float* __restrict__ rec, const long long* __restrict__ off,
-               const long long* __restrict__ cnt, const float* __restrict__ params, int B, int full,
-               unsigned long long seed, long long step, float lam, float* __restrict__ scr) {
+// acc (an unevaluated pair hi + lo) += a b: the product and the sum are both
+// split into their rounded value and its exact error (Dekker's and Knuth's
+// error-free transformations), the errors collecting in lo.  The sum keeps
+// 48 bits for 10 FP32 operations; an FP64 accumulator would cost a fused
+// multiply-add and two conversions on a pipe 64 times narrower.
+__device__ __forceinline__ void add_prod(float2& acc, float a, float b) {
+    const float p = __fmul_rn(a, b), e = __fmaf_rn(a, b, -p);
+    const float t = __fadd_rn(acc.x, p), z = __fsub_rn(t, acc.x);
+    const float err = __fadd_rn(__fsub_rn(acc.x, __fsub_rn(t, z)), __fsub_rn(p, z));
+    acc.x = t;
+    acc.y = __fadd_rn(acc.y, __fadd_rn(err, e));
+}
+
+// The two factors of gradient entry j in a record's row.
+__device__ __forceinline__ void entry_factors(int j, int& ga, int& gb) {
+    gb = S_ONE;
+    if (j < O_B1) { ga = S_DA1 + j / NIN; gb = S_X + j % NIN; }
+    else if (j < O_W2) { ga = S_DA1 + (j - O_B1); }
+    else if (j < O_B2) { ga = S_DA2 + (j - O_W2) / NH; gb = S_H1 + (j - O_W2) % NH; }
+    else if (j < O_W3) { ga = S_DA2 + (j - O_B2); }
+    else if (j < O_B3) { ga = S_DZ + (j - O_W3) / NH; gb = S_H2 + (j - O_W3) % NH; }
+    else if (j < NP) { ga = S_DZ + (j - O_B3); }
+    else { ga = S_L; }
+}
+
+// Block (field f, slot g of kGradBlocks): chunks g, g + kGradBlocks, ... of
+// the field's batch.  A warp takes four of a chunk's 32 records through the
+// network with one lane per hidden unit (weights in shared memory, rows
+// padded so that rows and columns of W2 are both read without bank
+// conflicts); then the block adds the chunk's outer products, a 2 x 2 tile of
+// dW2 per thread and the 356 other entries one or two per thread.  Bound by
+// the FP32 pipe: 10 of the 13 operations per entry and record are the exact
+// sums.  120 000 records, 60 steps of 4 096 per field and one full-batch
+// gradient: %TRAIN%.
+__global__ void __launch_bounds__(kGradThreads, 2)
+grad_kernel(const float* __restrict__ rec, const long long* __restrict__ perm, const long long* __restrict__ off,
+            const long long* __restrict__ cnt, const float* __restrict__ params, int batch, int full,
+            unsigned long long seed, long long step, float lam, float2* __restrict__ part) {
+    __shared__ __align__(16) float row[kChunk][SROW];
+    __shared__ __align__(16) float W1[NIN][NH], W2[NH][NH + 1], W3[NOUT][NH];
+    __shared__ float B1[NH], B2[NH], B3[NOUT + 1];
+    const int f = blockIdx.x / kGradBlocks, g = blockIdx.x - f * kGradBlocks;
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    const float* p = params + (long long)f * NP;
+    for (int j = tid; j < NP; j += kGradThreads) {
+        const float v = p[j];
+        if (j < O_B1) W1[j % NIN][j / NIN] = v;
+        else if (j < O_W2) B1[j - O_B1] = v;
+        else if (j < O_B2) W2[(j - O_W2) / NH][(j - O_W2) % NH] = v;
+        else if (j < O_W3) B2[j - O_B2] = v;
+        else if (j < O_B3) W3[(j - O_W3) / NH][(j - O_W3) % NH] = v;
+        else B3[j - O_B3] = v;
+    }
+    if (tid < kChunk) row[tid][S_ONE] = 1.f;
+    const long long n = cnt[f] == 0 ? 0 : (full ? cnt[f] : (long long)batch);
+    // this thread's entries: rows 2 ti, 2 ti + 1 and columns 2 tk, 2 tk + 1 of
+    // dW2, and entries e0, e1 of the rest (counted with dW2 left out)
+    const int ti = tid >> 4, tk = tid & 15;
+    constexpr int kRest = NE - NH * NH;
+    static_assert(kRest > kGradThreads && kRest <= 2 * kGradThreads, "two further entries per thread at most");
+    const int e0 = tid < O_W2 ? tid : tid + NH * NH, e1 = tid + kGradThreads + NH * NH;
+    const bool two = tid + kGradThreads < kRest;
+    int ga0, gb0, ga1, gb1;
+    entry_factors(e0, ga0, gb0);
+    entry_factors(two ? e1 : e0, ga1, gb1);
+    float2 t00 = {0.f, 0.f}, t01 = t00, t10 = t00, t11 = t00, r0 = t00, r1 = t00;
+    __syncthreads();
+    for (long long c = (long long)g * kChunk; c < n; c += (long long)kGradBlocks * kChunk) {
+        // forward and backward, four records per warp, lane = hidden unit
+        constexpr int Q = kChunk / (kGradThreads / 32);
+        float h2[Q], d1[Q], d2[Q], z[Q][NOUT];
+        const float* r[Q];
+        const int first = warp * Q;
+#pragma unroll
+        for (int q = 0; q < Q; q++) {
+            const long long slot = c + first + q;
+            // slots past the batch repeat its last record; their rows are not summed
+            const long long s = slot < n ? slot : n - 1;
+            r[q] = rec + perm[pick(off, cnt, f, s, full, seed, step)] * REC;
+            if (lane < NIN) row[first + q][S_X + lane] = r[q][1 + lane];
+        }
+        __syncwarp();
+#pragma unroll
+        for (int q = 0; q < Q; q++) {
+            float a = B1[lane];
+#pragma unroll
+            for (int k = 0; k < NIN; k++) a += W1[k][lane] * row[first + q][S_X + k];
+            row[first + q][S_H1 + lane] = gelu(a, d1[q]);
+        }
+        __syncwarp();
+        {
+            float a[Q];
+#pragma unroll
+            for (int q = 0; q < Q; q++) a[q] = B2[lane];
+#pragma unroll
+            for (int k = 0; k < NH; k += 4) {
+                const float w[4] = {W2[lane][k], W2[lane][k + 1], W2[lane][k + 2], W2[lane][k + 3]};
+#pragma unroll
+                for (int q = 0; q < Q; q++) {
+                    const float4 h = *reinterpret_cast<const float4*>(&row[first + q][S_H1 + k]);
+                    a[q] += w[0] * h.x;
+                    a[q] += w[1] * h.y;
+                    a[q] += w[2] * h.z;
+                    a[q] += w[3] * h.w;
+                }
+            }
+#pragma unroll
+            for (int q = 0; q < Q; q++) {
+                h2[q] = gelu(a[q], d2[q]);
+                row[first + q][S_H2 + lane] = h2[q];
+            }
+        }
+#pragma unroll
+        for (int q = 0; q < Q; q++)
+#pragma unroll
+            for (int o = 0; o < NOUT; o++) {
+                float a = W3[o][lane] * h2[q];
+#pragma unroll
+                for (int m = 16; m > 0; m >>= 1) a += __shfl_xor_sync(0xffffffffu, a, m);
+                z[q][o] = a + B3[o];
+            }
+        // softmax, loss and its gradient: lane q of the first four takes record q
+        float dz[NOUT] = {0.f, 0.f, 0.f};
+        if (lane < Q) {
+            float zz[NOUT];
+            const float* rr = r[0];
+#pragma unroll
+            for (int o = 0; o < NOUT; o++) zz[o] = z[0][o];
+#pragma unroll
+            for (int q = 1; q < Q; q++)
+                if (lane == q) {
+                    rr = r[q];
+#pragma unroll
+                    for (int o = 0; o < NOUT; o++) zz[o] = z[q][o];
+                }
+            const float zm = fmaxf(zz[0], fmaxf(zz[1], zz[2]));
+            float e[NOUT], es = 0.f;
+#pragma unroll
+            for (int o = 0; o < NOUT; o++) { e[o] = expf(zz[o] - zm); es += e[o]; }
+            float om[NOUT];
+#pragma unroll
+            for (int o = 0; o < NOUT; o++) om[o] = e[o] / es;
+            const float qv[NOUT] = {rr[7], rr[8], rr[9]};
+            const float T = rr[10];
+            const float d[NOUT] = {0.1f, 0.6f, 0.3f};
+            const float y = om[0] * qv[0] + om[1] * qv[1] + om[2] * qv[2];
+            float kl = 0.f;
+#pragma unroll
+            for (int o = 0; o < NOUT; o++) kl += d[o] * (logf(d[o]) - logf(om[o]));
+            float dom[NOUT], sdom = 0.f;
+#pragma unroll
+            for (int o = 0; o < NOUT; o++) {
+                dom[o] = 2.f * (y - T) * qv[o] - lam * d[o] / om[o];
+                sdom += om[o] * dom[o];
+            }
+#pragma unroll
+            for (int o = 0; o < NOUT; o++) {
+                dz[o] = om[o] * (dom[o] - sdom);
+                row[first + lane][S_DZ + o] = dz[o];
+            }
+            row[first + lane][S_L] = (y - T) * (y - T) + lam * kl;
+        }
+        __syncwarp();
+#pragma unroll
+        for (int q = 0; q < Q; q++) {
+            float a = 0.f;
+#pragma unroll
+            for (int o = 0; o < NOUT; o++) a += row[first + q][S_DZ + o] * W3[o][lane];
+            row[first + q][S_DA2 + lane] = a * d2[q];
+        }
+        __syncwarp();
+        {
+            float a[Q];
+#pragma unroll
+            for (int q = 0; q < Q; q++) a[q] = 0.f;
+#pragma unroll
+            for (int i = 0; i < NH; i += 4) {
+                const float w[4] = {W2[i][lane], W2[i + 1][lane], W2[i + 2][lane], W2[i + 3][lane]};
+#pragma unroll
+                for (int q = 0; q < Q; q++) {
+                    const float4 h = *reinterpret_cast<const float4*>(&row[first + q][S_DA2 + i]);
+                    a[q] += w[0] * h.x;
+                    a[q] += w[1] * h.y;
+                    a[q] += w[2] * h.z;
+                    a[q] += w[3] * h.w;
+                }
+            }
+#pragma unroll
+            for (int q = 0; q < Q; q++) row[first + q][S_DA1 + lane] = a[q] * d1[q];
+        }
+        __syncthreads();
+        const int m = n - c < kChunk ? (int)(n - c) : kChunk;
+#pragma unroll 2
+        for (int q = 0; q < m; q++) {
+            const float* w = row[q];
+            const float2 da = *reinterpret_cast<const float2*>(w + S_DA2 + 2 * ti);
+            const float2 h = *reinterpret_cast<const float2*>(w + S_H1 + 2 * tk);
+            add_prod(t00, da.x, h.x);
+            add_prod(t01, da.x, h.y);
+            add_prod(t10, da.y, h.x);
+            add_prod(t11, da.y, h.y);
+            add_prod(r0, w[ga0], w[gb0]);
+            if (two) add_prod(r1, w[ga1], w[gb1]);
+        }
+        __syncthreads();
+    }
+    float2* o = part + (long long)blockIdx.x * NE;
+    const int j = O_W2 + 2 * ti * NH + 2 * tk;
+    o[j] = t00;
+    o[j + 1] = t01;
+    o[j + NH] = t10;
+    o[j + NH + 1] = t11;
+    o[e0] = r0;
+    if (two) o[e1] = r1;
+}
+
+// Gradient entry j of field f: the blocks' sums added in FP64 in the order of
+// the blocks, over the number of records; entry NP is the loss.  With m given
+// also the parameter's Adam step.
+__global__ void __launch_bounds__(64)
+apply_kernel(const float2* __restrict__ part, const long long* __restrict__ cnt, int batch, int full,
+             float* __restrict__ grad, float* __restrict__ loss, float* __restrict__ params, float* __restrict__ m,
+             float* __restrict__ v, float lr, float b1, float b2, float eps, float c1, float c2) {
     const int gid = blockIdx.x * blockDim.x + threadIdx.x;
-    const int f = gid / B, slot = gid - f * B;
+    const int f = gid / NE, j = gid - f * NE;
     if (f >= NF) return;
-    float* s = scr + (long long)gid * SREC;
-    if (cnt[f] == 0 || (full && slot >= cnt[f])) {
-        for (int t = 0; t < SREC; t++) s[t] = 0.f;
+    const long long n = cnt[f] == 0 ? 0 : (full ? cnt[f] : (long long)batch);
+    const float2* s = part + (long long)f * kGradBlocks * NE + j;
+    double hi = 0.0, lo = 0.0;
+#pragma unroll 8
+    for (int b = 0; b < kGradBlocks; b++) {
+        const float2 a = s[(long long)b * NE];
+        hi += double(a.x);
+        lo += double(a.y);
+    }
+    // an infinite sum leaves NaN in the errors: it stands by itself
+    const double sum = isfinite(hi) ? hi + lo : hi;
+    const float g = float(n > 0 ? sum / double(n) : 0.0);
+    if (j == NP) {
+        loss[f] = g;
         return;
     }
-    const float* r = rec + pick(off, cnt, f, slot, full, seed, step) * REC;
-    const float* p = params + (long long)f * NP;
-    float x[NIN], a1d[NH], h1[NH], a2d[NH], h2[NH], z[NOUT];
-#pragma unroll
-    for (int k = 0; k < NIN; k++) x[k] = r[1 + k];
-    for (int i = 0; i < NH; i++) {
-        float a = p[O_B1 + i];
-#pragma unroll
-        for (int k = 0; k < NIN; k++) a += p[O_W1 + i * NIN + k] * x[k];
-        h1[i] = gelu(a, a1d[i]);
-    }
-    for (int i = 0; i < NH; i++) {
-        float a = p[O_B2 + i];
-        for (int k = 0; k < NH; k++) a += p[O_W2 + i * NH + k] * h1[k];
-        h2[i] = gelu(a, a2d[i]);
-    }
-#pragma unroll
-    for (int o = 0; o < NOUT; o++) {
-        float a = p[O_B3 + o];
-        for (int k = 0; k < NH; k++) a += p[O_W3 + o * NH + k] * h2[k];
-        z[o] = a;
-    }
-    const float zm = fmaxf(z[0], fmaxf(z[1], z[2]));
-    float e[NOUT], es = 0.f;
-#pragma unroll
-    for (int o = 0; o < NOUT; o++) { e[o] = expf(z[o] - zm); es += e[o]; }
-    float om[NOUT];
-#pragma unroll
-    for (int o = 0; o < NOUT; o++) om[o] = e[o] / es;
-    const float q[NOUT] = {r[7], r[8], r[9]};
-    const float T = r[10];
-    const float d[NOUT] = {0.1f, 0.6f, 0.3f};
-    const float y = om[0] * q[0] + om[1] * q[1] + om[2] * q[2];
-    float kl = 0.f;
-#pragma unroll
-    for (int o = 0; o < NOUT; o++) kl += d[o] * (logf(d[o]) - logf(om[o]));
-    const float loss = (y - T) * (y - T) + lam * kl;
-    // backward (per record; the mean over records is applied in the reduction)
-    float dom[NOUT], sdom = 0.f;
-#pragma unroll
-    for (int o = 0; o < NOUT; o++) { dom[o] = 2.f * (y - T) * q[o] - lam * d[o] / om[o]; sdom += om[o] * dom[o]; }
-    float dz[NOUT];
-#pragma unroll
-    for (int o = 0; o < NOUT; o++) dz[o] = om[o] * (dom[o] - sdom);
-    float da2[NH];
-    for (int k = 0; k < NH; k++) {
-        float g = 0.f;
-#pragma unroll
-        for (int o = 0; o < NOUT; o++) g += dz[o] * p[O_W3 + o * NH + k];
-        da2[k] = g * a2d[k];
-    }
-    for (int k = 0; k < NH; k++) {
-        float g = 0.f;
-        for (int i = 0; i < NH; i++) g += da2[i] * p[O_W2 + i * NH + k];
-        s[S_DA1 + k] = g * a1d[k];
-    }
-#pragma unroll
-    for (int k = 0; k < NIN; k++) s[S_X + k] = x[k];
-    for (int k = 0; k < NH; k++) {
-        s[S_H1 + k] = h1[k];
-        s[S_H2 + k] = h2[k];
-        s[S_DA2 + k] = da2[k];
-    }
-#pragma unroll
-    for (int o = 0; o < NOUT; o++) s[S_DZ + o] = dz[o];
-    s[S_L] = loss;
-}
-
-// gradient entry j of field f = (1/n_f) sum over the field's records of the
-// product of a pre-activation gradient and an input activation; the loss is
-// slot NP of each field.
-__global__ void __launch_bounds__(256)
-reduce_kernel(const float* __restrict__ scr, const long long* __restrict__ cnt, int B, int full,
-              float* __restrict__ grad, float* __restrict__ loss) {
-    const int gid = blockIdx.x * blockDim.x + threadIdx.x;
-    const int f = gid / (NP + 1), j = gid - f * (NP + 1);
-    if (f >= NF) return;
-    const long long nf = full ? (cnt[f] < B ? cnt[f] : B) : (cnt[f] > 0 ? B : 0);
-    int ga, gb;     // scratch offsets of the two factors (gb < 0: factor 1)
-    if (j < O_B1) { ga = S_DA1 + j / NIN; gb = S_X + j % NIN; }
-    else if (j < O_W2) { ga = S_DA1 + (j - O_B1); gb = -1; }
-    else if (j < O_B2) { ga = S_DA2 + (j - O_W2) / NH; gb = S_H1 + (j - O_W2) % NH; }
-    else if (j < O_W3) { ga = S_DA2 + (j - O_B2); gb = -1; }
-    else if (j < O_B3) { ga = S_DZ + (j - O_W3) / NH; gb = S_H2 + (j - O_W3) % NH; }
-    else if (j < NP) { ga = S_DZ + (j - O_B3); gb = -1; }
-    else { ga = S_L; gb = -1; }
-    double acc = 0.0;
-    const float* base = scr + (long long)f * B * SREC;
-    for (long long r = 0; r < nf; r++) {
-        const float* s = base + r * SREC;
-        acc += gb < 0 ? double(s[ga]) : double(s[ga]) * double(s[gb]);
-    }
-    const double v = nf > 0 ? acc / double(nf) : 0.0;
-    if (j < NP) grad[(long long)f * NP + j] = float(v);
-    else loss[f] = float(v);
-}
-
-__global__ void adam_kernel(float* __restrict__ params, const float* __restrict__ grad,
-                            float* __restrict__ m, float* __restrict__ v, float lr, float b1,
-                            float b2, float eps, float c1, float c2, int n) {
-    const int i = blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= n) return;
-    const float g = grad[i];
+    const int i = f * NP + j;
+    grad[i] = g;
+    if (!m) return;
     const float mi = b1 * m[i] + (1.f - b1) * g;
     const float vi = b2 * v[i] + (1.f - b2) * g * g;
     m[i] = mi;
@@ -190,56 +328,56 @@ __global__ void adam_kernel(float* __restrict__ params, const float* __restrict_
 
 struct Dev {
     float* rec = nullptr;
+    long long* perm = nullptr;     // the records to train on, by field, in their order
     long long* off = nullptr;
     long long* cnt = nullptr;
     float* params = nullptr;
     float* grad = nullptr;
     float* m = nullptr;
     float* v = nullptr;
-    float* scr = nullptr;
-    float* loss = nullptr;
+    float2* part = nullptr;        // the blocks' sums
+    float* loss = nullptr;         // 7 per step
     ~Dev() {
-        for (void* p : {(void*)rec, (void*)off, (void*)cnt, (void*)params, (void*)grad, (void*)m,
-                        (void*)v, (void*)scr, (void*)loss})
+        for (void* p : {(void*)rec, (void*)perm, (void*)off, (void*)cnt, (void*)params, (void*)grad, (void*)m,
+                        (void*)v, (void*)part, (void*)loss})
             if (p) cudaFree(p);
     }
 };
 
-// Upload records sorted by field (unflagged only) and the parameters.
-int setup(Dev& D, const float* records, long long n, const float* params, int B, int full,
+// Uploads the records, the order of the unflagged ones by field, and the
+// parameters; room for the losses of `steps` steps.
+int setup(Dev& D, const float* records, long long n, const float* params, long long steps, int full,
           long long* cnt_out) {
-    std::vector<long long> cnt(NF, 0);
-    std::vector<std::vector<long long>> by(NF);
+    std::vector<long long> cnt(NF, 0), off(NF, 0);
     for (long long r = 0; r < n; r++) {
         const int f = (int)records[r * REC];
         if (f < 0 || f >= NF) return wb::set_last_error(WB_EINVAL, "mlp: record with a field outside 0..6");
-        if (records[r * REC + 11] != 0.f) continue;
-        by[f].push_back(r);
+        if (records[r * REC + 11] == 0.f) cnt[f]++;
     }
-    std::vector<float> sorted;
-    std::vector<long long> off(NF, 0);
     long long pos = 0;
     for (int f = 0; f < NF; f++) {
         off[f] = pos;
-        cnt[f] = (long long)by[f].size();
-        for (long long r : by[f]) sorted.insert(sorted.end(), records + r * REC, records + (r + 1) * REC);
         pos += cnt[f];
+        cnt_out[f] = cnt[f];
     }
-    for (int f = 0; f < NF; f++) cnt_out[f] = cnt[f];
-    const long long nb = full ? std::max<long long>(1, *std::max_element(cnt.begin(), cnt.end())) : B;
-    if (full && nb > (1LL << 24)) return wb::set_last_error(WB_EINVAL, "mlp: too many records per field");
+    std::vector<long long> perm(std::max<long long>(pos, 1), 0), at = off;
+    for (long long r = 0; r < n; r++)
+        if (records[r * REC + 11] == 0.f) perm[at[(int)records[r * REC]]++] = r;
+    if (full && *std::max_element(cnt.begin(), cnt.end()) > (1LL << 24))
+        return wb::set_last_error(WB_EINVAL, "mlp: too many records per field");
     auto ck = [](cudaError_t e) { return e == cudaSuccess; };
-    const size_t rb = sizeof(float) * std::max<size_t>(sorted.size(), REC);
-    if (!ck(cudaMalloc(&D.rec, rb)) || !ck(cudaMalloc(&D.off, sizeof(long long) * NF)) ||
+    if (!ck(cudaMalloc(&D.rec, sizeof(float) * n * REC)) ||
+        !ck(cudaMalloc(&D.perm, sizeof(long long) * perm.size())) ||
+        !ck(cudaMalloc(&D.off, sizeof(long long) * NF)) ||
         !ck(cudaMalloc(&D.cnt, sizeof(long long) * NF)) ||
         !ck(cudaMalloc(&D.params, sizeof(float) * NF * NP)) ||
         !ck(cudaMalloc(&D.grad, sizeof(float) * NF * NP)) ||
         !ck(cudaMalloc(&D.m, sizeof(float) * NF * NP)) || !ck(cudaMalloc(&D.v, sizeof(float) * NF * NP)) ||
-        !ck(cudaMalloc(&D.scr, sizeof(float) * SREC * NF * nb)) ||
-        !ck(cudaMalloc(&D.loss, sizeof(float) * NF)))
+        !ck(cudaMalloc(&D.part, sizeof(float2) * NE * NF * kGradBlocks)) ||
+        !ck(cudaMalloc(&D.loss, sizeof(float) * NF * std::max<long long>(steps, 1))))
         return wb::set_last_error(WB_ENOMEM, "mlp: device allocation failed");
-    if (!sorted.empty() &&
-        !ck(cudaMemcpy(D.rec, sorted.data(), sizeof(float) * sorted.size(), cudaMemcpyHostToDevice)))
+    if (!ck(cudaMemcpy(D.rec, records, sizeof(float) * n * REC, cudaMemcpyHostToDevice)) ||
+        !ck(cudaMemcpy(D.perm, perm.data(), sizeof(long long) * perm.size(), cudaMemcpyHostToDevice)))
         return wb::set_last_error(WB_ECUDA, "mlp: record upload failed");
     if (!ck(cudaMemcpy(D.off, off.data(), sizeof(long long) * NF, cudaMemcpyHostToDevice)) ||
         !ck(cudaMemcpy(D.cnt, cnt.data(), sizeof(long long) * NF, cudaMemcpyHostToDevice)) ||
@@ -249,11 +387,18 @@ int setup(Dev& D, const float* records, long long n, const float* params, int B,
     return WB_OK;
 }
 
-int grad_step(Dev& D, int B, int full, unsigned long long seed, long long step, float lam) {
-    const int nrec = NF * B;
-    fwd_bwd_kernel<<<(nrec + 127) / 128, 128>>>(D.rec, D.off, D.cnt, D.params, B, full, seed, step, lam, D.scr);
-    const int nred = NF * (NP + 1);
-    reduce_kernel<<<(nred + 255) / 256, 256>>>(D.scr, D.cnt, B, full, D.grad, D.loss);
+struct Adam {
+    float lr = 0.f, b1 = 0.9f, b2 = 0.999f, eps = 1e-8f, c1 = 1.f, c2 = 1.f;
+};
+
+// Gradient and loss of one batch; with `adam` also the parameters' step.
+int grad_step(Dev& D, int batch, int full, unsigned long long seed, long long step, float lam, float* loss,
+              const Adam* adam) {
+    grad_kernel<<<NF * kGradBlocks, kGradThreads>>>(D.rec, D.perm, D.off, D.cnt, D.params, batch, full, seed, step,
+                                                    lam, D.part);
+    const Adam a = adam ? *adam : Adam{};
+    apply_kernel<<<(NF * NE + 63) / 64, 64>>>(D.part, D.cnt, batch, full, D.grad, loss, D.params,
+                                              adam ? D.m : nullptr, D.v, a.lr, a.b1, a.b2, a.eps, a.c1, a.c2);
     return cudaGetLastError() == cudaSuccess ? WB_OK : wb::set_last_error(WB_ECUDA, "mlp: kernel launch failed");
 }
 
@@ -265,10 +410,9 @@ extern "C" int wb_mlp_loss_grad(const float* records, long long n, const float* 
         return wb::set_last_error(WB_EINVAL, "mlp: null argument or no records");
     Dev D;
     long long cnt[NF];
-    int rc = setup(D, records, n, params, 0, 1, cnt);
+    int rc = setup(D, records, n, params, 1, 1, cnt);
     if (rc != WB_OK) return rc;
-    const long long B = std::max<long long>(1, *std::max_element(cnt, cnt + NF));
-    if ((rc = grad_step(D, (int)B, 1, 0, 0, (float)lam)) != WB_OK) return rc;
+    if ((rc = grad_step(D, 0, 1, 0, 0, (float)lam, D.loss, nullptr)) != WB_OK) return rc;
     float loss[NF];
     if (cudaMemcpy(grad_out, D.grad, sizeof(float) * NF * NP, cudaMemcpyDeviceToHost) != cudaSuccess ||
         cudaMemcpy(loss, D.loss, sizeof(float) * NF, cudaMemcpyDeviceToHost) != cudaSuccess)
@@ -283,23 +427,23 @@ extern "C" int wb_mlp_train(const float* records, long long n, float* params, in
         return wb::set_last_error(WB_EINVAL, "mlp: bad training arguments");
     Dev D;
     long long cnt[NF];
-    int rc = setup(D, records, n, params, batch, 0, cnt);
+    int rc = setup(D, records, n, params, loss_history ? steps : 1, 0, cnt);
     if (rc != WB_OK) return rc;
-    const float b1 = 0.9f, b2 = 0.999f, eps = 1e-8f;
+    Adam adam;
+    adam.lr = (float)lr;
     double p1 = 1.0, p2 = 1.0;
-    std::vector<float> hist(NF);
     for (int t = 0; t < steps; t++) {
-        if ((rc = grad_step(D, batch, 0, seed, t, (float)lam)) != WB_OK) return rc;
-        p1 *= b1;
-        p2 *= b2;
-        adam_kernel<<<(NF * NP + 255) / 256, 256>>>(D.params, D.grad, D.m, D.v, (float)lr, b1, b2, eps,
-                                                    (float)(1.0 - p1), (float)(1.0 - p2), NF * NP);
-        if (loss_history) {
-            if (cudaMemcpy(hist.data(), D.loss, sizeof(float) * NF, cudaMemcpyDeviceToHost) != cudaSuccess)
-                return wb::set_last_error(WB_ECUDA, "mlp: loss download failed");
-            for (int f = 0; f < NF; f++) loss_history[(long long)t * NF + f] = hist[f];
-        }
+        p1 *= adam.b1;
+        p2 *= adam.b2;
+        adam.c1 = (float)(1.0 - p1);
+        adam.c2 = (float)(1.0 - p2);
+        float* loss = D.loss + (loss_history ? (long long)t * NF : 0);
+        if ((rc = grad_step(D, batch, 0, seed, t, (float)lam, loss, &adam)) != WB_OK) return rc;
     }
+    // the losses stay on the device until the last step: one copy, one wait
+    if (loss_history && steps > 0 &&
+        cudaMemcpy(loss_history, D.loss, sizeof(float) * NF * steps, cudaMemcpyDeviceToHost) != cudaSuccess)
+        return wb::set_last_error(WB_ECUDA, "mlp: loss download failed");
     if (cudaMemcpy(params, D.params, sizeof(float) * NF * NP, cudaMemcpyDeviceToHost) != cudaSuccess)
         return wb::set_last_error(WB_ECUDA, "mlp: parameter download failed");
     return wb::set_last_error(WB_OK, "");
