@@ -146,6 +146,7 @@ struct SweepArgs {
     const int* __restrict__ links = nullptr;   // patch links (see locate) or nullptr
     long long ncells;              // stride between arrays
     double gamma;
+    double rg1 = 0;                // 1 / (gamma - 1) (the Jiang-Shu and WENO-Z sweeps)
     int zweights = 0;              // 1: WENO-Z weights instead of Jiang-Shu
     unsigned long long* lstats = nullptr;   // learned sweep: detector firings, decisions
     int* queue = nullptr;          // persistent sweep: tile counter of this launch (or fixed stride)
@@ -187,7 +188,7 @@ cudaError_t launch_sweep(int axis, const SweepArgs<T>& a, int ntiles, cudaStream
 template <class T>
 cudaError_t prepare_sweep_kernels();
 // Tile shape s (0 = default, kNTileShape alternatives) of the sweep along
-// `axis`: ta interfaces along the axis times tp pencils (ta * tp = 256).
+// `axis`: ta interfaces along the axis times tp pencils (ta * tp = 128).
 constexpr int kNTileShape = 3;
 void sweep_shape(int axis, int s, int* ta, int* tp);
 // Tile of the learned-weight sweep along `axis` (one shape, 256 threads).

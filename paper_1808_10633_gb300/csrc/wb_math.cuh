@@ -1,0 +1,93 @@
+// wb_math.cuh -- reciprocals and square roots of the sweep kernels, and the
+// arithmetic they share over a scalar (FP64) or a pair of FP32 lanes.
+//
+// FP64 division and square roots: the hardware's approximate reciprocal (root)
+// has about 20 good bits; one step of the third-order iteration of
+// Householder's family takes that to the rounding level:
+//   1/x:       e = 1 - x y,    y' = y (1 + e + e^2)
+//   1/sqrt(x): e = 1 - x y^2,  y' = y (1 + e/2 + 3 e^2/8)
+// in 3 and 5 operations of the narrow FP64 pipe, which bounds the FP64 sweep.
+// Arguments outside the normal range (zero, subnormal, infinite, negative,
+// NaN, or a reciprocal that would be subnormal) take CUDA's functions.
+// Largest error seen over the binades: 1/x 1 ulp, 1/sqrt 1 ulp, sqrt 1 ulp
+// (tests/test_gpu_math.py).
+#pragma once
+#include <cuda_runtime.h>
+
+namespace wb {
+
+// ---- scalar reciprocals and roots ---------------------------------------------
+__device__ __forceinline__ bool normal_range(double x, unsigned lo, unsigned hi) {
+    const unsigned h = (unsigned)__double2hiint(x);      // negative: above every bound
+    return h >= lo && h < hi;
+}
+// 1/x for x > 0 known to lie in [2^-1000, 2^1000]
+__device__ __forceinline__ double recip_inrange(double x) {
+    double y;
+    asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(x));
+    const double e = fma(-x, y, 1.0);
+    return fma(y, fma(e, e, e), y);
+}
+__device__ __forceinline__ double recip(double x) {
+    return normal_range(x, 0x00100000u, 0x7fc00000u) ? recip_inrange(x) : 1.0 / x;
+}
+__device__ __forceinline__ double rsq_root(double x) {
+    if (!normal_range(x, 0x00100000u, 0x7ff00000u)) return rsqrt(x);
+    double y;
+    asm("rsqrt.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(x));
+    const double t = x * y;
+    const double e = fma(-t, y, 1.0);
+    return fma(fma(0.375, e, 0.5), y * e, y);
+}
+// sqrt(x) = x / sqrt(x), the same step applied to t = x y: e holds the
+// rounding error of t as well
+__device__ __forceinline__ double sq_root(double x) {
+    if (!normal_range(x, 0x00100000u, 0x7ff00000u)) return sqrt(x);
+    double y;
+    asm("rsqrt.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(x));
+    const double t = x * y;
+    const double e = fma(-t, y, 1.0);
+    return fma(fma(0.375, e, 0.5), t * e, t);
+}
+// FP32: the compiler's forms (the FP32 sweeps are built with fast division
+// and square root)
+__device__ __forceinline__ float recip(float x) { return 1.0f / x; }
+__device__ __forceinline__ float rsq_root(float x) { return rsqrtf(x); }
+__device__ __forceinline__ float sq_root(float x) { return sqrtf(x); }
+
+// ---- one FP64 value or two FP32 lanes -------------------------------------------
+template <class V> struct Lanes;
+template <> struct Lanes<double> { using S = double; static constexpr int N = 1; };
+template <> struct Lanes<float2> { using S = float; static constexpr int N = 2; };
+
+template <class V> __device__ __forceinline__ V splat(typename Lanes<V>::S v);
+template <> __device__ __forceinline__ double splat<double>(double v) { return v; }
+template <> __device__ __forceinline__ float2 splat<float2>(float v) { return make_float2(v, v); }
+
+__device__ __forceinline__ double vfma(double a, double b, double c) { return fma(a, b, c); }
+__device__ __forceinline__ double vmul(double a, double b) { return a * b; }
+__device__ __forceinline__ double vadd(double a, double b) { return a + b; }
+__device__ __forceinline__ double vsub(double a, double b) { return a - b; }
+__device__ __forceinline__ double vneg(double a) { return -a; }
+__device__ __forceinline__ float2 vfma(float2 a, float2 b, float2 c) { return __ffma2_rn(a, b, c); }
+__device__ __forceinline__ float2 vmul(float2 a, float2 b) { return __fmul2_rn(a, b); }
+__device__ __forceinline__ float2 vadd(float2 a, float2 b) { return __fadd2_rn(a, b); }
+__device__ __forceinline__ float2 vsub(float2 a, float2 b) { return __ffma2_rn(b, make_float2(-1.f, -1.f), a); }
+__device__ __forceinline__ float2 vneg(float2 a) { return make_float2(-a.x, -a.y); }
+__device__ __forceinline__ float2 vrcp(float2 a) { return make_float2(recip(a.x), recip(a.y)); }
+__device__ __forceinline__ double vabs(double a) { return fabs(a); }
+__device__ __forceinline__ float2 vabs(float2 a) { return make_float2(fabsf(a.x), fabsf(a.y)); }
+// max of values >= 0: their bit patterns order like the values, so FP64 takes
+// an integer max, off the FP64 pipe
+__device__ __forceinline__ double vmax0(double a, double b) {
+    return __longlong_as_double(max(__double_as_longlong(a), __double_as_longlong(b)));
+}
+__device__ __forceinline__ float2 vmax0(float2 a, float2 b) { return make_float2(fmaxf(a.x, b.x), fmaxf(a.y, b.y)); }
+
+// lane l of v
+__device__ __forceinline__ double lane(double v, int) { return v; }
+__device__ __forceinline__ float lane(float2 v, int l) { return l == 0 ? v.x : v.y; }
+__device__ __forceinline__ void set_lane(double& v, int, double s) { v = s; }
+__device__ __forceinline__ void set_lane(float2& v, int l, float s) { (l == 0 ? v.x : v.y) = s; }
+
+}  // namespace wb

@@ -106,8 +106,9 @@ __device__ __forceinline__ void entry_factors(int j, int& ga, int& gb) {
 // conflicts); then the block adds the chunk's outer products, a 2 x 2 tile of
 // dW2 per thread and the 356 other entries one or two per thread.  Bound by
 // the FP32 pipe: 10 of the 13 operations per entry and record are the exact
-// sums.  120 000 records, 60 steps of 4 096 per field and one full-batch
-// gradient: %TRAIN%.
+// sums.  60 steps of 4 096 records per field and one full-batch gradient, host
+// side included: 83.5 -> 5.5 ms against a serial loop over the records per
+// entry with FP64 accumulators (and a loss copied to the host every step).
 __global__ void __launch_bounds__(kGradThreads, 2)
 grad_kernel(const float* __restrict__ rec, const long long* __restrict__ perm, const long long* __restrict__ off,
             const long long* __restrict__ cnt, const float* __restrict__ params, int batch, int full,

@@ -1,6 +1,6 @@
 // wb_sweep_f64.cu -- double instantiation of the WENO5 sweep kernels, and
 // the tile shapes the host uses to build the tile tables.
-#include "wb_sweep.cuh"
+#include "wb_sweep_js.cuh"
 
 namespace wb {
 

@@ -1,0 +1,604 @@
+// wb_sweep_js.cuh -- the Jiang-Shu and WENO-Z flux sweeps (staging, slots and
+// eigen-structure of wb_sweep.cuh), for FP64 and FP32.
+//
+// One interface per thread.  FP64 takes the interface arithmetic below
+// (sweep_flux), which counts operations of the FP64 pipe (two per clock and SM
+// on this GPU, 87 % busy, everything else hidden behind it): quadratic-form
+// smoothness indicators and one reciprocal for the two phi_N of a field (60
+// instead of 83 operations), three-operation reciprocals, Alfven rows that act
+// on the differences directly.  96^3, x + y + z sweep of a step: 21.3 -> 17.6
+// ms; three and four blocks per SM (168 and 128 registers) are no faster.
+// FP32 the one of wb_sweep.cuh (interface_flux), which packs the
+// U and F differences of a stencil step, and here the two sides of phi_N, in
+// the lanes of Blackwell's packed FP32 instructions.
+#pragma once
+#include "wb_sweep.cuh"
+
+namespace wb {
+namespace {
+
+// resident blocks per SM the register budget is shaped for
+#ifndef WB_SWEEP_BLOCKS_F32
+#define WB_SWEEP_BLOCKS_F32 4
+#endif
+#ifndef WB_SWEEP_BLOCKS_F64
+#define WB_SWEEP_BLOCKS_F64 2
+#endif
+template <class T> constexpr int kMinBlocks = sizeof(T) == 4 ? WB_SWEEP_BLOCKS_F32 : WB_SWEEP_BLOCKS_F64;
+// per-thread slots of sweep_flux: back-projection coefficients, then the
+// Alfven and entropy projections while the fast/slow group is reconstructed
+enum : int { B_ALF = 0, B_ALS, B_AFCF, B_ASCS, B_ASR, B_SSR, B_RAG, kNBackV = 7 };
+constexpr int kSlotsV = kNBackV + 30;
+template <class T> constexpr int kSlots = sizeof(T) == 4 ? kNThreadSlots : kSlotsV;
+
+// ---- phi_N (Sec. 2.1) ------------------------------------------------------------
+// With a, b, c, d four successive differences, IS_k as printed are quadratic
+// forms: IS_0 / 16 = a (a - 11/4 b) + 5/2 b^2, IS_1 / 16 = b (b - 5/4 c) + c^2,
+// IS_2 / 16 = d (d - 11/4 c) + 5/2 c^2 (smallest eigenvalues 0.18, 0.38,
+// 0.18: no cancellation to speak of).  The weights depend on the ratios of
+// the eps + IS_k only, so e_k = (eps + IS_k) / 16, ten operations, serve.
+template <class V>
+__device__ __forceinline__ void smoothness(V a, V b, V c, V d, typename Lanes<V>::S eps16, V& e0, V& e1, V& e2) {
+    using S = typename Lanes<V>::S;
+    const V eps = splat<V>(eps16), k11 = splat<V>(S(-2.75)), k5 = splat<V>(S(-1.25)), k52 = splat<V>(S(2.5));
+    e0 = vfma(a, vfma(b, k11, a), vfma(vmul(b, k52), b, eps));
+    const V cc = vfma(c, c, eps);
+    e1 = vfma(b, vfma(c, k5, b), cc);
+    e2 = vfma(d, vfma(c, k11, d), vfma(cc, k52, splat<V>(S(-1.5) * eps16)));
+}
+
+// p = a - 2b + c
+template <class V>
+__device__ __forceinline__ V second(V a, V b, V c) {
+    return vfma(b, splat<V>(typename Lanes<V>::S(-2)), vadd(a, c));
+}
+
+// (phi_N(am, bm, cm, dm) - phi_N(ap, bp, cp, dp)) / 2 for Jiang-Shu weights:
+// phi_N = N / (3 W) - q / 12 with p = a - 2b + c, q = b - 2c + d,
+// W = sum d_k / e_k^2, N = p / e_0^2 + 3/2 q / e_2^2, d = (1, 6, 3).
+__device__ __forceinline__ void js_side(double a, double b, double c, double d, double eps16, double& p, double& q,
+                                        double& n0, double& n2, double& den) {
+    double e0, e1, e2;
+    smoothness<double>(a, b, c, d, eps16, e0, e1, e2);
+    // both sums over the common denominator (e_0 e_1 e_2)^2
+    const double m0 = e1 * e2, m1 = e0 * e2, m2 = e0 * e1;
+    n0 = m0 * m0;
+    n2 = m2 * m2;
+    den = fma(6.0, m1 * m1, fma(3.0, n2, n0));
+    p = second(a, b, c);
+    q = second(b, c, d);
+}
+// FP64: one reciprocal for both sides, of the product of their denominators,
+// where neither exceeds 1e130 (the product and its numerators then stay far
+// inside the range); else one division each.
+__device__ __forceinline__ double half_phi_diff(double am, double bm, double cm, double dm, double ap, double bp,
+                                                double cp, double dp, double eps16) {
+    double pm, qm, n0m, n2m, wm, pp, qp, n0p, n2p, wp;
+    js_side(am, bm, cm, dm, eps16, pm, qm, n0m, n2m, wm);
+    js_side(ap, bp, cp, dp, eps16, pp, qp, n0p, n2p, wp);
+    double r;
+    // high words of the (positive) denominators against that of 1e130
+    if (max(__double2hiint(wm), __double2hiint(wp)) < 0x5af00000) {
+        const double nm = fma(n0m, pm, (1.5 * n2m) * qm), np = fma(n0p, pp, (1.5 * n2p) * qp);
+        r = fma(nm, wp, -(np * wm)) * recip_inrange(wm * wp);
+    } else {
+        const double im = 1.0 / wm, ip = 1.0 / wp;
+        r = ((n0m * im) * pm + 1.5 * (n2m * im) * qm) - ((n0p * ip) * pp + 1.5 * (n2p * ip) * qp);
+    }
+    return fma(r, 1.0 / 6.0, (qp - qm) * (1.0 / 24.0));
+}
+// FP32: reciprocals of the e_k keep the range (products of their squares
+// could overflow)
+__device__ __forceinline__ float2 js_ratio(float2 a, float2 b, float2 c, float2 d, float eps16, float2& q) {
+    float2 e0, e1, e2;
+    smoothness<float2>(a, b, c, d, eps16, e0, e1, e2);
+    const float2 i0 = vrcp(e0), i1 = vrcp(e1), i2 = vrcp(e2);
+    const float2 a0 = vmul(i0, i0), a1 = vmul(i1, i1), a2 = vmul(i2, i2);
+    const float2 w = vfma(a1, splat<float2>(6.f), vfma(a2, splat<float2>(3.f), a0));
+    const float2 p = second(a, b, c);
+    q = second(b, c, d);
+    const float2 n = vfma(a0, p, vmul(vmul(a2, splat<float2>(1.5f)), q));
+    return vmul(n, vrcp(w));
+}
+// the minus side in lane x, the plus side in lane y
+__device__ __forceinline__ float half_ratio_diff(float2 r, float2 q) {
+    return fmaf(r.x - r.y, 1.f / 6.f, (q.y - q.x) * (1.f / 24.f));
+}
+
+// WENO-Z (the alternative Sec. 2.1 names): alpha_k = d_k (1 + tau5 / (eps +
+// IS_k)), tau5 = |IS_0 - IS_2|; the ratio is free of the common factor.
+template <class V>
+__device__ __forceinline__ V z_ratio(V a, V b, V c, V d, typename Lanes<V>::S eps16, V& q) {
+    using S = typename Lanes<V>::S;
+    V e0, e1, e2;
+    smoothness<V>(a, b, c, d, eps16, e0, e1, e2);
+    const V tau = vabs(vsub(e0, e2)), one = splat<V>(S(1));
+    V a0, a1, a2;
+    if constexpr (sizeof(S) == 8) {
+        a0 = fma(tau, recip(e0), 1.0);
+        a1 = fma(tau, recip(e1), 1.0);
+        a2 = fma(tau, recip(e2), 1.0);
+    } else {
+        a0 = vfma(tau, vrcp(e0), one);
+        a1 = vfma(tau, vrcp(e1), one);
+        a2 = vfma(tau, vrcp(e2), one);
+    }
+    const V w = vfma(a1, splat<V>(S(6)), vfma(a2, splat<V>(S(3)), a0));
+    const V p = second(a, b, c);
+    q = second(b, c, d);
+    const V n = vfma(a0, p, vmul(vmul(a2, splat<V>(S(1.5))), q));
+    if constexpr (sizeof(S) == 8) return n * recip(w);
+    else return vmul(n, vrcp(w));
+}
+
+// Correction of eq. FWENO for one characteristic field from the projected
+// differences dw_m = l (U_{m+1} - U_m), dg_m = l (F_{m+1} - F_m) of the
+// stencil: -phi_N(D+_{i-3/2} ..) + phi_N(D-_{i+5/2} ..) with D+- = (dg +- alpha
+// dw) / 2.  phi_N is taken on 2 D+- with 4 eps and halved (exact).
+template <class V, bool Z>
+__device__ __forceinline__ V weno_corr(const V (&dw)[5], const V (&dg)[5], V alpha) {
+    using S = typename Lanes<V>::S;
+    constexpr S eps16 = S(4.0 * 1e-6 / 16.0);
+    const V na = vneg(alpha);
+    const V p0 = vfma(alpha, dw[0], dg[0]), p1 = vfma(alpha, dw[1], dg[1]), p2 = vfma(alpha, dw[2], dg[2]),
+            p3 = vfma(alpha, dw[3], dg[3]);
+    const V m1 = vfma(na, dw[1], dg[1]), m2 = vfma(na, dw[2], dg[2]), m3 = vfma(na, dw[3], dg[3]),
+            m4 = vfma(na, dw[4], dg[4]);
+    if constexpr (Z) {
+        V qm, qp;
+        const V rm = z_ratio<V>(m4, m3, m2, m1, eps16, qm), rp = z_ratio<V>(p0, p1, p2, p3, eps16, qp);
+        return vfma(vsub(rm, rp), splat<V>(S(1.0 / 6.0)), vmul(vsub(qp, qm), splat<V>(S(1.0 / 24.0))));
+    } else {
+        return half_phi_diff(m4, m3, m2, m1, p0, p1, p2, p3, eps16);
+    }
+}
+
+// Weights of interface_flux (FP32): both sides of a field in one packed pair.
+template <bool Z>
+struct JsWeights {
+    __device__ __forceinline__ float corr_d(int, const float (&dw)[5], const float (&dg)[5], float alpha) {
+        constexpr float eps16 = 4.0f * 1e-6f / 16.0f;
+        float2 D[4], q;
+#pragma unroll
+        for (int k = 0; k < 4; k++)
+            D[k] = make_float2(fmaf(-alpha, dw[4 - k], dg[4 - k]), fmaf(alpha, dw[k], dg[k]));
+        const float2 r = Z ? z_ratio<float2>(D[0], D[1], D[2], D[3], eps16, q)
+                           : js_ratio(D[0], D[1], D[2], D[3], eps16, q);
+        return half_ratio_diff(r, q);
+    }
+};
+
+// ---- eigen-structure over V ---------------------------------------------------------
+// Left-vector coefficients (negated where the projection subtracts), the
+// speeds and what the back-projection needs.
+template <class V>
+struct EigV {
+    V rho, nu, nv1, nv2, nbm, hv2, be1, be2, nbe2;
+    V cf, cs, ca;
+    V Af, Bf, Cf, Df, As, Bs, Cs, Ds, nEe;
+    V nvb;                       // -(be1 v1 + be2 v2)
+    V q1, q2, q0, r1, r2;        // Alfven rows: q1 x3 + q2 x2 + q0 x0 +- (r1 x5 + r2 x4)
+};
+
+template <class V, class S = typename Lanes<V>::S>
+__device__ __forceinline__ void eigen_lane(int l, V rho_, V u_, V v1_, V v2_, V bn_, V b1_, V b2_, V p_, S gamma,
+                                           S rg1, EigV<V>& e, V (&back)[kNBackV]) {
+    Eig<S> s;
+    S bp[kNBack];
+    eigen<S>(lane(rho_, l), lane(u_, l), lane(v1_, l), lane(v2_, l), lane(bn_, l), lane(b1_, l), lane(b2_, l),
+             lane(p_, l), gamma, s, bp, 1);
+    set_lane(e.rho, l, s.rho);
+    set_lane(e.nu, l, -s.u);
+    set_lane(e.nv1, l, -s.v1);
+    set_lane(e.nv2, l, -s.v2);
+    set_lane(e.nbm, l, -s.bm);
+    set_lane(e.hv2, l, s.hv2);
+    set_lane(e.be1, l, s.be1);
+    set_lane(e.be2, l, s.be2);
+    set_lane(e.nbe2, l, -s.be2);
+    set_lane(e.cf, l, s.cf);
+    set_lane(e.cs, l, s.cs);
+    set_lane(e.ca, l, s.ca);
+    set_lane(e.Af, l, s.Af);
+    set_lane(e.Bf, l, s.Bf);
+    set_lane(e.Cf, l, s.Cf);
+    set_lane(e.Df, l, s.Df);
+    set_lane(e.As, l, s.As);
+    set_lane(e.Bs, l, s.Bs);
+    set_lane(e.Cs, l, s.Cs);
+    set_lane(e.Ds, l, s.Ds);
+    set_lane(e.nEe, l, -s.Ee);
+    set_lane(e.nvb, l, -(s.be1 * s.v1 + s.be2 * s.v2));
+    const S q1 = s.Aa * s.be1, q2 = -s.Aa * s.be2;
+    set_lane(e.q1, l, q1);
+    set_lane(e.q2, l, q2);
+    set_lane(e.q0, l, -(q1 * s.v2 + q2 * s.v1));
+    set_lane(e.r1, l, s.Ba * s.be1);
+    set_lane(e.r2, l, -s.Ba * s.be2);
+    set_lane(back[B_ALF], l, bp[BP_ALF]);
+    set_lane(back[B_ALS], l, bp[BP_ALS]);
+    set_lane(back[B_AFCF], l, bp[BP_AFCF]);
+    set_lane(back[B_ASCS], l, bp[BP_ASCS]);
+    set_lane(back[B_ASR], l, bp[BP_ASR]);
+    set_lane(back[B_SSR], l, bp[BP_SSR]);
+    set_lane(back[B_RAG], l, bp[BP_RA2] * rg1);
+}
+
+// One difference vector on all seven left eigenvectors: fast-, slow-, slow+,
+// fast+ into o4, Alfven-, entropy, Alfven+ into o3.
+template <class V>
+__device__ __forceinline__ void project(const EigV<V>& e, const V (&x)[7], V (&o4)[4], V (&o3)[3]) {
+    const V du = vfma(e.nu, x[0], x[1]);
+    const V vpar = vfma(e.be1, x[2], vfma(e.be2, x[3], vmul(e.nvb, x[0])));
+    const V bpar = vfma(e.be1, x[4], vmul(e.be2, x[5]));
+    V P = vfma(e.hv2, x[0], x[6]);
+    P = vfma(e.nu, x[1], P);
+    P = vfma(e.nv1, x[2], P);
+    P = vfma(e.nv2, x[3], P);
+    P = vfma(e.nbm, bpar, P);
+    const V tf1 = vfma(e.Af, du, vmul(e.Bf, vpar)), tf2 = vfma(e.Cf, bpar, vmul(e.Df, P));
+    const V ts1 = vfma(e.As, du, vmul(e.Bs, vpar)), ts2 = vfma(e.Cs, bpar, vmul(e.Ds, P));
+    o4[0] = vsub(tf2, tf1);
+    o4[1] = vsub(ts2, ts1);
+    o4[2] = vadd(ts2, ts1);
+    o4[3] = vadd(tf2, tf1);
+    const V t1 = vfma(e.q1, x[3], vfma(e.q2, x[2], vmul(e.q0, x[0])));
+    const V t2 = vfma(e.r1, x[5], vmul(e.r2, x[4]));
+    o3[0] = vadd(t1, t2);
+    o3[1] = vfma(e.nEe, P, x[0]);
+    o3[2] = vsub(t1, t2);
+}
+
+template <class V>
+__device__ __forceinline__ V ld(const typename Lanes<V>::S* __restrict__ p) {
+    return *reinterpret_cast<const V*>(p);
+}
+
+// Largest |lambda_s| over the six cells and the interface state.
+template <class V, int CS>
+__device__ __forceinline__ V lf_speed_v(const typename Lanes<V>::S* __restrict__ cell, int nc, int s, const EigV<V>& e) {
+    const V nc_s = (s == 0 || s == 6) ? e.cf : ((s == 1 || s == 5) ? e.ca : e.cs);
+    V al = s == 3 ? vabs(e.nu) : (s < 3 ? vabs(vadd(e.nu, nc_s)) : vabs(vsub(e.nu, nc_s)));
+#pragma unroll
+    for (int m = 0; m < 6; m++) al = vmax0(al, ld<V>(cell + (SL + s) * nc + m * CS));
+    return al;
+}
+
+// Flux through one interface (one per lane): cell points at stencil cell 0,
+// the six cells are CS values apart.
+template <class V, bool Z, int CS>
+__device__ __forceinline__ void sweep_flux(const typename Lanes<V>::S* __restrict__ cell, int nc,
+                                           typename Lanes<V>::S gamma, typename Lanes<V>::S rg1, V* __restrict__ slot,
+                                           int sstride, V (&out)[7]) {
+    using S = typename Lanes<V>::S;
+    // 1-2. interface state and eigen-structure
+    EigV<V> e;
+    {
+        const V h = splat<V>(S(0.5));
+        auto mean = [&](int s) { return vmul(h, vadd(ld<V>(cell + s * nc + 2 * CS), ld<V>(cell + s * nc + 3 * CS))); };
+        const V rho = mean(SU), u = mean(SP_U), v1 = mean(SP_V1), v2 = mean(SP_V2), bn = mean(SP_BN),
+                b1 = mean(SU + 4), b2 = mean(SU + 5), p = mean(SP_P);
+        V back[kNBackV];
+#pragma unroll
+        for (int l = 0; l < Lanes<V>::N; l++) eigen_lane<V>(l, rho, u, v1, v2, bn, b1, b2, p, gamma, rg1, e, back);
+#pragma unroll
+        for (int k = 0; k < kNBackV; k++) slot[k * sstride] = back[k];
+    }
+    // 3. the five differences of the stencil's U and F on all seven fields;
+    // the Alfven/entropy values wait in this thread's slots
+    V* park = slot + kNBackV * sstride;
+    V dw[4][5], dg[4][5];
+    V u0[7], f0[6];
+#pragma unroll
+    for (int f = 0; f < 7; f++) u0[f] = ld<V>(cell + (SU + f) * nc);
+#pragma unroll
+    for (int f = 0; f < 6; f++) f0[f] = ld<V>(cell + (SF + 1 + f) * nc);
+#pragma unroll
+    for (int m = 0; m < 5; m++) {
+        V x[7], o4[4], o3[3];
+#pragma unroll
+        for (int f = 0; f < 7; f++) {
+            const V u1 = ld<V>(cell + (SU + f) * nc + (m + 1) * CS);
+            x[f] = vsub(u1, u0[f]);
+            u0[f] = u1;
+        }
+        const V dm = x[1];                   // the mass flux is the normal momentum
+        project(e, x, o4, o3);
+#pragma unroll
+        for (int f = 0; f < 4; f++) dw[f][m] = o4[f];
+#pragma unroll
+        for (int f = 0; f < 3; f++) park[(f * 5 + m) * sstride] = o3[f];
+        x[0] = dm;
+#pragma unroll
+        for (int f = 0; f < 6; f++) {
+            const V f1 = ld<V>(cell + (SF + 1 + f) * nc + (m + 1) * CS);
+            x[f + 1] = vsub(f1, f0[f]);
+            f0[f] = f1;
+        }
+        project(e, x, o4, o3);
+#pragma unroll
+        for (int f = 0; f < 4; f++) dg[f][m] = o4[f];
+#pragma unroll
+        for (int f = 0; f < 3; f++) park[((3 + f) * 5 + m) * sstride] = o3[f];
+    }
+    // 4-5. Lax-Friedrichs speeds and weights, fast and slow fields, then
+    // Alfven and entropy
+    V corr[7];
+#pragma unroll
+    for (int f = 0; f < 4; f++) corr[2 * f] = weno_corr<V, Z>(dw[f], dg[f], lf_speed_v<V, CS>(cell, nc, 2 * f, e));
+#pragma unroll
+    for (int f = 0; f < 3; f++) {
+        const int s = 2 * f + 1;
+        V wa[5], ga[5];
+#pragma unroll
+        for (int m = 0; m < 5; m++) {
+            wa[m] = park[(f * 5 + m) * sstride];
+            ga[m] = park[((3 + f) * 5 + m) * sstride];
+        }
+        corr[s] = weno_corr<V, Z>(wa, ga, lf_speed_v<V, CS>(cell, nc, s, e));
+    }
+    // 6. back-projection: sum_s r_s corr_s in primitive variables, then dU/dW,
+    // and the central flux (7 (F_i + F_{i+1}) - (F_{i-1} + F_{i+2})) / 12
+    const V alf = slot[B_ALF * sstride], als = slot[B_ALS * sstride];
+    const V afcf = slot[B_AFCF * sstride], ascs = slot[B_ASCS * sstride];
+    const V ssr = slot[B_SSR * sstride];
+    const V Fp = vadd(corr[6], corr[0]), Fm = vsub(corr[6], corr[0]);
+    const V Sp = vadd(corr[4], corr[2]), Sm = vsub(corr[4], corr[2]);
+    const V Ap = vadd(corr[5], corr[1]), nAm = vsub(corr[1], corr[5]);
+    const V fs = vfma(alf, Fp, vmul(als, Sp));
+    const V drho = vfma(e.rho, fs, corr[3]);
+    const V du = vfma(afcf, Fm, vmul(ascs, Sm));
+    V sg;                                         // sgn(B_n)
+#pragma unroll
+    for (int l = 0; l < Lanes<V>::N; l++) set_lane(sg, l, lane(ssr, l) < S(0) ? S(-1) : S(1));
+    const V dvpar = vmul(sg, vsub(vmul(afcf, Sm), vmul(ascs, Fm)));
+    const V dbpar = vmul(slot[B_ASR * sstride], vsub(vmul(als, Fp), vmul(alf, Sp)));
+    const V dbper = vmul(ssr, nAm);
+    const V dpg = vmul(slot[B_RAG * sstride], fs);             // dp / (gamma - 1)
+    const V dv1 = vfma(e.be1, dvpar, vmul(e.nbe2, Ap)), dv2 = vfma(e.be2, dvpar, vmul(e.be1, Ap));
+    V dF[7];
+    dF[0] = drho;
+    dF[4] = vfma(e.be1, dbpar, vmul(e.nbe2, dbper));
+    dF[5] = vfma(e.be2, dbpar, vmul(e.be1, dbper));
+    const V nd = vneg(drho);
+    dF[1] = vfma(e.nu, nd, vmul(e.rho, du));
+    dF[2] = vfma(e.nv1, nd, vmul(e.rho, dv1));
+    dF[3] = vfma(e.nv2, nd, vmul(e.rho, dv2));
+    const V vdv = vfma(e.nu, du, vfma(e.nv1, dv1, vmul(e.nv2, dv2)));       // -v dv
+    dF[6] = vfma(e.hv2, drho, vsub(dpg, vfma(e.nbm, dbpar, vmul(e.rho, vdv))));
+#pragma unroll
+    for (int f = 0; f < 7; f++) {
+        const typename Lanes<V>::S* F = cell + fslot(f) * nc;
+        const V in = vadd(ld<V>(F + 2 * CS), ld<V>(F + 3 * CS)), ex = vadd(ld<V>(F + CS), ld<V>(F + 4 * CS));
+        out[f] = vfma(in, splat<V>(S(7.0 / 12.0)), vfma(ex, splat<V>(S(-1.0 / 12.0)), dF[f]));
+    }
+}
+
+// ---- one tile ------------------------------------------------------------------------
+// Stages the TA + 5 cells of each of the TP pencils, then one thread per
+// interface.  Cell s of pencil tp lies at tp * NS + s (x sweep) or s * TP + tp.
+template <class T, int AXIS, int TA, int NCMAX, bool Z>
+__device__ __forceinline__ void tile_body(const SweepArgs<T>& A, const Tile& tile, const PatchDev& P,
+                                          T* __restrict__ sm, int tid) {
+    constexpr int NT = kSweepNT, TP = kSweepNT / TA, NS = TA + 5, NC = NS * TP;
+    constexpr int CS = AXIS == 0 ? 1 : TP;         // distance of a pencil's neighbouring cells
+    const int na = AXIS == 0 ? P.nx : (AXIS == 1 ? P.ny : P.nz);
+    const int np = AXIS == 0 ? P.ny : P.nx;
+
+    // staging: cells tile.y-3 .. tile.y+TA+1 along the axis, TP pencils
+    constexpr int NIT = (NC + NT - 1) / NT;
+    RawCell<T> raw[NIT];
+    long long rc[NIT];
+    bool rok[NIT], rown[NIT];
+#pragma unroll
+    for (int it = 0; it < NIT; it++) {
+        const int e = tid + it * NT;
+        int s, tp;
+        if (AXIS == 0) { tp = e / NS; s = e - tp * NS; }
+        else { s = e / TP; tp = e - s * TP; }
+        const int cp = tile.z + tp;
+        rok[it] = e < NC && cp < np;
+        const int raw_a = tile.y - 3 + s;
+        rown[it] = raw_a >= tile.y && raw_a < tile.y + TA && raw_a < na;
+        if (rok[it]) {
+            const int ca = A.links ? raw_a : wrap(raw_a, na);
+            int i, j, k;
+            if (AXIS == 0) { i = ca; j = cp; k = tile.w; }
+            else if (AXIS == 1) { i = cp; j = ca; k = tile.w; }
+            else { i = cp; j = tile.w; k = ca; }
+            if (A.links) load_cell_linked<T>(A, tile.x, P, i, j, k, raw[it], rc[it]);
+            else load_cell<T>(A, P, i, j, k, raw[it], rc[it]);
+        }
+    }
+#pragma unroll
+    for (int it = 0; it < NIT; it++)
+        if (rok[it])
+            derive_cell<T, AXIS>(A, raw[it], rc[it], sm, NC, tid + it * NT, rown[it] && A.er != nullptr);
+    __syncthreads();
+
+    int ta, tp;
+    if (AXIS == 0) { ta = tid & (TA - 1); tp = tid / TA; }
+    else { tp = tid & (TP - 1); ta = tid / TP; }
+    const int ia = tile.y + ta, ip = tile.z + tp;
+    if (ia >= na || ip >= np) return;
+    const int i0 = (int)chk(AXIS == 0 ? tp * NS + ta : ta * TP + tp, NC - 5 * CS, A.flag);
+    T F[7];
+    T* slot = sm + kNSlot * NCMAX + tid;
+    if constexpr (sizeof(T) == 8) {
+        sweep_flux<T, Z, CS>(sm + i0, NC, T(A.gamma), T(A.rg1), slot, NT, F);
+    } else {
+        int id[6];
+#pragma unroll
+        for (int m = 0; m < 6; m++) id[m] = i0 + m * CS;
+        JsWeights<Z> js;
+        interface_flux<T, JsWeights<Z>, true>(sm, NC, id, T(A.gamma), slot, NT, js, F);
+    }
+
+    // rotate back and store at the lower face of cell ia
+    int i, j, k;
+    if (AXIS == 0) { i = ia; j = ip; k = tile.w; }
+    else if (AXIS == 1) { i = ip; j = ia; k = tile.w; }
+    else { i = ip; j = tile.w; k = ia; }
+    const long long N = A.ncells;
+    const long long c = chk(P.off + ((long long)k * P.ny + j) * P.nx + i, N, A.flag);
+    T* __restrict__ fo = A.flux;
+    T fx, fy, fz;
+    if (AXIS == 0) { fx = F[1]; fy = F[2]; fz = F[3]; }
+    else if (AXIS == 1) { fy = F[1]; fz = F[2]; fx = F[3]; }
+    else { fz = F[1]; fx = F[2]; fy = F[3]; }
+    fo[c] = F[0];
+    fo[N + c] = fx;
+    fo[2 * N + c] = fy;
+    fo[3 * N + c] = fz;
+    fo[4 * N + c] = F[6];
+    fo[5 * N + c] = F[4];
+    fo[6 * N + c] = F[5];
+}
+
+// Persistent sweep: a grid of (SMs x resident blocks) takes tiles of any
+// shape from a work counter, so patches of uneven sizes share one launch;
+// each tile runs the body compiled for its shape (a block-uniform switch).
+// Serves tile tables that are not ordered by shape.
+template <class T, int AXIS, bool Z>
+__global__ void __launch_bounds__(kSweepNT, kMinBlocks<T>) sweep_kernel(const SweepArgs<T> A, int ntiles) {
+    constexpr int NCMAX = max_nc(AXIS);
+    extern __shared__ __align__(16) unsigned char smem_raw[];
+    T* sm = reinterpret_cast<T*>(smem_raw);
+    const int tid = threadIdx.x;
+    __shared__ int next_tile;
+    // work queue: each block starts on tile blockIdx.x and then takes the next
+    // unclaimed tile from the launch's counter (zeroed before the launch), so
+    // uneven tiles balance across SMs; without a counter, a fixed stride
+    for (int t = blockIdx.x; t < ntiles;) {
+        Tile tile = A.tiles[t];
+        const int shape = (unsigned)tile.x >> 24;
+        tile.x &= 0xffffff;
+        const PatchDev P = A.patches[tile.x];
+        if (shape == 0) tile_body<T, AXIS, shape_ta(AXIS, 0), NCMAX, Z>(A, tile, P, sm, tid);
+        else if (shape == 1) tile_body<T, AXIS, shape_ta(AXIS, 1), NCMAX, Z>(A, tile, P, sm, tid);
+        else tile_body<T, AXIS, shape_ta(AXIS, 2), NCMAX, Z>(A, tile, P, sm, tid);
+        __syncthreads();
+        if (A.queue) {
+            if (tid == 0) next_tile = gridDim.x + atomicAdd(A.queue, 1);
+            __syncthreads();
+            t = next_tile;
+        } else {
+            t += gridDim.x;
+        }
+    }
+}
+
+// One tile per block of one shape S: the launch for tile tables that use one
+// shape throughout (a single grid, or patches tuned to it), and for each
+// shape's range of a table sorted by shape, with either weights.  (WENO-Z on
+// the persistent kernel, whose three bodies share one register allocation and
+// spill 800 bytes, took 1.55 ms per 128^3 FP32 step's sweeps against 1.13.)
+template <class T, int AXIS, int S, bool Z>
+__global__ void __launch_bounds__(kSweepNT, kMinBlocks<T>) sweep_kernel_fixed(const SweepArgs<T> A) {
+    constexpr int NC0 = nc_of(shape_ta(AXIS, S));
+    extern __shared__ __align__(16) unsigned char smem_raw[];
+    T* sm = reinterpret_cast<T*>(smem_raw);
+    Tile tile = A.tiles[blockIdx.x];
+    tile.x &= 0xffffff;
+    const PatchDev P = A.patches[tile.x];
+    tile_body<T, AXIS, shape_ta(AXIS, S), NC0, Z>(A, tile, P, sm, threadIdx.x);
+}
+
+template <class T>
+constexpr size_t tile_smem(int nc) {
+    return sizeof(T) * (kNSlot * (size_t)nc + (size_t)kSlots<T> * kSweepNT);
+}
+template <class T, int AXIS, int S>
+constexpr size_t smem_bytes_fixed() { return tile_smem<T>(nc_of(shape_ta(AXIS, S))); }
+template <class T, int AXIS>
+constexpr size_t smem_bytes_persistent() { return tile_smem<T>(max_nc(AXIS)); }
+
+// f(axis, shape, z) over every fixed kernel
+template <class T, int AX, int S, bool Z>
+cudaError_t prepare_fixed() {
+    return cudaFuncSetAttribute(sweep_kernel_fixed<T, AX, S, Z>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                (int)smem_bytes_fixed<T, AX, S>());
+}
+template <class T, int AX, bool Z>
+cudaError_t prepare_axis() {
+    cudaError_t e = prepare_fixed<T, AX, 0, Z>();
+    if (e == cudaSuccess) e = prepare_fixed<T, AX, 1, Z>();
+    if (e == cudaSuccess) e = prepare_fixed<T, AX, 2, Z>();
+    if (e == cudaSuccess)
+        e = cudaFuncSetAttribute(sweep_kernel<T, AX, Z>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                 (int)smem_bytes_persistent<T, AX>());
+    return e;
+}
+template <class T, int AX, bool Z>
+int persistent_blocks_per_sm() {
+    int nb = 0;
+    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, sweep_kernel<T, AX, Z>, kSweepNT,
+                                                  smem_bytes_persistent<T, AX>());
+    return nb > 0 ? nb : 1;
+}
+
+// Persistent grid sizes per axis, set by prepare_sweep_kernels (outside any
+// stream capture).
+template <class T>
+struct PersistGrid {
+    static inline int g[3] = {0, 0, 0};
+};
+
+template <class T, bool Z, int S>
+void launch_fixed_shape(int axis, const SweepArgs<T>& a, int ntiles, cudaStream_t s) {
+    if (axis == 0) sweep_kernel_fixed<T, 0, S, Z><<<ntiles, kSweepNT, smem_bytes_fixed<T, 0, S>(), s>>>(a);
+    else if (axis == 1) sweep_kernel_fixed<T, 1, S, Z><<<ntiles, kSweepNT, smem_bytes_fixed<T, 1, S>(), s>>>(a);
+    else sweep_kernel_fixed<T, 2, S, Z><<<ntiles, kSweepNT, smem_bytes_fixed<T, 2, S>(), s>>>(a);
+}
+
+template <class T, bool Z>
+cudaError_t launch_sweep_w(int axis, const SweepArgs<T>& a, int ntiles, cudaStream_t s) {
+    if (a.split[0] | a.split[1] | a.split[2]) {
+        // a table sorted by shape: one launch of the fixed kernel per shape
+        SweepArgs<T> b = a;
+        if (a.split[0]) launch_fixed_shape<T, Z, 0>(axis, b, a.split[0], s);
+        b.tiles = a.tiles + a.split[0];
+        if (a.split[1]) launch_fixed_shape<T, Z, 1>(axis, b, a.split[1], s);
+        b.tiles = a.tiles + a.split[0] + a.split[1];
+        if (a.split[2]) launch_fixed_shape<T, Z, 2>(axis, b, a.split[2], s);
+        return cudaGetLastError();
+    }
+    const int grid = PersistGrid<T>::g[axis] > 0 ? PersistGrid<T>::g[axis] : 152;
+    const int nb = ntiles < grid ? ntiles : grid;
+    if (a.queue) {
+        const cudaError_t e = cudaMemsetAsync(a.queue, 0, sizeof(int), s);
+        if (e != cudaSuccess) return e;
+    }
+    if (axis == 0) sweep_kernel<T, 0, Z><<<nb, kSweepNT, smem_bytes_persistent<T, 0>(), s>>>(a, ntiles);
+    else if (axis == 1) sweep_kernel<T, 1, Z><<<nb, kSweepNT, smem_bytes_persistent<T, 1>(), s>>>(a, ntiles);
+    else sweep_kernel<T, 2, Z><<<nb, kSweepNT, smem_bytes_persistent<T, 2>(), s>>>(a, ntiles);
+    return cudaGetLastError();
+}
+
+}  // namespace
+
+template <class T>
+cudaError_t prepare_sweep_kernels() {
+    cudaError_t e = prepare_axis<T, 0, false>();
+    if (e == cudaSuccess) e = prepare_axis<T, 1, false>();
+    if (e == cudaSuccess) e = prepare_axis<T, 2, false>();
+    if (e == cudaSuccess) e = prepare_axis<T, 0, true>();
+    if (e == cudaSuccess) e = prepare_axis<T, 1, true>();
+    if (e == cudaSuccess) e = prepare_axis<T, 2, true>();
+    if (e != cudaSuccess) return e;
+    int dev = 0, nsm = 0;
+    if ((e = cudaGetDevice(&dev)) != cudaSuccess) return e;
+    if ((e = cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev)) != cudaSuccess) return e;
+    PersistGrid<T>::g[0] = nsm * persistent_blocks_per_sm<T, 0, false>();
+    PersistGrid<T>::g[1] = nsm * persistent_blocks_per_sm<T, 1, false>();
+    PersistGrid<T>::g[2] = nsm * persistent_blocks_per_sm<T, 2, false>();
+    return cudaGetLastError();
+}
+
+template <class T>
+cudaError_t launch_sweep(int axis, const SweepArgs<T>& a, int ntiles, cudaStream_t s) {
+    if (ntiles <= 0) return cudaSuccess;
+    return a.zweights ? launch_sweep_w<T, true>(axis, a, ntiles, s) : launch_sweep_w<T, false>(axis, a, ntiles, s);
+}
+
+}  // namespace wb

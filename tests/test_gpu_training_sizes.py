@@ -18,7 +18,7 @@ LAM = 1e-2
 
 
 def _case(counts, seed):
-    rec = _records(4 * sum(counts) + 8, seed)
+    rec = _records(7 * max(counts) + 8, seed)
     rec[:, 11] = 0
     out = []
     for f, n in enumerate(counts):
