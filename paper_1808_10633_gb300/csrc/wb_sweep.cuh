@@ -62,6 +62,14 @@ __device__ __forceinline__ int wrap(int v, int n) {
     return r < 0 ? r + n : r;
 }
 
+// The same for v within one period of [0, n) in nearly every call (a tile's
+// halo): no division then.
+__device__ __forceinline__ int wrap_near(int v, int n) {
+    if (v < 0) v += n;
+    else if (v >= n) v -= n;
+    return (unsigned)v < (unsigned)n ? v : wrap(v, n);
+}
+
 // Sec. 2.1: phi_N(a,b,c,d) = 1/3 w0 (a-2b+c) + 1/6 (w2-1/2)(b-2c+d) with
 // IS_0..2 as printed, alpha_k = d_k/(eps+IS_k)^2, d = (1, 6, 3), eps = 1e-6.
 // The weights depend only on the ratios of the eps + IS_k, so each is formed
@@ -129,11 +137,10 @@ struct Eig {
 // slot per thread) while the WENO step runs, to keep registers for it.
 enum : int { BP_ALF = 0, BP_ALS, BP_AFCF, BP_ASCS, BP_ASR, BP_SSR, BP_RA2, BP_IGM1, kNBack = 8 };
 // Per-thread slots after the back-projection ones where the Alfven/entropy
-// projections (3 fields x (w, g) x 5 differences) wait while
-// the fast/slow group is reconstructed, when each stencil vector is
+// split differences (3 fields x 2 sides x the steps the weights read) wait
+// while the fast/slow group is reconstructed, when each stencil vector is
 // projected only once.
-constexpr int kNPark = 30;
-constexpr int kNThreadSlots = kNBack + kNPark;
+constexpr int thread_slots(int steps) { return kNBack + 6 * steps; }
 
 // |lambda_s| of the interface state, s = 0..6 (u-cf, u-ca, u-cs, u, u+cs,
 // u+ca, u+cf)
@@ -511,11 +518,21 @@ __device__ __forceinline__ void interface_flux(const T* __restrict__ sm, int nc,
     }
     T corr[7];
     if constexpr (PARK) {
-        // 3. the five differences of the stencil's U and F, each projected
-        // once onto all seven fields; the Alfven/entropy values wait in
-        // this thread's shared-memory slots
+        // 3. the five differences of the stencil's U and F, each projected once
+        // onto all seven fields; the Alfven/entropy values wait in this
+        // thread's shared-memory slots
+        constexpr bool kSplit = Wt::kSplit;
+        constexpr int K = kSplit ? 4 : 5;      // values per field, twice
         T* park = bp + kNBack * bstride;
-        T dw[4][5], dg[4][5];
+        T fa[4][K], fb[4][K];
+        // 4. kSplit: the projected differences are split at once, 2 D+- = l dF
+        // +- alpha l dU (steps 0..3 and 1..4 of the two sides), which keeps
+        // eight values per field instead of ten; the learned weights read all
+        // five steps of both sides and split them themselves
+        T al[7];
+        if constexpr (kSplit)
+#pragma unroll
+            for (int s = 0; s < 7; s++) al[s] = lf_speed(sm, nc, id, s, lam_avg(e, s));
         // U and F differences of a stencil step as one packed pair
         float2 p0[7];
 #pragma unroll
@@ -529,33 +546,39 @@ __device__ __forceinline__ void interface_flux(const T* __restrict__ sm, int nc,
                 x[f] = __ffma2_rn(p0[f], splat2(-1.0f), p1[f]);
             }
             project_all2(e, x, o4, o3);
+            const int lo = kSplit ? m - 1 : m;
 #pragma unroll
-            for (int f = 0; f < 4; f++) { dw[f][m] = o4[f].x; dg[f][m] = o4[f].y; }
+            for (int f = 0; f < 4; f++) {
+                if (m < K) fa[f][m] = kSplit ? fmaf(al[2 * f], o4[f].x, o4[f].y) : o4[f].x;
+                if (lo >= 0) fb[f][lo] = kSplit ? fmaf(-al[2 * f], o4[f].x, o4[f].y) : o4[f].y;
+            }
 #pragma unroll
             for (int f = 0; f < 3; f++) {
-                park[(f * 5 + m) * bstride] = o3[f].x;
-                park[((3 + f) * 5 + m) * bstride] = o3[f].y;
+                if (m < K) park[(2 * f * K + m) * bstride] = kSplit ? fmaf(al[2 * f + 1], o3[f].x, o3[f].y) : o3[f].x;
+                if (lo >= 0)
+                    park[((2 * f + 1) * K + lo) * bstride] = kSplit ? fmaf(-al[2 * f + 1], o3[f].x, o3[f].y) : o3[f].y;
             }
 #pragma unroll
             for (int f = 0; f < 7; f++) p0[f] = p1[f];
         }
-        // 4-5. fast and slow fields
+        // 5. fast and slow fields, then Alfven and entropy
 #pragma unroll
         for (int f = 0; f < 4; f++) {
             const int s = 2 * f;
-            corr[s] = wt.corr_d(s, dw[f], dg[f], lf_speed(sm, nc, id, s, lam_avg(e, s)));
+            if constexpr (kSplit) corr[s] = wt.corr_s(fa[f], fb[f]);
+            else corr[s] = wt.corr_d(s, fa[f], fb[f], lf_speed(sm, nc, id, s, lam_avg(e, s)));
         }
-        // 4-5. Alfven and entropy fields
 #pragma unroll
         for (int f = 0; f < 3; f++) {
-            T wa[5], ga[5];
+            T pa[K], na[K];
 #pragma unroll
-            for (int m = 0; m < 5; m++) {
-                wa[m] = park[(f * 5 + m) * bstride];
-                ga[m] = park[((3 + f) * 5 + m) * bstride];
+            for (int m = 0; m < K; m++) {
+                pa[m] = park[(2 * f * K + m) * bstride];
+                na[m] = park[((2 * f + 1) * K + m) * bstride];
             }
             const int s = 2 * f + 1;
-            corr[s] = wt.corr_d(s, wa, ga, lf_speed(sm, nc, id, s, lam_avg(e, s)));
+            if constexpr (kSplit) corr[s] = wt.corr_s(pa, na);
+            else corr[s] = wt.corr_d(s, pa, na, lf_speed(sm, nc, id, s, lam_avg(e, s)));
         }
     } else {
     // 3-5. fast and slow fields

@@ -8,9 +8,16 @@
 // instead of 83 operations), three-operation reciprocals, Alfven rows that act
 // on the differences directly.  96^3, x + y + z sweep of a step: 21.3 -> 17.6
 // ms; three and four blocks per SM (168 and 128 registers) are no faster.
-// FP32 the one of wb_sweep.cuh (interface_flux), which packs the
-// U and F differences of a stencil step, and here the two sides of phi_N, in
-// the lanes of Blackwell's packed FP32 instructions.
+// FP32 takes the one of wb_sweep.cuh (interface_flux), which packs the U and F
+// differences of a stencil step, and here the two sides of phi_N, in the lanes
+// of Blackwell's packed FP32 instructions: 1 376 to 1 419 instructions per
+// interface, issued on 60 to 64 % of cycles by sixteen warps per SM.  256^3,
+// x, y, z sweeps of a step: 2.88 / 2.83 / 3.01 -> 2.67 / 2.79 / 2.97 ms.  Two
+// interfaces per thread (neighbouring pencils in the two lanes) need only
+// 1 107 instructions per interface, but 200 to 255 registers: eight warps per
+// SM issue on 41 % of cycles, and with the staging moved to further warps
+// (cp.async, registers split between the warps) on 50 %: 3.1 to 3.5 and 2.6 to
+// 3.0 ms per axis.
 #pragma once
 #include "wb_sweep.cuh"
 
@@ -28,8 +35,8 @@ template <class T> constexpr int kMinBlocks = sizeof(T) == 4 ? WB_SWEEP_BLOCKS_F
 // per-thread slots of sweep_flux: back-projection coefficients, then the
 // Alfven and entropy projections while the fast/slow group is reconstructed
 enum : int { B_ALF = 0, B_ALS, B_AFCF, B_ASCS, B_ASR, B_SSR, B_RAG, kNBackV = 7 };
-constexpr int kSlotsV = kNBackV + 30;
-template <class T> constexpr int kSlots = sizeof(T) == 4 ? kNThreadSlots : kSlotsV;
+constexpr int kSlotsV = kNBackV + 24;
+template <class T> constexpr int kSlots = sizeof(T) == 4 ? thread_slots(4) : kSlotsV;
 
 // ---- phi_N (Sec. 2.1) ------------------------------------------------------------
 // With a, b, c, d four successive differences, IS_k as printed are quadratic
@@ -131,39 +138,33 @@ __device__ __forceinline__ V z_ratio(V a, V b, V c, V d, typename Lanes<V>::S ep
     else return vmul(n, vrcp(w));
 }
 
-// Correction of eq. FWENO for one characteristic field from the projected
-// differences dw_m = l (U_{m+1} - U_m), dg_m = l (F_{m+1} - F_m) of the
-// stencil: -phi_N(D+_{i-3/2} ..) + phi_N(D-_{i+5/2} ..) with D+- = (dg +- alpha
-// dw) / 2.  phi_N is taken on 2 D+- with 4 eps and halved (exact).
+// Correction of eq. FWENO for one characteristic field, -phi_N(D+_{i-3/2} ..) +
+// phi_N(D-_{i+5/2} ..), from the split differences taken twice over, p_m = 2 D+
+// of steps m = 0..3 and n_m = 2 D- of steps m = 1..4 of the stencil: phi_N with
+// 4 eps on them, halved (exact).
 template <class V, bool Z>
-__device__ __forceinline__ V weno_corr(const V (&dw)[5], const V (&dg)[5], V alpha) {
+__device__ __forceinline__ V weno_corr(const V (&p)[4], const V (&n)[4]) {
     using S = typename Lanes<V>::S;
     constexpr S eps16 = S(4.0 * 1e-6 / 16.0);
-    const V na = vneg(alpha);
-    const V p0 = vfma(alpha, dw[0], dg[0]), p1 = vfma(alpha, dw[1], dg[1]), p2 = vfma(alpha, dw[2], dg[2]),
-            p3 = vfma(alpha, dw[3], dg[3]);
-    const V m1 = vfma(na, dw[1], dg[1]), m2 = vfma(na, dw[2], dg[2]), m3 = vfma(na, dw[3], dg[3]),
-            m4 = vfma(na, dw[4], dg[4]);
     if constexpr (Z) {
         V qm, qp;
-        const V rm = z_ratio<V>(m4, m3, m2, m1, eps16, qm), rp = z_ratio<V>(p0, p1, p2, p3, eps16, qp);
+        const V rm = z_ratio<V>(n[3], n[2], n[1], n[0], eps16, qm), rp = z_ratio<V>(p[0], p[1], p[2], p[3], eps16, qp);
         return vfma(vsub(rm, rp), splat<V>(S(1.0 / 6.0)), vmul(vsub(qp, qm), splat<V>(S(1.0 / 24.0))));
     } else {
-        return half_phi_diff(m4, m3, m2, m1, p0, p1, p2, p3, eps16);
+        return half_phi_diff(n[3], n[2], n[1], n[0], p[0], p[1], p[2], p[3], eps16);
     }
 }
 
 // Weights of interface_flux (FP32): both sides of a field in one packed pair.
 template <bool Z>
 struct JsWeights {
-    __device__ __forceinline__ float corr_d(int, const float (&dw)[5], const float (&dg)[5], float alpha) {
+    static constexpr bool kSplit = true;
+    __device__ __forceinline__ float corr_s(const float (&p)[4], const float (&n)[4]) {
         constexpr float eps16 = 4.0f * 1e-6f / 16.0f;
-        float2 D[4], q;
-#pragma unroll
-        for (int k = 0; k < 4; k++)
-            D[k] = make_float2(fmaf(-alpha, dw[4 - k], dg[4 - k]), fmaf(alpha, dw[k], dg[k]));
-        const float2 r = Z ? z_ratio<float2>(D[0], D[1], D[2], D[3], eps16, q)
-                           : js_ratio(D[0], D[1], D[2], D[3], eps16, q);
+        float2 q;
+        const float2 a = make_float2(n[3], p[0]), b = make_float2(n[2], p[1]), c = make_float2(n[1], p[2]),
+                     d = make_float2(n[0], p[3]);
+        const float2 r = Z ? z_ratio<float2>(a, b, c, d, eps16, q) : js_ratio(a, b, c, d, eps16, q);
         return half_ratio_diff(r, q);
     }
 };
@@ -284,10 +285,15 @@ __device__ __forceinline__ void sweep_flux(const typename Lanes<V>::S* __restric
 #pragma unroll
         for (int k = 0; k < kNBackV; k++) slot[k * sstride] = back[k];
     }
-    // 3. the five differences of the stencil's U and F on all seven fields;
-    // the Alfven/entropy values wait in this thread's slots
+    // 4. Lax-Friedrichs speeds
+    V al[7];
+#pragma unroll
+    for (int s = 0; s < 7; s++) al[s] = lf_speed_v<V, CS>(cell, nc, s, e);
+    // 3-4. the five differences of the stencil's U and F on all seven fields,
+    // split: 2 D+- = l dF +- alpha l dU (eight values per field; those of the
+    // Alfven and entropy fields wait in this thread's slots)
     V* park = slot + kNBackV * sstride;
-    V dw[4][5], dg[4][5];
+    V dp[7][4], dn[7][4];
     V u0[7], f0[6];
 #pragma unroll
     for (int f = 0; f < 7; f++) u0[f] = ld<V>(cell + (SU + f) * nc);
@@ -295,7 +301,7 @@ __device__ __forceinline__ void sweep_flux(const typename Lanes<V>::S* __restric
     for (int f = 0; f < 6; f++) f0[f] = ld<V>(cell + (SF + 1 + f) * nc);
 #pragma unroll
     for (int m = 0; m < 5; m++) {
-        V x[7], o4[4], o3[3];
+        V x[7], w4[4], w3[3], g4[4], g3[3];
 #pragma unroll
         for (int f = 0; f < 7; f++) {
             const V u1 = ld<V>(cell + (SU + f) * nc + (m + 1) * CS);
@@ -303,11 +309,7 @@ __device__ __forceinline__ void sweep_flux(const typename Lanes<V>::S* __restric
             u0[f] = u1;
         }
         const V dm = x[1];                   // the mass flux is the normal momentum
-        project(e, x, o4, o3);
-#pragma unroll
-        for (int f = 0; f < 4; f++) dw[f][m] = o4[f];
-#pragma unroll
-        for (int f = 0; f < 3; f++) park[(f * 5 + m) * sstride] = o3[f];
+        project(e, x, w4, w3);
         x[0] = dm;
 #pragma unroll
         for (int f = 0; f < 6; f++) {
@@ -315,27 +317,35 @@ __device__ __forceinline__ void sweep_flux(const typename Lanes<V>::S* __restric
             x[f + 1] = vsub(f1, f0[f]);
             f0[f] = f1;
         }
-        project(e, x, o4, o3);
+        project(e, x, g4, g3);
 #pragma unroll
-        for (int f = 0; f < 4; f++) dg[f][m] = o4[f];
-#pragma unroll
-        for (int f = 0; f < 3; f++) park[((3 + f) * 5 + m) * sstride] = o3[f];
+        for (int s = 0; s < 7; s++) {
+            const V w = s & 1 ? w3[s >> 1] : w4[s >> 1], g = s & 1 ? g3[s >> 1] : g4[s >> 1];
+            V* mine = park + (s >> 1) * 8 * sstride;
+            if (m < 4) {
+                const V d = vfma(al[s], w, g);
+                if (s & 1) mine[m * sstride] = d;
+                else dp[s][m] = d;
+            }
+            if (m > 0) {
+                const V d = vfma(vneg(al[s]), w, g);
+                if (s & 1) mine[(3 + m) * sstride] = d;
+                else dn[s][m - 1] = d;
+            }
+        }
     }
-    // 4-5. Lax-Friedrichs speeds and weights, fast and slow fields, then
-    // Alfven and entropy
+    // 5. weights, fast and slow fields, then Alfven and entropy
     V corr[7];
 #pragma unroll
-    for (int f = 0; f < 4; f++) corr[2 * f] = weno_corr<V, Z>(dw[f], dg[f], lf_speed_v<V, CS>(cell, nc, 2 * f, e));
+    for (int s = 0; s < 7; s += 2) corr[s] = weno_corr<V, Z>(dp[s], dn[s]);
 #pragma unroll
-    for (int f = 0; f < 3; f++) {
-        const int s = 2 * f + 1;
-        V wa[5], ga[5];
+    for (int s = 1; s < 7; s += 2) {
 #pragma unroll
-        for (int m = 0; m < 5; m++) {
-            wa[m] = park[(f * 5 + m) * sstride];
-            ga[m] = park[((3 + f) * 5 + m) * sstride];
+        for (int m = 0; m < 4; m++) {
+            dp[s][m] = park[((s >> 1) * 8 + m) * sstride];
+            dn[s][m] = park[((s >> 1) * 8 + 4 + m) * sstride];
         }
-        corr[s] = weno_corr<V, Z>(wa, ga, lf_speed_v<V, CS>(cell, nc, s, e));
+        corr[s] = weno_corr<V, Z>(dp[s], dn[s]);
     }
     // 6. back-projection: sum_s r_s corr_s in primitive variables, then dU/dW,
     // and the central flux (7 (F_i + F_{i+1}) - (F_{i-1} + F_{i+2})) / 12
@@ -374,6 +384,24 @@ __device__ __forceinline__ void sweep_flux(const typename Lanes<V>::S* __restric
     }
 }
 
+// The flux through the lower face of cell c, rotated back, to the axis' arrays.
+template <class T, int AXIS>
+__device__ __forceinline__ void store_flux(const SweepArgs<T>& A, long long c, const T (&F)[7]) {
+    const long long N = A.ncells;
+    T* __restrict__ fo = A.flux;
+    T fx, fy, fz;
+    if (AXIS == 0) { fx = F[1]; fy = F[2]; fz = F[3]; }
+    else if (AXIS == 1) { fy = F[1]; fz = F[2]; fx = F[3]; }
+    else { fz = F[1]; fx = F[2]; fy = F[3]; }
+    fo[c] = F[0];
+    fo[N + c] = fx;
+    fo[2 * N + c] = fy;
+    fo[3 * N + c] = fz;
+    fo[4 * N + c] = F[6];
+    fo[5 * N + c] = F[4];
+    fo[6 * N + c] = F[5];
+}
+
 // ---- one tile ------------------------------------------------------------------------
 // Stages the TA + 5 cells of each of the TP pencils, then one thread per
 // interface.  Cell s of pencil tp lies at tp * NS + s (x sweep) or s * TP + tp.
@@ -401,7 +429,7 @@ __device__ __forceinline__ void tile_body(const SweepArgs<T>& A, const Tile& til
         const int raw_a = tile.y - 3 + s;
         rown[it] = raw_a >= tile.y && raw_a < tile.y + TA && raw_a < na;
         if (rok[it]) {
-            const int ca = A.links ? raw_a : wrap(raw_a, na);
+            const int ca = A.links ? raw_a : wrap_near(raw_a, na);
             int i, j, k;
             if (AXIS == 0) { i = ca; j = cp; k = tile.w; }
             else if (AXIS == 1) { i = cp; j = ca; k = tile.w; }
@@ -439,20 +467,7 @@ __device__ __forceinline__ void tile_body(const SweepArgs<T>& A, const Tile& til
     if (AXIS == 0) { i = ia; j = ip; k = tile.w; }
     else if (AXIS == 1) { i = ip; j = ia; k = tile.w; }
     else { i = ip; j = tile.w; k = ia; }
-    const long long N = A.ncells;
-    const long long c = chk(P.off + ((long long)k * P.ny + j) * P.nx + i, N, A.flag);
-    T* __restrict__ fo = A.flux;
-    T fx, fy, fz;
-    if (AXIS == 0) { fx = F[1]; fy = F[2]; fz = F[3]; }
-    else if (AXIS == 1) { fy = F[1]; fz = F[2]; fx = F[3]; }
-    else { fz = F[1]; fx = F[2]; fy = F[3]; }
-    fo[c] = F[0];
-    fo[N + c] = fx;
-    fo[2 * N + c] = fy;
-    fo[3 * N + c] = fz;
-    fo[4 * N + c] = F[6];
-    fo[5 * N + c] = F[4];
-    fo[6 * N + c] = F[5];
+    store_flux<T, AXIS>(A, chk(P.off + ((long long)k * P.ny + j) * P.nx + i, A.ncells, A.flag), F);
 }
 
 // Persistent sweep: a grid of (SMs x resident blocks) takes tiles of any

@@ -251,7 +251,7 @@ __device__ __forceinline__ void mlp_warp(const uint32_t* __restrict__ Ws, const 
 
 // Weight policy of the learned scheme.
 struct LearnedWeights {
-    static constexpr bool kDiff = WB_LEARNED_DELTA != 0;
+    static constexpr bool kSplit = false;
     const uint32_t* W;        // shared, [field][34][32]
     uint32_t* in;             // shared, this warp's 64 x 4 words
     float* om;                // shared, this warp's 64 x 2
@@ -477,7 +477,7 @@ __global__ void __launch_bounds__(kLearnedNT, WB_LEARNED_MINB) sweep_learned_ker
     // weight fragments read from global memory (L1-resident, 32 KB); each
     // thread's back-projection and parked slots after the staged cells
     const uint32_t* Wsm = mlp;
-    uint32_t* wbuf = reinterpret_cast<uint32_t*>(sm + (kNSlot * NC + kNThreadSlots * TA * TP));
+    uint32_t* wbuf = reinterpret_cast<uint32_t*>(sm + (kNSlot * NC + thread_slots(5) * TA * TP));
 #else
     uint32_t* Wsm = reinterpret_cast<uint32_t*>(sm + (kNSlot * NC + kNBack * TA * TP));
     uint32_t* wbuf = Wsm + kMlpSmemWords;                 // per warp 256 + 128 words
@@ -582,7 +582,7 @@ constexpr size_t learned_smem_bytes() {
     constexpr size_t TA = LShape<AXIS>::TA, TP = LShape<AXIS>::TP;
     constexpr size_t wbuf = sizeof(uint32_t) * (kLearnedNT / 32) * 384;     // per warp 256 + 128 words
 #if WB_LEARNED_DELTA
-    return sizeof(float) * (kNSlot * (TA + 5) * TP + kNThreadSlots * TA * TP) + wbuf;
+    return sizeof(float) * (kNSlot * (TA + 5) * TP + thread_slots(5) * TA * TP) + wbuf;
 #else
     return sizeof(float) * (kNSlot * (TA + 5) * TP + kNBack * TA * TP) + sizeof(uint32_t) * kMlpSmemWords + wbuf;
 #endif

@@ -157,7 +157,6 @@ __device__ __forceinline__ void gelu_row(const float (&v)[32], unsigned char* ti
 // Weight policy of the tensor-core learned scheme (one block, 128 threads,
 // every thread calling corr for the same field in the same order).
 struct LearnedWeightsTc {
-    static constexpr bool kDiff = false;     // works on the stencil values themselves
     const unsigned char* W;   // shared: the seven fields' weight images
     unsigned char* X;         // shared: A of layers 1 and 3 (two row tiles)
     unsigned char* Y;         // shared: A of layer 2 (two row tiles, K = 48)
