@@ -112,10 +112,11 @@ struct wb_grid {
     cudaEvent_t ev_branch[4] = {nullptr, nullptr, nullptr, nullptr};   // their ends, and the forks
     double kappa = 4.0, pjump = 0.5, smooth = 1.03;   // detector thresholds, smoothness gate
     int tile_policy[3] = {-2, -2, -2};    // build_tiles policy of each axis' table
-    int tile_split[3][3] = {};            // per axis: tiles of each shape of a table sorted
+    int tile_split[3][4] = {};            // per axis: tiles of each shape of a table sorted
                                           // by shape, or all 0 (wb::SweepArgs::split)
     wb::PatchDev* d_patches = nullptr;
     std::vector<wb::PatchDev> h_patches;
+    bool links = false;                   // the descriptor links patches
     int* d_links = nullptr;               // 27 per patch (wb::locate) or nullptr
     wb::Tile* d_tiles[3] = {nullptr, nullptr, nullptr};
     int ntiles[3] = {0, 0, 0};
@@ -143,13 +144,13 @@ static_assert(WB_NTILE_SHAPE == wb::kNTileShape, "tile shape count");
 
 // Tiles of each shape when the table is sorted by shape (then each shape
 // runs as its own fixed-shape launch), else all 0.
-void tile_split(const std::vector<wb::Tile>& t, int split[3]) {
-    split[0] = split[1] = split[2] = 0;
+void tile_split(const std::vector<wb::Tile>& t, int split[4]) {
+    split[0] = split[1] = split[2] = split[3] = 0;
     int prev = 0;
     for (const wb::Tile& x : t) {
         const int sh = (int)((unsigned)x.x >> 24);
-        if (sh < prev || sh >= wb::kNTileShape) {
-            split[0] = split[1] = split[2] = 0;
+        if (sh < prev || sh > wb::kFlatShape) {
+            split[0] = split[1] = split[2] = split[3] = 0;
             return;
         }
         split[sh]++;
@@ -158,8 +159,8 @@ void tile_split(const std::vector<wb::Tile>& t, int split[3]) {
 }
 
 template <class T>
-void set_split(wb::SweepArgs<T>& a, const int split[3]) {
-    for (int i = 0; i < 3; i++) a.split[i] = split[i];
+void set_split(wb::SweepArgs<T>& a, const int split[4]) {
+    for (int i = 0; i < 4; i++) a.split[i] = split[i];
 }
 
 // Forks branch b off the grid's stream / joins it again (inside a capture:
@@ -448,6 +449,8 @@ void release(wb_grid* g) {
 // (ragged tiles at the patch edges idle threads), ties to the lower shape
 // (FP64: to the longer tile);
 // policy -2 then orders the table by shape (a fixed-shape launch per shape).
+// A periodic patch one cell deep along the axis takes flat tiles under every
+// policy (the learned sweep counts its decisions there as everywhere).
 // The shape goes into the top byte of the tile's patch field.
 std::vector<wb::Tile> build_tiles(const wb_grid* g, int axis, int policy) {
     std::vector<wb::Tile> out;
@@ -456,6 +459,12 @@ std::vector<wb::Tile> build_tiles(const wb_grid* g, int axis, int policy) {
         const int na = axis == 0 ? P.nx : (axis == 1 ? P.ny : P.nz);
         const int npn = axis == 0 ? P.ny : P.nx;
         const int n3 = axis == 0 ? P.nz : (axis == 1 ? P.nz : P.ny);
+        if (na == 1 && !g->links && g->precision != WB_FP32_LEARNED) {
+            const long long np = (long long)P.nx * P.ny * P.nz;
+            for (long long c = 0; c < np; c += wb::kFlatCells)
+                out.push_back(wb::Tile{p | (wb::kFlatShape << 24), (int)c, 0, 0});
+            continue;
+        }
         int best = policy;
         if (policy < 0) {
             long long slots = -1;
@@ -496,7 +505,7 @@ std::vector<wb::Tile> build_tiles(const wb_grid* g, int axis, int policy) {
                     for (int x0 = 0; x0 < P.nx; x0 += tp) out.push_back(wb::Tile{px, z0, x0, y});
         }
     }
-    if (policy == -2)
+    if (policy != -1)
         std::stable_sort(out.begin(), out.end(), [](const wb::Tile& a, const wb::Tile& b) {
             return ((unsigned)a.x >> 24) < ((unsigned)b.x >> 24);
         });
@@ -603,7 +612,7 @@ int face_fluxes_impl(wb_grid* g, int axis, double* F_out) {
 }
 
 template <class T>
-int time_sweep(wb_grid* g, int axis, const wb::Tile* tiles, int ntiles, const int split[3], float* ms) {
+int time_sweep(wb_grid* g, int axis, const wb::Tile* tiles, int ntiles, const int split[4], float* ms) {
     wb::SweepArgs<T> a;
     a.src = static_cast<const T*>(g->un);
     a.flux = static_cast<T*>(g->flux) + (long long)axis * wb::kNFlux * g->N;
@@ -673,6 +682,7 @@ int wb_init_grid(const wb_grid_desc* d, const double* U0, const double* b0, void
     g->dx = d->dx; g->dy = d->dy; g->dz = d->dz; g->gamma = d->gamma;
     g->precision = d->precision; g->integrator = d->integrator; g->emf_mode = d->emf_mode;
     g->weights = d->weights;
+    g->links = d->links != nullptr;
     g->tsize = d->precision == WB_FP64 ? 8 : 4;
     long long off = 0;
     for (int p = 0; p < d->npatch; p++) {
@@ -1182,7 +1192,7 @@ int wb_autotune(wb_grid* g, double* ms_out) {
             float ms = 0.f;
             if (cudaMemcpy(d, t.data(), sizeof(wb::Tile) * t.size(), cudaMemcpyHostToDevice) != cudaSuccess)
                 rc = fail(WB_ECUDA, "autotune: tile upload failed");
-            int split[3];
+            int split[4];
             tile_split(t, split);
             if (rc == WB_OK)
                 rc = g->precision == WB_FP64 ? time_sweep<double>(g, axis, d, (int)t.size(), split, &ms)

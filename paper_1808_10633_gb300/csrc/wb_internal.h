@@ -150,8 +150,9 @@ struct SweepArgs {
     int zweights = 0;              // 1: WENO-Z weights instead of Jiang-Shu
     unsigned long long* lstats = nullptr;   // learned sweep: detector firings, decisions
     int* queue = nullptr;          // persistent sweep: tile counter of this launch (or fixed stride)
-    int split[3] = {0, 0, 0};      // tiles of shape 0, 1, 2 of a table sorted by shape
-                                   // (one fixed launch per shape, a tile per block);
+    int split[4] = {0, 0, 0, 0};   // tiles of shape 0, 1, 2 and flat ones of a table
+                                   // sorted by shape (one fixed launch per shape, a
+                                   // tile per block);
                                    // all 0: the persistent runtime-shape launch
     unsigned int* flag = nullptr;  // status word (bounds-checked builds)
 };
@@ -190,6 +191,9 @@ cudaError_t prepare_sweep_kernels();
 // Tile shape s (0 = default, kNTileShape alternatives) of the sweep along
 // `axis`: ta interfaces along the axis times tp pencils (ta * tp = 128).
 constexpr int kNTileShape = 3;
+// Shape code of flat tiles: 128 successive cells of a periodic patch one cell
+// deep along the axis (tile.y the first).
+constexpr int kFlatShape = 3, kFlatCells = 128;
 void sweep_shape(int axis, int s, int* ta, int* tp);
 // Tile of the learned-weight sweep along `axis` (one shape, 256 threads).
 void learned_shape(int axis, int* ta, int* tp);

@@ -670,6 +670,7 @@ __device__ __forceinline__ void interface_flux(const T* __restrict__ sm, int nc,
 #endif
 // interfaces per tile of the Jiang-Shu / WENO-Z sweeps
 constexpr int kSweepNT = 128;
+static_assert(kSweepNT == kFlatCells, "a flat tile is one cell per thread");
 template <int AXIS> struct Shape;
 template <> struct Shape<0> { static constexpr int TA = WB_SWEEP_TA_X, TP = 256 / WB_SWEEP_TA_X; };
 template <> struct Shape<1> { static constexpr int TA = WB_SWEEP_TA_YZ, TP = 256 / WB_SWEEP_TA_YZ; };

@@ -470,6 +470,42 @@ __device__ __forceinline__ void tile_body(const SweepArgs<T>& A, const Tile& til
     store_flux<T, AXIS>(A, chk(P.off + ((long long)k * P.ny + j) * P.nx + i, A.ncells, A.flag), F);
 }
 
+// ---- an axis of one cell ----------------------------------------------------------------
+// A periodic patch one cell deep along the axis (2-D and 1-D runs): all six
+// stencil cells of an interface are its one cell, every projected difference
+// is zero, and the flux is the central combination of four equal fluxes.  One
+// thread per cell; tile.y is the first of kSweepNT cells.  As ordinary tiles
+// these sweeps ran one warp per block at half its lanes through the whole
+// interface arithmetic (64^2 x 1, RK4, FP64, four steps: 2.24 -> 1.24 ms).
+template <class T, int AXIS>
+__device__ __forceinline__ void flat_body(const SweepArgs<T>& A, const Tile& tile, const PatchDev& P,
+                                          T* __restrict__ sm, int tid) {
+    const int local = tile.y + tid, nxy = P.nx * P.ny;
+    if (local >= nxy * P.nz) return;
+    const int k = local / nxy, rem = local - k * nxy, j = rem / P.nx, i = rem - j * P.nx;
+    RawCell<T> r;
+    long long c;
+    load_cell<T>(A, P, i, j, k, r, c);
+    derive_cell<T, AXIS>(A, r, c, sm, kSweepNT, tid, A.er != nullptr);
+    T F[7];
+#pragma unroll
+    for (int f = 0; f < 7; f++) {
+        const T f2 = sm[fslot(f) * kSweepNT + tid] + sm[fslot(f) * kSweepNT + tid];
+        if constexpr (sizeof(T) == 8) F[f] = fma(f2, 7.0 / 12.0, f2 * (-1.0 / 12.0));
+        else F[f] = (T(7) * f2 - f2) * T(1.0 / 12.0);
+    }
+    store_flux<T, AXIS>(A, c, F);
+}
+
+template <class T, int AXIS>
+__global__ void __launch_bounds__(kSweepNT) sweep_flat_kernel(const SweepArgs<T> A) {
+    extern __shared__ __align__(16) unsigned char smem_raw[];
+    Tile tile = A.tiles[blockIdx.x];
+    tile.x &= 0xffffff;
+    const PatchDev P = A.patches[tile.x];
+    flat_body<T, AXIS>(A, tile, P, reinterpret_cast<T*>(smem_raw), threadIdx.x);
+}
+
 // Persistent sweep: a grid of (SMs x resident blocks) takes tiles of any
 // shape from a work counter, so patches of uneven sizes share one launch;
 // each tile runs the body compiled for its shape (a block-uniform switch).
@@ -491,7 +527,8 @@ __global__ void __launch_bounds__(kSweepNT, kMinBlocks<T>) sweep_kernel(const Sw
         const PatchDev P = A.patches[tile.x];
         if (shape == 0) tile_body<T, AXIS, shape_ta(AXIS, 0), NCMAX, Z>(A, tile, P, sm, tid);
         else if (shape == 1) tile_body<T, AXIS, shape_ta(AXIS, 1), NCMAX, Z>(A, tile, P, sm, tid);
-        else tile_body<T, AXIS, shape_ta(AXIS, 2), NCMAX, Z>(A, tile, P, sm, tid);
+        else if (shape == 2) tile_body<T, AXIS, shape_ta(AXIS, 2), NCMAX, Z>(A, tile, P, sm, tid);
+        else flat_body<T, AXIS>(A, tile, P, sm, tid);
         __syncthreads();
         if (A.queue) {
             if (tid == 0) next_tile = gridDim.x + atomicAdd(A.queue, 1);
@@ -566,9 +603,18 @@ void launch_fixed_shape(int axis, const SweepArgs<T>& a, int ntiles, cudaStream_
     else sweep_kernel_fixed<T, 2, S, Z><<<ntiles, kSweepNT, smem_bytes_fixed<T, 2, S>(), s>>>(a);
 }
 
+template <class T>
+void launch_flat(int axis, const SweepArgs<T>& a, int ntiles, cudaStream_t s) {
+    constexpr size_t smem = sizeof(T) * kNSlot * kSweepNT;
+    static_assert(smem <= 48 * 1024, "within the default limit");
+    if (axis == 0) sweep_flat_kernel<T, 0><<<ntiles, kSweepNT, smem, s>>>(a);
+    else if (axis == 1) sweep_flat_kernel<T, 1><<<ntiles, kSweepNT, smem, s>>>(a);
+    else sweep_flat_kernel<T, 2><<<ntiles, kSweepNT, smem, s>>>(a);
+}
+
 template <class T, bool Z>
 cudaError_t launch_sweep_w(int axis, const SweepArgs<T>& a, int ntiles, cudaStream_t s) {
-    if (a.split[0] | a.split[1] | a.split[2]) {
+    if (a.split[0] | a.split[1] | a.split[2] | a.split[3]) {
         // a table sorted by shape: one launch of the fixed kernel per shape
         SweepArgs<T> b = a;
         if (a.split[0]) launch_fixed_shape<T, Z, 0>(axis, b, a.split[0], s);
@@ -576,6 +622,8 @@ cudaError_t launch_sweep_w(int axis, const SweepArgs<T>& a, int ntiles, cudaStre
         if (a.split[1]) launch_fixed_shape<T, Z, 1>(axis, b, a.split[1], s);
         b.tiles = a.tiles + a.split[0] + a.split[1];
         if (a.split[2]) launch_fixed_shape<T, Z, 2>(axis, b, a.split[2], s);
+        b.tiles = a.tiles + a.split[0] + a.split[1] + a.split[2];
+        if (a.split[3]) launch_flat<T>(axis, b, a.split[3], s);
         return cudaGetLastError();
     }
     const int grid = PersistGrid<T>::g[axis] > 0 ? PersistGrid<T>::g[axis] : 152;
