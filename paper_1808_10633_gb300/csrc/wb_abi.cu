@@ -252,13 +252,17 @@ int enqueue_stages(wb_grid* g, Prof* pf) {
         u.integrator = g->integrator;
         u.emf_mode = g->emf_mode;
         u.emf = static_cast<T*>(g->emf);
-        if ((rc = prof_begin(pf, g->stream)) != WB_OK) return rc;
-        WB_CK(wb::launch_emf<T>(u, g->nblocks, g->stream));
-        if ((rc = prof_end(pf, g->stream, WB_K_EMF)) != WB_OK) return rc;
+        const bool fused = wb::ct_update_fused<T>(u);
+        if (!fused) {
+            if ((rc = prof_begin(pf, g->stream)) != WB_OK) return rc;
+            WB_CK(wb::launch_emf<T>(u, g->nblocks, g->stream));
+            if ((rc = prof_end(pf, g->stream, WB_K_EMF)) != WB_OK) return rc;
+        }
         // the first update is the first to read dt
         if (st == 0 && !pf && (rc = join_branch(g, 2)) != WB_OK) return rc;
         if ((rc = prof_begin(pf, g->stream)) != WB_OK) return rc;
-        WB_CK(wb::launch_update<T>(u, g->nblocks, g->stream));
+        if (fused) WB_CK(wb::launch_ct_update<T>(u, g->nblocks, g->stream));
+        else WB_CK(wb::launch_update<T>(u, g->nblocks, g->stream));
         if ((rc = prof_end(pf, g->stream, WB_K_UPDATE)) != WB_OK) return rc;
     }
     return WB_OK;

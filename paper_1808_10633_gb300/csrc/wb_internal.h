@@ -202,6 +202,12 @@ template <class T>
 cudaError_t launch_emf(const UpdateArgs<T>& a, int nblocks, cudaStream_t s);
 template <class T>
 cudaError_t launch_update(const UpdateArgs<T>& a, int nblocks, cudaStream_t s);
+// EMFs and update of a stage in one launch (u.emf unused), and whether a grid
+// of this size takes it.
+template <class T>
+bool ct_update_fused(const UpdateArgs<T>& a);
+template <class T>
+cudaError_t launch_ct_update(const UpdateArgs<T>& a, int nblocks, cudaStream_t s);
 // Cells per thread of the vector forms of the EMF and update kernels (16 bytes).
 int update_vector_width(bool fp64);
 

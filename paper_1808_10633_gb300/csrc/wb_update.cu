@@ -3,7 +3,8 @@
 // constrained transport of the face-centred field on the staggered mesh
 // (Sec. 2.1), and the Runge-Kutta stage combination.
 //
-// Two kernels per stage.  The EMF kernel forms the three edge EMFs at each
+// Two kernels per stage, or for small grids one that does the work of both.
+// The EMF kernel forms the three edge EMFs at each
 // cell's own edge index (E_x at (i, j-1/2, k-1/2), E_y at (i-1/2, j, k-1/2),
 // E_z at (i-1/2, j-1/2, k)), each from the stored face fluxes:
 //   E_z(i-1/2, j-1/2) from -F_x(B_y) on the two x faces and F_y(B_x) on the
@@ -318,6 +319,87 @@ __global__ void __launch_bounds__(kCellBlock / 2, 6) update_kernel2(const Update
     }
 }
 
+// ---- EMFs and update in one launch ----------------------------------------------
+// One thread per cell forms the nine edge EMFs its three faces need itself (54
+// loads instead of 9, nearly all from L1 and L2), so a stage is one launch
+// shorter and the EMFs are neither written nor read; identical bits.  For small
+// grids, where a stage's time is the latency of its launches (ct_update_fused).
+template <class T, bool LINKED>
+__global__ void __launch_bounds__(kCellBlock / 2) ct_update_kernel(const UpdateArgs<T> A) {
+    const CellBlock cb = A.blocks[blockIdx.x >> 1];
+    const Geo<T, LINKED> G{A.patches[cb.x], A.patches, A.links, cb.x, A.ncells, A.flag};
+    const int local = cb.y + (blockIdx.x & 1) * (kCellBlock / 2) + threadIdx.x;
+    const int nx = G.P.nx, nxy = nx * G.P.ny;
+    if (local >= nxy * G.P.nz) return;
+    const int k = local / nxy;
+    const int rem = local - k * nxy;
+    const int j = rem / nx;
+    const int i = rem - j * nx;
+    const long long N = A.ncells;
+    const long long c = chk(G.P.off + local, N, A.flag);
+    // cells away from the patch's faces reach their neighbours without a lookup
+    const bool inner = i > 0 && i + 1 < nx && j > 0 && j + 1 < G.P.ny && k > 0 && k + 1 < G.P.nz;
+    auto at = [&](int di, int dj, int dk) -> long long {
+        if (inner) return chk(c + di + (long long)dj * nx + (long long)dk * nxy, N, A.flag);
+        return G.at(i + di, j + dj, k + dk);
+    };
+    const long long xp = at(1, 0, 0), yp = at(0, 1, 0), zp = at(0, 0, 1);
+    const long long xm = at(-1, 0, 0), ym = at(0, -1, 0), zm = at(0, 0, -1);
+    const T* __restrict__ Fx = A.flux;
+    const T* __restrict__ Fy = A.flux + 7 * N;
+    const T* __restrict__ Fz = A.flux + 14 * N;
+    T Lq[8];
+    const T idx = T(A.idx), idy = T(A.idy), idz = T(A.idz);
+#pragma unroll
+    for (int q = 0; q < 5; q++) {
+        const long long o = q * N;
+        Lq[q] = flux_rate(Fx[o + xp], Fx[o + c], Fy[o + yp], Fy[o + c], Fz[o + zp], Fz[o + c], idx, idy, idz);
+    }
+    const bool m0 = A.emf_mode == 0;
+    // E_x (E_y, E_z cyclically) at the cell's own edge, one up along e and one
+    // up along f: s P(-f) s P, -s Q(-e) -s Q with P on e faces and Q on f faces,
+    // and the cell values C of -v x B at (-e,-f), (-f), (-e), own (the order
+    // of emf_kernel, whose E_y takes its x faces first)
+    auto edge = [&](const T* __restrict__ P, const T* __restrict__ Q, const T* __restrict__ C, T s, long long c0,
+                    long long cp, long long cq, long long cpq) {
+        return edge_emf(s * P[cp], s * P[c0], -s * Q[cq], -s * Q[c0], m0 ? C[cpq] : T(0), m0 ? C[cp] : T(0),
+                        m0 ? C[cq] : T(0), m0 ? C[c0] : T(0), A.emf_mode);
+    };
+    const long long ymzm = at(0, -1, -1), ypzm = at(0, 1, -1), ymzp = at(0, -1, 1);
+    const long long xmzm = at(-1, 0, -1), xpzm = at(1, 0, -1), xmzp = at(-1, 0, 1);
+    const long long xmym = at(-1, -1, 0), xpym = at(1, -1, 0), xmyp = at(-1, 1, 0);
+    const T* __restrict__ Er = A.er;
+    const T mone = T(-1), one = T(1);
+    // E_x: -F_y(B_z) at (k-1), (k); F_z(B_y) at (j-1), (j)
+    const T ex = edge(Fy + 5 * N, Fz + 6 * N, Er, mone, c, zm, ym, ymzm);
+    const T ex_y = edge(Fy + 5 * N, Fz + 6 * N, Er, mone, yp, ypzm, c, zm);
+    const T ex_z = edge(Fy + 5 * N, Fz + 6 * N, Er, mone, zp, c, ymzp, ym);
+    // E_y: F_x(B_z) at (k-1), (k); -F_z(B_x) at (i-1), (i)
+    const T* __restrict__ Ey_ = m0 ? Er + N : Er;
+    const T ey = edge(Fx + 6 * N, Fz + 5 * N, Ey_, one, c, zm, xm, xmzm);
+    const T ey_x = edge(Fx + 6 * N, Fz + 5 * N, Ey_, one, xp, xpzm, c, zm);
+    const T ey_z = edge(Fx + 6 * N, Fz + 5 * N, Ey_, one, zp, c, xmzp, xm);
+    // E_z: -F_x(B_y) at (j-1), (j); F_y(B_x) at (i-1), (i)
+    const T* __restrict__ Ez_ = m0 ? Er + 2 * N : Er;
+    const T ez = edge(Fx + 5 * N, Fy + 6 * N, Ez_, mone, c, ym, xm, xmym);
+    const T ez_x = edge(Fx + 5 * N, Fy + 6 * N, Ez_, mone, xp, xpym, c, ym);
+    const T ez_y = edge(Fx + 5 * N, Fy + 6 * N, Ez_, mone, yp, c, xmyp, xm);
+    Lq[5] = face_rate(ez_y, ez, idy, ey_z, ey, idz);
+    Lq[6] = face_rate(ex_z, ex, idz, ez_x, ez, idx);
+    Lq[7] = face_rate(ey_x, ey, idx, ex_y, ex, idy);
+    const T dt = T(*A.dt);
+#pragma unroll
+    for (int q = 0; q < 8; q++) {
+        const long long o = q * N + c;
+        const T un = A.un[o];
+        const T uk = A.stage > 0 && A.integrator == 0 ? A.uk[o] : T(0);
+        T acc = A.integrator == 1 && A.stage > 0 ? A.acc[o] : T(0);
+        const T out = combine_value(A.integrator, A.stage, un, uk, acc, Lq[q], dt);
+        if (A.integrator == 1 && A.stage < 3) A.acc[o] = acc;
+        A.dst[o] = out;
+    }
+}
+
 // ---- one thread per vector of V cells along x (periodic patches) -------------
 template <class T> struct Vec;
 template <> struct Vec<float> { using type = float4; static constexpr int V = 4; };
@@ -559,10 +641,30 @@ cudaError_t launch_update(const UpdateArgs<T>& a, int nblocks, cudaStream_t s) {
     return cudaGetLastError();
 }
 
+// Up to here one launch beats two, beyond it the recomputed EMFs' loads cost
+// more than the launch (EMFs and update of one step, two launches against one:
+// FP32 32 x 1 x 1 44 / 26 us, 48^3 54 / 37, 64^3 55 / 55, 80^3 79 / 107; FP64,
+// whose EMF arithmetic the narrow pipe pays for, 64^2 87 / 44, 32^3 88 / 60,
+// 48^3 135 / 141).
+template <class T>
+bool ct_update_fused(const UpdateArgs<T>& a) { return a.ncells <= (sizeof(T) == 4 ? 180000 : 80000); }
+
+template <class T>
+cudaError_t launch_ct_update(const UpdateArgs<T>& a, int nblocks, cudaStream_t s) {
+    if (nblocks <= 0) return cudaSuccess;
+    if (a.links) ct_update_kernel<T, true><<<2 * nblocks, kCellBlock / 2, 0, s>>>(a);
+    else ct_update_kernel<T, false><<<2 * nblocks, kCellBlock / 2, 0, s>>>(a);
+    return cudaGetLastError();
+}
+
 int update_vector_width(bool fp64) { return fp64 ? Vec<double>::V : Vec<float>::V; }
 
 template cudaError_t launch_emf<float>(const UpdateArgs<float>&, int, cudaStream_t);
 template cudaError_t launch_emf<double>(const UpdateArgs<double>&, int, cudaStream_t);
+template bool ct_update_fused<float>(const UpdateArgs<float>&);
+template bool ct_update_fused<double>(const UpdateArgs<double>&);
+template cudaError_t launch_ct_update<float>(const UpdateArgs<float>&, int, cudaStream_t);
+template cudaError_t launch_ct_update<double>(const UpdateArgs<double>&, int, cudaStream_t);
 template cudaError_t launch_update<float>(const UpdateArgs<float>&, int, cudaStream_t);
 template cudaError_t launch_update<double>(const UpdateArgs<double>&, int, cudaStream_t);
 
