@@ -311,17 +311,35 @@ __device__ __forceinline__ void load_cell(const SweepArgs<T>& A, const PatchDev&
                  c + (long long)(kp - k) * P.nx * P.ny, r);
 }
 
-// (i, j, k) are coordinates of patch p of a linked grid and may lie outside
-// it (the stencil reaching into a neighbour).
-template <class T>
-__device__ __forceinline__ void load_cell_linked(const SweepArgs<T>& A, int p, const PatchDev& P,
-                                                 int i, int j, int k, RawCell<T>& r, long long& c) {
-    c = locate(A.patches, A.links, p, P, i, j, k);
-    load_cell_at(A, c, locate(A.patches, A.links, p, P, i + 1, j, k),
-                 locate(A.patches, A.links, p, P, i, j + 1, k),
-                 locate(A.patches, A.links, p, P, i, j, k + 1), r);
+// Cell (i, j, k) of patch p as a tile meets it: outside the patch along the
+// sweep axis where the stencil reaches past its end.  Most cells lie inside with
+// their three upper neighbours and need no wrap and no link.
+template <class T, int AXIS>
+__device__ __forceinline__ void load_cell_tile(const SweepArgs<T>& A, int p, const PatchDev& P, int i, int j, int k,
+                                               RawCell<T>& r, long long& c) {
+    long long cx, cy, cz;
+    const int nxy = P.nx * P.ny;
+    if ((unsigned)i < (unsigned)(P.nx - 1) && (unsigned)j < (unsigned)(P.ny - 1) && (unsigned)k < (unsigned)(P.nz - 1)) {
+        c = P.off + (k * P.ny + j) * P.nx + i;
+        cx = c + 1;
+        cy = c + P.nx;
+        cz = c + nxy;
+    } else if (A.links) {
+        c = locate(A.patches, A.links, p, P, i, j, k);
+        cx = locate(A.patches, A.links, p, P, i + 1, j, k);
+        cy = locate(A.patches, A.links, p, P, i, j + 1, k);
+        cz = locate(A.patches, A.links, p, P, i, j, k + 1);
+    } else {
+        if (AXIS == 0) i = wrap_near(i, P.nx);
+        else if (AXIS == 1) j = wrap_near(j, P.ny);
+        else k = wrap_near(k, P.nz);
+        c = P.off + (k * P.ny + j) * P.nx + i;
+        cx = c + (i + 1 == P.nx ? 1 - P.nx : 1);
+        cy = c + (j + 1 == P.ny ? P.nx - nxy : P.nx);
+        cz = c + (k + 1 == P.nz ? (long long)nxy * (1 - P.nz) : nxy);
+    }
+    load_cell_at(A, c, cx, cy, cz, r);
 }
-
 
 template <class T, int AXIS>
 __device__ __forceinline__ void derive_cell(const SweepArgs<T>& A, const RawCell<T>& r, long long c,
