@@ -145,7 +145,7 @@ grad_kernel(const float* __restrict__ rec, const long long* __restrict__ perm, c
     for (long long c = (long long)g * kChunk; c < n; c += (long long)kGradBlocks * kChunk) {
         // forward and backward, four records per warp, lane = hidden unit
         constexpr int Q = kChunk / (kGradThreads / 32);
-        float h2[Q], d1[Q], d2[Q], z[Q][NOUT];
+        float d1[Q], d2[Q];
         const float* r[Q];
         const int first = warp * Q;
 #pragma unroll
@@ -183,33 +183,36 @@ grad_kernel(const float* __restrict__ rec, const long long* __restrict__ perm, c
             }
 #pragma unroll
             for (int q = 0; q < Q; q++) {
-                h2[q] = gelu(a[q], d2[q]);
-                row[first + q][S_H2 + lane] = h2[q];
+                row[first + q][S_H2 + lane] = gelu(a[q], d2[q]);
             }
         }
+        __syncwarp();
+        // output layer: lane 3 q + o sums output o of record q over the hidden
+        // units in their order
+        float zo = 0.f;
+        if (lane < Q * NOUT) {
+            const int q = lane / NOUT, o = lane - q * NOUT;
+            zo = B3[o];
 #pragma unroll
-        for (int q = 0; q < Q; q++)
-#pragma unroll
-            for (int o = 0; o < NOUT; o++) {
-                float a = W3[o][lane] * h2[q];
-#pragma unroll
-                for (int m = 16; m > 0; m >>= 1) a += __shfl_xor_sync(0xffffffffu, a, m);
-                z[q][o] = a + B3[o];
+            for (int k = 0; k < NH; k += 4) {
+                const float4 h = *reinterpret_cast<const float4*>(&row[first + q][S_H2 + k]);
+                const float4 w = *reinterpret_cast<const float4*>(&W3[o][k]);
+                zo += w.x * h.x;
+                zo += w.y * h.y;
+                zo += w.z * h.z;
+                zo += w.w * h.w;
             }
+        }
+        float zz[NOUT];
+#pragma unroll
+        for (int o = 0; o < NOUT; o++) zz[o] = __shfl_sync(0xffffffffu, zo, (lane < Q ? NOUT * lane : 0) + o);
         // softmax, loss and its gradient: lane q of the first four takes record q
         float dz[NOUT] = {0.f, 0.f, 0.f};
         if (lane < Q) {
-            float zz[NOUT];
             const float* rr = r[0];
 #pragma unroll
-            for (int o = 0; o < NOUT; o++) zz[o] = z[0][o];
-#pragma unroll
             for (int q = 1; q < Q; q++)
-                if (lane == q) {
-                    rr = r[q];
-#pragma unroll
-                    for (int o = 0; o < NOUT; o++) zz[o] = z[q][o];
-                }
+                if (lane == q) rr = r[q];
             const float zm = fmaxf(zz[0], fmaxf(zz[1], zz[2]));
             float e[NOUT], es = 0.f;
 #pragma unroll
