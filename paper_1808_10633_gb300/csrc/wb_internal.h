@@ -74,8 +74,8 @@ __device__ __forceinline__ long long chk(long long i, long long n, unsigned int*
     return i;
 }
 
-// Sweep tile: x = patch, y = start along the sweep axis, z = start along the
-// pencil axis, w = fixed third coordinate.
+// Sweep tile: x = patch, y = start along the sweep axis, z, w = first pencil's
+// place along the pencil axis and along the third (see tile_pencil).
 using Tile = int4;
 
 // Cell block for the per-cell kernels: x = patch, y = first local cell.

@@ -311,6 +311,31 @@ __device__ __forceinline__ void load_cell(const SweepArgs<T>& A, const PatchDev&
                  c + (long long)(kp - k) * P.nx * P.ny, r);
 }
 
+// Pencil tp of a tile: the pencils of a patch are numbered along the pencil
+// axis and then along the third, and a tile takes consecutive ones from (tile.z,
+// tile.w) on, past the end of a row into the next.  cp: place along the pencil
+// axis (of np), w: along the third.
+__device__ __forceinline__ void tile_pencil(const Tile& tile, int tp, int np, int& cp, int& w) {
+    cp = tile.z + tp;
+    w = tile.w;
+    if (cp >= np) {
+        cp -= np;
+        w++;
+        if (cp >= np) {                // rows shorter than the tile is wide
+            const int r = cp / np;
+            cp -= r * np;
+            w += r;
+        }
+    }
+}
+
+// Cell of the patch at place ia along the sweep axis of pencil (ip, w).
+template <int AXIS>
+__device__ __forceinline__ int tile_cell(const PatchDev& P, int ia, int ip, int w) {
+    const int i = AXIS == 0 ? ia : ip, j = AXIS == 0 ? ip : (AXIS == 1 ? ia : w), k = AXIS == 2 ? ia : w;
+    return (k * P.ny + j) * P.nx + i;
+}
+
 // Cell (i, j, k) of patch p as a tile meets it: outside the patch along the
 // sweep axis where the stencil reaches past its end.  Most cells lie inside with
 // their three upper neighbours and need no wrap and no link.

@@ -411,7 +411,7 @@ __device__ __forceinline__ void tile_body(const SweepArgs<T>& A, const Tile& til
     constexpr int NT = kSweepNT, TP = kSweepNT / TA, NS = TA + 5, NC = NS * TP;
     constexpr int CS = AXIS == 0 ? 1 : TP;         // distance of a pencil's neighbouring cells
     const int na = AXIS == 0 ? P.nx : (AXIS == 1 ? P.ny : P.nz);
-    const int np = AXIS == 0 ? P.ny : P.nx;
+    const int np = AXIS == 0 ? P.ny : P.nx, n3 = AXIS == 2 ? P.ny : P.nz;
 
     // staging: cells tile.y-3 .. tile.y+TA+1 along the axis, TP pencils
     constexpr int NIT = (NC + NT - 1) / NT;
@@ -424,15 +424,16 @@ __device__ __forceinline__ void tile_body(const SweepArgs<T>& A, const Tile& til
         int s, tp;
         if (AXIS == 0) { tp = e / NS; s = e - tp * NS; }
         else { s = e / TP; tp = e - s * TP; }
-        const int cp = tile.z + tp;
-        rok[it] = e < NC && cp < np;
+        int cp, w;
+        tile_pencil(tile, tp, np, cp, w);
+        rok[it] = e < NC && w < n3;
         const int raw_a = tile.y - 3 + s;
         rown[it] = raw_a >= tile.y && raw_a < tile.y + TA && raw_a < na;
         if (rok[it]) {
             int i, j, k;
-            if (AXIS == 0) { i = raw_a; j = cp; k = tile.w; }
-            else if (AXIS == 1) { i = cp; j = raw_a; k = tile.w; }
-            else { i = cp; j = tile.w; k = raw_a; }
+            if (AXIS == 0) { i = raw_a; j = cp; k = w; }
+            else if (AXIS == 1) { i = cp; j = raw_a; k = w; }
+            else { i = cp; j = w; k = raw_a; }
             load_cell_tile<T, AXIS>(A, tile.x, P, i, j, k, raw[it], rc[it]);
         }
     }
@@ -445,8 +446,11 @@ __device__ __forceinline__ void tile_body(const SweepArgs<T>& A, const Tile& til
     int ta, tp;
     if (AXIS == 0) { ta = tid & (TA - 1); tp = tid / TA; }
     else { tp = tid & (TP - 1); ta = tid / TP; }
-    const int ia = tile.y + ta, ip = tile.z + tp;
-    if (ia >= na || ip >= np) return;
+    const int ia = tile.y + ta;
+    int ip, w3;
+    tile_pencil(tile, tp, np, ip, w3);
+    if (ia >= na || w3 >= n3) return;
+    const int mine = tile_cell<AXIS>(P, ia, ip, w3);
     const int i0 = (int)chk(AXIS == 0 ? tp * NS + ta : ta * TP + tp, NC - 5 * CS, A.flag);
     T F[7];
     T* slot = sm + kNSlot * NCMAX + tid;
@@ -460,12 +464,7 @@ __device__ __forceinline__ void tile_body(const SweepArgs<T>& A, const Tile& til
         interface_flux<T, JsWeights<Z>, true>(sm, NC, id, T(A.gamma), slot, NT, js, F);
     }
 
-    // rotate back and store at the lower face of cell ia
-    int i, j, k;
-    if (AXIS == 0) { i = ia; j = ip; k = tile.w; }
-    else if (AXIS == 1) { i = ip; j = ia; k = tile.w; }
-    else { i = ip; j = tile.w; k = ia; }
-    store_flux<T, AXIS>(A, chk(P.off + ((long long)k * P.ny + j) * P.nx + i, A.ncells, A.flag), F);
+    store_flux<T, AXIS>(A, chk(P.off + mine, A.ncells, A.flag), F);
 }
 
 // ---- an axis of one cell ----------------------------------------------------------------

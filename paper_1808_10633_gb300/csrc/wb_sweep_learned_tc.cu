@@ -398,7 +398,7 @@ __global__ void __launch_bounds__(kTcNT, 2) sweep_learned_tc_kernel(const SweepA
     const Tile tile = A.tiles[blockIdx.x];
     const PatchDev P = A.patches[tile.x & 0xffffff];
     const int na = AXIS == 0 ? P.nx : (AXIS == 1 ? P.ny : P.nz);
-    const int np = AXIS == 0 ? P.ny : P.nx;
+    const int np = AXIS == 0 ? P.ny : P.nx, n3 = AXIS == 2 ? P.ny : P.nz;
     constexpr int NIT = (NC + kTcNT - 1) / kTcNT;
     RawCell<T> raw[NIT];
     long long rc[NIT];
@@ -410,16 +410,17 @@ __global__ void __launch_bounds__(kTcNT, 2) sweep_learned_tc_kernel(const SweepA
         int s, tp;
         if (AXIS == 0) { tp = e / NS; s = e - tp * NS; }
         else { s = e / TP; tp = e - s * TP; }
-        const int cp = tile.z + tp;
-        rok[it] = e < NC && cp < np;
+        int cp, w;
+        tile_pencil(tile, tp, np, cp, w);
+        rok[it] = e < NC && w < n3;
         const int raw_a = tile.y - 3 + s;
         rown[it] = raw_a >= tile.y && raw_a < tile.y + TA && raw_a < na;
         ridx[it] = AXIS == 0 ? tp * NS + s : s * TP + tp;
         if (rok[it]) {
             int i, j, k;
-            if (AXIS == 0) { i = raw_a; j = cp; k = tile.w; }
-            else if (AXIS == 1) { i = cp; j = raw_a; k = tile.w; }
-            else { i = cp; j = tile.w; k = raw_a; }
+            if (AXIS == 0) { i = raw_a; j = cp; k = w; }
+            else if (AXIS == 1) { i = cp; j = raw_a; k = w; }
+            else { i = cp; j = w; k = raw_a; }
             load_cell_tile<T, AXIS>(A, tile.x & 0xffffff, P, i, j, k, raw[it], rc[it]);
         }
     }
@@ -434,9 +435,12 @@ __global__ void __launch_bounds__(kTcNT, 2) sweep_learned_tc_kernel(const SweepA
     int ta, tp0;
     if (AXIS == 0) { ta = tid & (TA - 1); tp0 = tid >> LG_TA; }
     else { tp0 = tid & (TP - 1); ta = tid >> (7 - LG_TA); }
-    const int ia = tile.y + ta, ip = tile.z + tp0;
-    const bool valid = ia < na && ip < np;
-    const int tp = ip < np ? tp0 : 0;                      // stand-in stencil for idle threads
+    const int ia = tile.y + ta;
+    int ip, w3;
+    tile_pencil(tile, tp0, np, ip, w3);
+    const bool valid = ia < na && w3 < n3;
+    const int tp = w3 < n3 ? tp0 : 0;                      // stand-in stencil for idle lanes
+    const int mine = tile_cell<AXIS>(P, ia, ip, w3);
     int id[6];
 #pragma unroll
     for (int m = 0; m < 6; m++) id[m] = (int)chk(AXIS == 0 ? tp * NS + ta + m : (ta + m) * TP + tp, NC, A.flag);
@@ -460,12 +464,8 @@ __global__ void __launch_bounds__(kTcNT, 2) sweep_learned_tc_kernel(const SweepA
         }
     }
     if (valid) {
-        int i, j, k;
-        if (AXIS == 0) { i = ia; j = ip; k = tile.w; }
-        else if (AXIS == 1) { i = ip; j = ia; k = tile.w; }
-        else { i = ip; j = tile.w; k = ia; }
         const long long N = A.ncells;
-        const long long c = chk(P.off + ((long long)k * P.ny + j) * P.nx + i, N, A.flag);
+        const long long c = chk(P.off + mine, N, A.flag);
         T* __restrict__ fo = A.flux;
         T fx, fy, fz;
         if (AXIS == 0) { fx = F[1]; fy = F[2]; fz = F[3]; }
