@@ -44,7 +44,8 @@ constexpr int NE = NP + 1;                   // entries per field: the parameter
 constexpr int kChunk = 32;                   // records per pass of a block
 constexpr int kGradThreads = 256;
 // Blocks per field: two resident blocks per SM over seven fields, which cuts
-// a 4 096-record batch into three chunks per block.
+// a 4 096-record batch into three chunks per block (three and four blocks per SM
+// with 64 to 128 of them per field: 2 to 8 % slower per step).
 constexpr int kGradBlocks = 43;
 
 // GELU in its sigmoid form, gelu(t) = t sigma(1.702 t) = t/2 (1 + tanh(0.851 t)),
@@ -74,18 +75,24 @@ __device__ __forceinline__ long long pick(const long long* off, const long long*
     return off[f] + (long long)(h % (unsigned long long)cnt[f]);
 }
 
-// acc (an unevaluated pair hi + lo) += a b: the product and the sum are both
-// split into their rounded value and its exact error (Dekker's and Knuth's
-// error-free transformations), the errors collecting in lo.  The sum keeps
-// 48 bits for 10 FP32 operations; an FP64 accumulator would cost a fused
+// Two entries' sums at once, in the lanes of the packed FP32 instructions: each
+// an unevaluated pair hi + lo, += a b (nb = -b).  The product and the sum are
+// both split into their rounded value and its exact error (Dekker's and Knuth's
+// error-free transformations), the errors collecting in lo.  The sum keeps 48
+// bits for 10 FP32 operations; an FP64 accumulator would cost a fused
 // multiply-add and two conversions on a pipe 64 times narrower.
-__device__ __forceinline__ void add_prod(float2& acc, float a, float b) {
-    const float p = __fmul_rn(a, b), e = __fmaf_rn(a, b, -p);
-    const float t = __fadd_rn(acc.x, p), z = __fsub_rn(t, acc.x);
-    const float err = __fadd_rn(__fsub_rn(acc.x, __fsub_rn(t, z)), __fsub_rn(p, z));
-    acc.x = t;
-    acc.y = __fadd_rn(acc.y, __fadd_rn(err, e));
-}
+struct Sum2 {
+    float2 hi = {0.f, 0.f}, lo = {0.f, 0.f};
+    __device__ __forceinline__ void add(float2 a, float2 b, float2 nb) {
+        const float2 m1 = make_float2(-1.f, -1.f);
+        const float2 n = __fmul2_rn(a, nb), e = __ffma2_rn(a, b, n);              // -p, a b - p
+        const float2 t = __ffma2_rn(n, m1, hi), z = __ffma2_rn(hi, m1, t);        // hi + p
+        const float2 back = __ffma2_rn(__ffma2_rn(z, m1, t), m1, hi);             // hi - (t - z)
+        const float2 err = __ffma2_rn(__fadd2_rn(n, z), m1, back);                // + (p - z)
+        hi = t;
+        lo = __fadd2_rn(lo, __fadd2_rn(err, e));
+    }
+};
 
 // The two factors of gradient entry j in a record's row.
 __device__ __forceinline__ void entry_factors(int j, int& ga, int& gb) {
@@ -107,7 +114,8 @@ __device__ __forceinline__ void entry_factors(int j, int& ga, int& gb) {
 // dW2 per thread and the 356 other entries one or two per thread.  Bound by
 // the FP32 pipe: 10 of the 13 operations per entry and record are the exact
 // sums.  60 steps of 4 096 records per field and one full-batch gradient, host
-// side included: 83.5 -> 5.5 ms against a serial loop over the records per
+// side included: 83.5 -> 4.2 ms (33 us per step here, 7 in apply_kernel) against
+// a serial loop over the records per
 // entry with FP64 accumulators (and a loss copied to the host every step).
 __global__ void __launch_bounds__(kGradThreads, 2)
 grad_kernel(const float* __restrict__ rec, const long long* __restrict__ perm, const long long* __restrict__ off,
@@ -134,27 +142,30 @@ grad_kernel(const float* __restrict__ rec, const long long* __restrict__ perm, c
     // dW2, and entries e0, e1 of the rest (counted with dW2 left out)
     const int ti = tid >> 4, tk = tid & 15;
     constexpr int kRest = NE - NH * NH;
+    static_assert(kChunk / (kGradThreads / 32) == 4, "four records per warp");
     static_assert(kRest > kGradThreads && kRest <= 2 * kGradThreads, "two further entries per thread at most");
     const int e0 = tid < O_W2 ? tid : tid + NH * NH, e1 = tid + kGradThreads + NH * NH;
     const bool two = tid + kGradThreads < kRest;
     int ga0, gb0, ga1, gb1;
     entry_factors(e0, ga0, gb0);
     entry_factors(two ? e1 : e0, ga1, gb1);
-    float2 t00 = {0.f, 0.f}, t01 = t00, t10 = t00, t11 = t00, r0 = t00, r1 = t00;
+    Sum2 top, bot, rest;           // the tile's two rows, and e0 with e1
     __syncthreads();
     for (long long c = (long long)g * kChunk; c < n; c += (long long)kGradBlocks * kChunk) {
         // forward and backward, four records per warp, lane = hidden unit
         constexpr int Q = kChunk / (kGradThreads / 32);
         float d1[Q], d2[Q];
-        const float* r[Q];
         const int first = warp * Q;
-#pragma unroll
-        for (int q = 0; q < Q; q++) {
-            const long long slot = c + first + q;
-            // slots past the batch repeat its last record; their rows are not summed
-            const long long s = slot < n ? slot : n - 1;
-            r[q] = rec + perm[pick(off, cnt, f, s, full, seed, step)] * REC;
-            if (lane < NIN) row[first + q][S_X + lane] = r[q][1 + lane];
+        // lane q of the first four draws record q; slots past the batch repeat
+        // its last record, and their rows are not summed
+        const long long slot = c + first + lane;
+        const float* rr = rec;
+        if (lane < Q) rr += perm[pick(off, cnt, f, slot < n ? slot : n - 1, full, seed, step)] * REC;
+        {
+            // lane 8 q + k reads x_k of record q
+            const float* r = reinterpret_cast<const float*>(
+                __shfl_sync(0xffffffffu, (unsigned long long)rr, lane >> 3));
+            if ((lane & 7) < NIN) row[first + (lane >> 3)][S_X + (lane & 7)] = r[1 + (lane & 7)];
         }
         __syncwarp();
 #pragma unroll
@@ -209,10 +220,6 @@ grad_kernel(const float* __restrict__ rec, const long long* __restrict__ perm, c
         // softmax, loss and its gradient: lane q of the first four takes record q
         float dz[NOUT] = {0.f, 0.f, 0.f};
         if (lane < Q) {
-            const float* rr = r[0];
-#pragma unroll
-            for (int q = 1; q < Q; q++)
-                if (lane == q) rr = r[q];
             const float zm = fmaxf(zz[0], fmaxf(zz[1], zz[2]));
             float e[NOUT], es = 0.f;
 #pragma unroll
@@ -275,23 +282,22 @@ grad_kernel(const float* __restrict__ rec, const long long* __restrict__ perm, c
             const float* w = row[q];
             const float2 da = *reinterpret_cast<const float2*>(w + S_DA2 + 2 * ti);
             const float2 h = *reinterpret_cast<const float2*>(w + S_H1 + 2 * tk);
-            add_prod(t00, da.x, h.x);
-            add_prod(t01, da.x, h.y);
-            add_prod(t10, da.y, h.x);
-            add_prod(t11, da.y, h.y);
-            add_prod(r0, w[ga0], w[gb0]);
-            if (two) add_prod(r1, w[ga1], w[gb1]);
+            const float2 nh = make_float2(-h.x, -h.y);
+            top.add(make_float2(da.x, da.x), h, nh);
+            bot.add(make_float2(da.y, da.y), h, nh);
+            const float2 f = make_float2(w[gb0], w[gb1]);
+            rest.add(make_float2(w[ga0], w[ga1]), f, make_float2(-f.x, -f.y));
         }
         __syncthreads();
     }
     float2* o = part + (long long)blockIdx.x * NE;
     const int j = O_W2 + 2 * ti * NH + 2 * tk;
-    o[j] = t00;
-    o[j + 1] = t01;
-    o[j + NH] = t10;
-    o[j + NH + 1] = t11;
-    o[e0] = r0;
-    if (two) o[e1] = r1;
+    o[j] = make_float2(top.hi.x, top.lo.x);
+    o[j + 1] = make_float2(top.hi.y, top.lo.y);
+    o[j + NH] = make_float2(bot.hi.x, bot.lo.x);
+    o[j + NH + 1] = make_float2(bot.hi.y, bot.lo.y);
+    o[e0] = make_float2(rest.hi.x, rest.lo.x);
+    if (two) o[e1] = make_float2(rest.hi.y, rest.lo.y);
 }
 
 // Gradient entry j of field f: the blocks' sums added in FP64 in the order of
@@ -306,15 +312,18 @@ apply_kernel(const float2* __restrict__ part, const long long* __restrict__ cnt,
     if (f >= NF) return;
     const long long n = cnt[f] == 0 ? 0 : (full ? cnt[f] : (long long)batch);
     const float2* s = part + (long long)f * kGradBlocks * NE + j;
-    double hi = 0.0, lo = 0.0;
-#pragma unroll 8
+    // the same pair sums as in the blocks (FP64 additions would run on the
+    // narrow pipe: 13 us instead of 7)
+    float hi = 0.f, lo = 0.f;
+#pragma unroll
     for (int b = 0; b < kGradBlocks; b++) {
         const float2 a = s[(long long)b * NE];
-        hi += double(a.x);
-        lo += double(a.y);
+        const float t = __fadd_rn(hi, a.x), z = __fsub_rn(t, hi);
+        lo = __fadd_rn(lo, __fadd_rn(a.y, __fadd_rn(__fsub_rn(hi, __fsub_rn(t, z)), __fsub_rn(a.x, z))));
+        hi = t;
     }
     // an infinite sum leaves NaN in the errors: it stands by itself
-    const double sum = isfinite(hi) ? hi + lo : hi;
+    const double sum = isfinite(hi) ? double(hi) + double(lo) : double(hi);
     const float g = float(n > 0 ? sum / double(n) : 0.0);
     if (j == NP) {
         loss[f] = g;
@@ -330,21 +339,21 @@ apply_kernel(const float2* __restrict__ part, const long long* __restrict__ cnt,
     params[i] -= lr * (mi / c1) / (sqrtf(vi / c2) + eps);
 }
 
+// Device buffers of one call, cut from one allocation.
 struct Dev {
+    char* all = nullptr;
     float* rec = nullptr;
     long long* perm = nullptr;     // the records to train on, by field, in their order
-    long long* off = nullptr;
+    long long* off = nullptr;      // 7 offsets, then 7 counts
     long long* cnt = nullptr;
     float* params = nullptr;
     float* grad = nullptr;
-    float* m = nullptr;
+    float* m = nullptr;            // Adam's moments, m then v
     float* v = nullptr;
     float2* part = nullptr;        // the blocks' sums
     float* loss = nullptr;         // 7 per step
     ~Dev() {
-        for (void* p : {(void*)rec, (void*)perm, (void*)off, (void*)cnt, (void*)params, (void*)grad, (void*)m,
-                        (void*)v, (void*)part, (void*)loss})
-            if (p) cudaFree(p);
+        if (all) cudaFree(all);
     }
 };
 
@@ -369,24 +378,42 @@ int setup(Dev& D, const float* records, long long n, const float* params, long l
         if (records[r * REC + 11] == 0.f) perm[at[(int)records[r * REC]]++] = r;
     if (full && *std::max_element(cnt.begin(), cnt.end()) > (1LL << 24))
         return wb::set_last_error(WB_EINVAL, "mlp: too many records per field");
-    auto ck = [](cudaError_t e) { return e == cudaSuccess; };
-    if (!ck(cudaMalloc(&D.rec, sizeof(float) * n * REC)) ||
-        !ck(cudaMalloc(&D.perm, sizeof(long long) * perm.size())) ||
-        !ck(cudaMalloc(&D.off, sizeof(long long) * NF)) ||
-        !ck(cudaMalloc(&D.cnt, sizeof(long long) * NF)) ||
-        !ck(cudaMalloc(&D.params, sizeof(float) * NF * NP)) ||
-        !ck(cudaMalloc(&D.grad, sizeof(float) * NF * NP)) ||
-        !ck(cudaMalloc(&D.m, sizeof(float) * NF * NP)) || !ck(cudaMalloc(&D.v, sizeof(float) * NF * NP)) ||
-        !ck(cudaMalloc(&D.part, sizeof(float2) * NE * NF * kGradBlocks)) ||
-        !ck(cudaMalloc(&D.loss, sizeof(float) * NF * std::max<long long>(steps, 1))))
+    size_t used = 0;
+    auto place = [&](size_t bytes) {
+        const size_t at = used;
+        used += (bytes + 255) & ~size_t(255);
+        return at;
+    };
+    const size_t np = sizeof(float) * NF * NP;
+    const size_t rec = place(sizeof(float) * n * REC), prm = place(sizeof(long long) * perm.size()),
+                 tab = place(sizeof(long long) * 2 * NF), par = place(np), grd = place(np), mom = place(2 * np),
+                 prt = place(sizeof(float2) * NE * NF * kGradBlocks),
+                 los = place(sizeof(float) * NF * std::max<long long>(steps, 1));
+    if (cudaMalloc(&D.all, used) != cudaSuccess) {
+        cudaGetLastError();
         return wb::set_last_error(WB_ENOMEM, "mlp: device allocation failed");
-    if (!ck(cudaMemcpy(D.rec, records, sizeof(float) * n * REC, cudaMemcpyHostToDevice)) ||
-        !ck(cudaMemcpy(D.perm, perm.data(), sizeof(long long) * perm.size(), cudaMemcpyHostToDevice)))
+    }
+    D.rec = reinterpret_cast<float*>(D.all + rec);
+    D.perm = reinterpret_cast<long long*>(D.all + prm);
+    D.off = reinterpret_cast<long long*>(D.all + tab);
+    D.cnt = D.off + NF;
+    D.params = reinterpret_cast<float*>(D.all + par);
+    D.grad = reinterpret_cast<float*>(D.all + grd);
+    D.m = reinterpret_cast<float*>(D.all + mom);
+    D.v = D.m + NF * NP;
+    D.part = reinterpret_cast<float2*>(D.all + prt);
+    D.loss = reinterpret_cast<float*>(D.all + los);
+    long long table[2 * NF];
+    for (int f = 0; f < NF; f++) {
+        table[f] = off[f];
+        table[NF + f] = cnt[f];
+    }
+    if (cudaMemcpy(D.rec, records, sizeof(float) * n * REC, cudaMemcpyHostToDevice) != cudaSuccess ||
+        cudaMemcpy(D.perm, perm.data(), sizeof(long long) * perm.size(), cudaMemcpyHostToDevice) != cudaSuccess)
         return wb::set_last_error(WB_ECUDA, "mlp: record upload failed");
-    if (!ck(cudaMemcpy(D.off, off.data(), sizeof(long long) * NF, cudaMemcpyHostToDevice)) ||
-        !ck(cudaMemcpy(D.cnt, cnt.data(), sizeof(long long) * NF, cudaMemcpyHostToDevice)) ||
-        !ck(cudaMemcpy(D.params, params, sizeof(float) * NF * NP, cudaMemcpyHostToDevice)) ||
-        !ck(cudaMemset(D.m, 0, sizeof(float) * NF * NP)) || !ck(cudaMemset(D.v, 0, sizeof(float) * NF * NP)))
+    if (cudaMemcpy(D.off, table, sizeof(table), cudaMemcpyHostToDevice) != cudaSuccess ||
+        cudaMemcpy(D.params, params, np, cudaMemcpyHostToDevice) != cudaSuccess ||
+        cudaMemset(D.m, 0, 2 * np) != cudaSuccess)
         return wb::set_last_error(WB_ECUDA, "mlp: upload failed");
     return WB_OK;
 }
