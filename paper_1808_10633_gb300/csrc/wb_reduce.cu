@@ -209,17 +209,27 @@ __device__ __forceinline__ double face_div(double xp, double x, double yp, doubl
                                            double idy, double idz) {
     return (xp - x) * idx + (yp - y) * idy + (zp - z) * idz;
 }
-// FP32 faces: the three differences are exact in FP32 wherever neighbouring
-// faces are alike (two-sum error zero), and then only the three products run
-// on the narrow FP64 pipe.
-__device__ __forceinline__ double face_div(float xp, float x, float yp, float y, float zp, float z, double idx,
-                                           double idy, double idz) {
-    float dx, dy, dz, ex, ey, ez;
-    two_sum(xp, -x, dx, ex);
-    two_sum(yp, -y, dy, ey);
-    two_sum(zp, -z, dz, ez);
-    if (ex == 0.f && ey == 0.f && ez == 0.f) return widen(dx) * idx + widen(dy) * idy + widen(dz) * idz;
-    return face_div(widen(xp), widen(x), widen(yp), widen(y), widen(zp), widen(z), idx, idy, idz);
+// FP32 faces: an upper bound of its magnitude, and whether that is below
+// `least`, from pairs of FP32 values (differences exact, products and sums to
+// 2^-42 of the terms' magnitudes; ih + il = 1 / dx to 2^-48).
+__device__ __forceinline__ bool face_div_below(float xp, float x, float yp, float y, float zp, float z, float2 ix,
+                                               float2 iy, float2 iz, float least) {
+    float hi = 0.f, lo = 0.f, mag = 0.f;
+    auto term = [&](float up, float own, float2 inv) {
+        float d, e, s, r;
+        two_sum(up, -own, d, e);
+        const float p = __fmul_rn(d, inv.x);
+        const float pe = __fmaf_rn(d, inv.x, -p) + (d * inv.y + e * inv.x);
+        two_sum(hi, p, s, r);
+        hi = s;
+        lo += r + pe;
+        mag += fabsf(p);
+    };
+    term(xp, x, ix);
+    term(yp, y, iy);
+    term(zp, z, iz);
+    // NaN and overflow compare false: the caller then takes the FP64 value
+    return fabsf(hi + lo) * 1.000001f + mag * 3e-13f + 1e-37f < least;
 }
 
 // Face divergence of b per cell (the quantity constrained transport keeps at
@@ -233,15 +243,23 @@ divb_kernel(const T* __restrict__ q, const CellBlock* __restrict__ blocks, int n
             const PatchDev* __restrict__ patches, const int* __restrict__ links, long long N,
             double idx, double idy, double idz, unsigned long long* out_bits, unsigned int* flag) {
     // |d| as its FP64 bit pattern (non-negative values: an integer maximum
-    // orders them), max |b| in the grid's precision; NaN counts in neither
+    // orders them), max |b| in the grid's precision; NaN counts in neither.
+    // FP32 grids evaluate d in FP64 only where it can exceed the warp's largest
+    // so far (`least`, rounded down), which a few cells of a warp's share do:
+    // the FP64 pipe was the bound (192^3: 235 -> 88 us with the host's part).
     long long dmax = 0;
     T bmax = T(0);
+    float least = 0.f;
+    auto pair = [](double v) { const float h = float(v); return make_float2(h, float(v - double(h))); };
+    const float2 ix = pair(idx), iy = pair(idy), iz = pair(idz);
     for (int b = blockIdx.x; b < nblocks; b += gridDim.x) {
         const CellBlock cb = blocks[b];
         const PatchDev P = patches[cb.x];
         const int local = cb.y + threadIdx.x;
         const int nxy = P.nx * P.ny;
-        if (local < nxy * P.nz) {
+        const bool in = local < nxy * P.nz;
+        T bx = T(0), by = T(0), bz = T(0), xp = T(0), yp = T(0), zp = T(0);
+        if (in) {
             const int k = local / nxy;
             const int rem = local - k * nxy;
             const int j = rem / P.nx;
@@ -250,11 +268,28 @@ divb_kernel(const T* __restrict__ q, const CellBlock* __restrict__ blocks, int n
             const long long cx = chk(upper<LINKED>(patches, links, cb.x, P, i + 1, j, k), N, flag);
             const long long cy = chk(upper<LINKED>(patches, links, cb.x, P, i, j + 1, k), N, flag);
             const long long cz = chk(upper<LINKED>(patches, links, cb.x, P, i, j, k + 1), N, flag);
-            const T bx = q[5 * N + c], by = q[6 * N + c], bz = q[7 * N + c];
-            const double d = face_div(q[5 * N + cx], bx, q[6 * N + cy], by, q[7 * N + cz], bz, idx, idy, idz);
+            bx = q[5 * N + c]; by = q[6 * N + c]; bz = q[7 * N + c];
+            xp = q[5 * N + cx]; yp = q[6 * N + cy]; zp = q[7 * N + cz];
+            bmax = fmax(bmax, fmax(fabs(bx), fmax(fabs(by), fabs(bz))));
+        }
+        bool need = in;
+        if constexpr (sizeof(T) == 4) {
+            need = in && !face_div_below(xp, bx, yp, by, zp, bz, ix, iy, iz, least);
+            if (!__any_sync(0xffffffffu, need)) continue;
+        }
+        if (need) {
+            double d;
+            if constexpr (sizeof(T) == 4)
+                d = face_div(widen(xp), widen(bx), widen(yp), widen(by), widen(zp), widen(bz), idx, idy, idz);
+            else
+                d = face_div(xp, bx, yp, by, zp, bz, idx, idy, idz);
             const long long bits = __double_as_longlong(d) & 0x7fffffffffffffffll;
             if (bits <= 0x7ff0000000000000ll) dmax = max(dmax, bits);
-            bmax = fmax(bmax, fmax(fabs(bx), fmax(fabs(by), fabs(bz))));
+        }
+        if constexpr (sizeof(T) == 4) {
+#pragma unroll
+            for (int o = 16; o > 0; o >>= 1) dmax = max(dmax, __shfl_xor_sync(0xffffffffu, dmax, o));
+            least = __double2float_rd(__longlong_as_double(dmax));
         }
     }
 #pragma unroll
@@ -296,6 +331,23 @@ __global__ void set_dt_kernel(const unsigned long long* smax_bits, double cfl, d
 // patch the sum of the face means equals the sum over faces).  Pass 1: each
 // block reduces a fixed contiguous chunk in a fixed order; pass 2: one block
 // reduces the partials.  Same order on every call, so bitwise repeatable.
+// Sum over the block of each thread's eight values, in a fixed order: warp f
+// adds field f, each lane eight threads' values and then the lanes (a tree over
+// all fields on the block's first warps would queue on one scheduler's FP64
+// pipe).  Valid in lane 0 of warp f.
+__device__ __forceinline__ double block_sum8(const double (&acc)[8], double (*red)[256]) {
+#pragma unroll
+    for (int f = 0; f < 8; f++) red[f][threadIdx.x] = acc[f];
+    __syncthreads();
+    const int f = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    double s = red[f][lane];
+#pragma unroll
+    for (int u = 1; u < 8; u++) s += red[f][lane + 32 * u];
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+    return s;
+}
+
 template <class T>
 __global__ void __launch_bounds__(256)
 totals_pass1(const T* __restrict__ q, long long N, long long chunk, double* __restrict__ partial) {
@@ -304,40 +356,38 @@ totals_pass1(const T* __restrict__ q, long long N, long long chunk, double* __re
     if (end > N) end = N;
     double acc[8] = {0, 0, 0, 0, 0, 0, 0, 0};
     if constexpr (sizeof(T) == 4) {
-        // Four values are first added in FP32 with their rounding errors kept
-        // (two-sum): one FP64 addition for the four, the errors in an FP32
-        // pair of their own that joins at the end.  Each step is exact but for
-        // the pair's last bits, 2^-72 of the sum.  One FP64 addition per value
-        // was the bound (the pipe 79 % busy): 192^3 totals, div b and dt of a state: 488 -> 330 us.
-        float eh[8] = {0, 0, 0, 0, 0, 0, 0, 0}, el[8] = {0, 0, 0, 0, 0, 0, 0, 0};
-        for (long long c = beg + threadIdx.x; c < end; c += 1024) {
-            float x[8][4];
-#pragma unroll
-            for (int u = 0; u < 4; u++) {
-                const bool in = c + 256 * u < end;
-#pragma unroll
-                for (int f = 0; f < 8; f++) x[f][u] = in ? q[f * N + c + 256 * u] : 0.f;
-            }
+        // FP32 values are added in FP32 with every rounding error kept: s the
+        // running sum, eh + el the sum of its errors (two-sum at both levels,
+        // el rounds at 2^-72 of the sum), joined in FP64 at the end.  An FP64
+        // addition per value was the bound (the pipe 79 % busy): 192^3, totals
+        // of a state 153 -> 91 us with the host's part.
+        float s[8] = {0, 0, 0, 0, 0, 0, 0, 0}, eh[8] = {0, 0, 0, 0, 0, 0, 0, 0}, el[8] = {0, 0, 0, 0, 0, 0, 0, 0};
+        for (long long c = beg + threadIdx.x; c < end; c += 512) {
+            const bool two = c + 256 < end;
+            float x[8][2];
 #pragma unroll
             for (int f = 0; f < 8; f++) {
-                float s0, s1, s, e0, e1, e2, u, v, w, z;
-                two_sum(x[f][0], x[f][1], s0, e0);
-                two_sum(x[f][2], x[f][3], s1, e1);
-                two_sum(s0, s1, s, e2);
-                if (fabsf(s) <= 3.4e38f) {
-                    acc[f] += widen(s);
-                    two_sum(e0, e1, u, v);
-                    two_sum(u, e2, w, z);
-                    two_sum(eh[f], w, eh[f], u);
-                    el[f] += v + z + u;
-                } else {                       // out of the FP32 range, infinite or NaN
-#pragma unroll
-                    for (int k = 0; k < 4; k++) acc[f] += widen(x[f][k]);
-                }
+                x[f][0] = q[f * N + c];
+                x[f][1] = two ? q[f * N + c + 256] : 0.f;
             }
+#pragma unroll
+            for (int f = 0; f < 8; f++)
+#pragma unroll
+                for (int u = 0; u < 2; u++) {
+                    float e, r;
+                    two_sum(s[f], x[f][u], s[f], e);
+                    two_sum(eh[f], e, eh[f], r);
+                    el[f] += r;
+                }
         }
 #pragma unroll
-        for (int f = 0; f < 8; f++) acc[f] += double(eh[f]) + double(el[f]);
+        for (int f = 0; f < 8; f++) {
+            if (fabsf(s[f]) <= 3.4e38f && fabsf(eh[f]) <= 3.4e38f) {
+                acc[f] = widen(s[f]) + widen(eh[f] + el[f]);
+            } else {                           // out of the FP32 range, infinite or NaN
+                for (long long c = beg + threadIdx.x; c < end; c += 256) acc[f] += widen(q[f * N + c]);
+            }
+        }
     } else {
         for (long long c = beg + threadIdx.x; c < end; c += 256) {
 #pragma unroll
@@ -345,17 +395,8 @@ totals_pass1(const T* __restrict__ q, long long N, long long chunk, double* __re
         }
     }
     __shared__ double red[8][256];
-#pragma unroll
-    for (int f = 0; f < 8; f++) red[f][threadIdx.x] = acc[f];
-    __syncthreads();
-    for (int w = 128; w > 0; w >>= 1) {
-        if (threadIdx.x < w) {
-#pragma unroll
-            for (int f = 0; f < 8; f++) red[f][threadIdx.x] += red[f][threadIdx.x + w];
-        }
-        __syncthreads();
-    }
-    if (threadIdx.x < 8) partial[blockIdx.x * 8 + threadIdx.x] = red[threadIdx.x][0];
+    const double sum = block_sum8(acc, red);
+    if ((threadIdx.x & 31) == 0) partial[blockIdx.x * 8 + (threadIdx.x >> 5)] = sum;
 }
 
 __global__ void __launch_bounds__(256)
@@ -366,28 +407,11 @@ totals_pass2(const double* __restrict__ partial, int npartial, double dV, double
         for (int f = 0; f < 8; f++) acc[f] += partial[b * 8 + f];
     }
     __shared__ double red[8][256];
-#pragma unroll
-    for (int f = 0; f < 8; f++) red[f][threadIdx.x] = acc[f];
-    __syncthreads();
-    for (int w = 128; w > 0; w >>= 1) {
-        if (threadIdx.x < w) {
-#pragma unroll
-            for (int f = 0; f < 8; f++) red[f][threadIdx.x] += red[f][threadIdx.x + w];
-        }
-        __syncthreads();
-    }
-    if (threadIdx.x == 0) {
-        // state order rho, mx, my, mz, E, bx, by, bz -> ABI order
-        // rho, mx, my, mz, Bx, By, Bz, E
-        out[0] = red[0][0] * dV;
-        out[1] = red[1][0] * dV;
-        out[2] = red[2][0] * dV;
-        out[3] = red[3][0] * dV;
-        out[4] = red[5][0] * dV;
-        out[5] = red[6][0] * dV;
-        out[6] = red[7][0] * dV;
-        out[7] = red[4][0] * dV;
-    }
+    const double sum = block_sum8(acc, red);
+    // state order rho, mx, my, mz, E, bx, by, bz -> ABI order
+    // rho, mx, my, mz, Bx, By, Bz, E
+    const int f = threadIdx.x >> 5;
+    if ((threadIdx.x & 31) == 0) out[f < 4 ? f : (f == 4 ? 7 : f - 1)] = sum * dV;
 }
 
 // ABI layout (FP64, or FP32 for the FP32 entry points, type H): U[patch][8][cells]
