@@ -38,13 +38,20 @@ namespace {
 // ---- shared-memory slots per staged cell ----------------------------------
 enum : int {
     SU = 0,      // U7: rho, m_n, m_t1, m_t2, B_t1, B_t2, E        (0..6)
-    SF = 6,      // F7 in the same order: F_1..F_6 at SF + f       (7..12),
-                 // the mass flux F_0 is U_1 = m_n (see fslot)
-    SL = 13,     // |lambda_s|, s = 0..6                           (13..19)
-    SP_U = 20, SP_V1, SP_V2, SP_BN, SP_P,   // primitives for the mean
-    kNSlot = 25
+    SF = 7,      // F7 in the same order                           (7..13)
+    SL = 14,     // |lambda_s|, s = 0..6                           (14..20)
+    SP_U = 21, SP_V1, SP_V2, SP_BN, SP_P,   // primitives for the mean
+    kNSlot = 26
 };
-__host__ __device__ constexpr int fslot(int f) { return f == 0 ? SU + 1 : SF + f; }
+// Place of U_f and F_f of staged cell idx.  FP32 keeps them side by side: the
+// projection works on (U, F) pairs, one 8-byte load each; FP64 by field, the
+// mass flux F_0 being U_1 = m_n.
+template <class T> __device__ __forceinline__ constexpr int at_u(int f, int nc, int idx) {
+    return sizeof(T) == 4 ? 2 * (f * nc + idx) : (SU + f) * nc + idx;
+}
+template <class T> __device__ __forceinline__ constexpr int at_f(int f, int nc, int idx) {
+    return sizeof(T) == 4 ? 2 * (f * nc + idx) + 1 : (f == 0 ? SU + 1 : SF + f) * nc + idx;
+}
 
 template <class T> __device__ __forceinline__ T tmax(T a, T b) { return a > b ? a : b; }
 // |a| by clearing the sign bit (no floating-point compare on the FP64 pipe)
@@ -388,19 +395,18 @@ __device__ __forceinline__ void derive_cell(const SweepArgs<T>& A, const RawCell
     const T p = (g - T(1)) * (E - kin - T(0.5) * bb);
     const T pt = p + T(0.5) * bb;
     const T vb = u * bn + v1 * b1 + v2 * b2;
-    sm[(SU + 0) * nc + idx] = rho;
-    sm[(SU + 1) * nc + idx] = mn;
-    sm[(SU + 2) * nc + idx] = m1;
-    sm[(SU + 3) * nc + idx] = m2;
-    sm[(SU + 4) * nc + idx] = b1;
-    sm[(SU + 5) * nc + idx] = b2;
-    sm[(SU + 6) * nc + idx] = E;
-    sm[(SF + 1) * nc + idx] = mn * u + pt - bn * bn;
-    sm[(SF + 2) * nc + idx] = m1 * u - bn * b1;
-    sm[(SF + 3) * nc + idx] = m2 * u - bn * b2;
-    sm[(SF + 4) * nc + idx] = u * b1 - v1 * bn;
-    sm[(SF + 5) * nc + idx] = u * b2 - v2 * bn;
-    sm[(SF + 6) * nc + idx] = (E + pt) * u - bn * vb;
+    const T U[7] = {rho, mn, m1, m2, b1, b2, E};
+    const T F[7] = {mn, mn * u + pt - bn * bn, m1 * u - bn * b1, m2 * u - bn * b2, u * b1 - v1 * bn, u * b2 - v2 * bn,
+                    (E + pt) * u - bn * vb};
+#pragma unroll
+    for (int f = 0; f < 7; f++) {
+        if constexpr (sizeof(T) == 4) {
+            *reinterpret_cast<float2*>(sm + at_u<T>(f, nc, idx)) = make_float2(U[f], F[f]);
+        } else {
+            sm[at_u<T>(f, nc, idx)] = U[f];
+            if (f > 0) sm[at_f<T>(f, nc, idx)] = F[f];
+        }
+    }
     const T a2 = g * p * rinv;
     const T ca2 = bn * bn * rinv;
     // fast and slow speeds without cancellation: D = cf^2 - cs^2 from a sum
@@ -438,7 +444,7 @@ __device__ __forceinline__ void derive_cell(const SweepArgs<T>& A, const RawCell
 template <class T>
 __device__ __forceinline__ void load7(const T* __restrict__ sm, int nc, int base, int idx, T (&x)[7]) {
 #pragma unroll
-    for (int f = 0; f < 7; f++) x[f] = sm[(base == SF ? fslot(f) : base + f) * nc + idx];
+    for (int f = 0; f < 7; f++) x[f] = sm[base == SF ? at_f<T>(f, nc, idx) : at_u<T>(f, nc, idx)];
 }
 
 // first projection group: fast-, slow-, slow+, fast+ (s = 0, 2, 4, 6)
@@ -550,13 +556,13 @@ __device__ __forceinline__ void interface_flux(const T* __restrict__ sm, int nc,
     {
         const int l = id[2], r = id[3];
         const T h = T(0.5);
-        eigen<T>(h * (sm[SU * nc + l] + sm[SU * nc + r]),
+        eigen<T>(h * (sm[at_u<T>(0, nc, l)] + sm[at_u<T>(0, nc, r)]),
                  h * (sm[SP_U * nc + l] + sm[SP_U * nc + r]),
                  h * (sm[SP_V1 * nc + l] + sm[SP_V1 * nc + r]),
                  h * (sm[SP_V2 * nc + l] + sm[SP_V2 * nc + r]),
                  h * (sm[SP_BN * nc + l] + sm[SP_BN * nc + r]),
-                 h * (sm[(SU + 4) * nc + l] + sm[(SU + 4) * nc + r]),
-                 h * (sm[(SU + 5) * nc + l] + sm[(SU + 5) * nc + r]),
+                 h * (sm[at_u<T>(4, nc, l)] + sm[at_u<T>(4, nc, r)]),
+                 h * (sm[at_u<T>(5, nc, l)] + sm[at_u<T>(5, nc, r)]),
                  h * (sm[SP_P * nc + l] + sm[SP_P * nc + r]), gamma, e, bp, bstride);
     }
     T corr[7];
@@ -579,13 +585,13 @@ __device__ __forceinline__ void interface_flux(const T* __restrict__ sm, int nc,
         // U and F differences of a stencil step as one packed pair
         float2 p0[7];
 #pragma unroll
-        for (int f = 0; f < 7; f++) p0[f] = make_float2(sm[(SU + f) * nc + id[0]], sm[fslot(f) * nc + id[0]]);
+        for (int f = 0; f < 7; f++) p0[f] = *reinterpret_cast<const float2*>(sm + at_u<T>(f, nc, id[0]));
 #pragma unroll
         for (int m = 0; m < 5; m++) {
             float2 p1[7], x[7], o4[4], o3[3];
 #pragma unroll
             for (int f = 0; f < 7; f++) {
-                p1[f] = make_float2(sm[(SU + f) * nc + id[m + 1]], sm[fslot(f) * nc + id[m + 1]]);
+                p1[f] = *reinterpret_cast<const float2*>(sm + at_u<T>(f, nc, id[m + 1]));
                 x[f] = __ffma2_rn(p0[f], splat2(-1.0f), p1[f]);
             }
             project_all2(e, x, o4, o3);
@@ -690,8 +696,8 @@ __device__ __forceinline__ void interface_flux(const T* __restrict__ sm, int nc,
     const T db2 = e.be2 * dbpar + e.be1 * dbperp;
 #pragma unroll
     for (int f = 0; f < 7; f++) {
-        const T* F = sm + fslot(f) * nc;
-        out[f] = (T(7) * (F[id[2]] + F[id[3]]) - (F[id[1]] + F[id[4]])) * T(1.0 / 12.0);
+        auto F = [&](int m) { return sm[at_f<T>(f, nc, id[m])]; };
+        out[f] = (T(7) * (F(2) + F(3)) - (F(1) + F(4))) * T(1.0 / 12.0);
     }
     out[0] += drho;
     out[1] += e.u * drho + e.rho * du;
@@ -801,10 +807,10 @@ __device__ void harvest_one(const HarvestArgs<T>& H, long long t, T* sm, int nc,
     {
         const int l = id[2], r = id[3];
         const T h = T(0.5);
-        eigen<T>(h * (sm[SU * nc + l] + sm[SU * nc + r]), h * (sm[SP_U * nc + l] + sm[SP_U * nc + r]),
+        eigen<T>(h * (sm[at_u<T>(0, nc, l)] + sm[at_u<T>(0, nc, r)]), h * (sm[SP_U * nc + l] + sm[SP_U * nc + r]),
                  h * (sm[SP_V1 * nc + l] + sm[SP_V1 * nc + r]), h * (sm[SP_V2 * nc + l] + sm[SP_V2 * nc + r]),
-                 h * (sm[SP_BN * nc + l] + sm[SP_BN * nc + r]), h * (sm[(SU + 4) * nc + l] + sm[(SU + 4) * nc + r]),
-                 h * (sm[(SU + 5) * nc + l] + sm[(SU + 5) * nc + r]), h * (sm[SP_P * nc + l] + sm[SP_P * nc + r]),
+                 h * (sm[SP_BN * nc + l] + sm[SP_BN * nc + r]), h * (sm[at_u<T>(4, nc, l)] + sm[at_u<T>(4, nc, r)]),
+                 h * (sm[at_u<T>(5, nc, l)] + sm[at_u<T>(5, nc, r)]), h * (sm[SP_P * nc + l] + sm[SP_P * nc + r]),
                  T(H.gamma), e, bp, bstride);
     }
     T hu[7], hf[7];
@@ -906,8 +912,8 @@ __global__ void __launch_bounds__(128) cell_state_flux_kernel(const SweepArgs<T>
     load_cell<T>(A, P, i, j, k, r, c);
     derive_cell<T, AXIS>(A, r, c, sm, nc, threadIdx.x, false);
     for (int f = 0; f < 7; f++) {
-        X[f * np + t] = double(sm[(SU + f) * nc + threadIdx.x]);
-        F[f * np + t] = double(sm[fslot(f) * nc + threadIdx.x]);
+        X[f * np + t] = double(sm[at_u<T>(f, nc, threadIdx.x)]);
+        F[f * np + t] = double(sm[at_f<T>(f, nc, threadIdx.x)]);
     }
 }
 

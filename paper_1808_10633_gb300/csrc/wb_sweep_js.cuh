@@ -298,7 +298,7 @@ __device__ __forceinline__ void sweep_flux(const typename Lanes<V>::S* __restric
 #pragma unroll
     for (int f = 0; f < 7; f++) u0[f] = ld<V>(cell + (SU + f) * nc);
 #pragma unroll
-    for (int f = 0; f < 6; f++) f0[f] = ld<V>(cell + (SF + 1 + f) * nc);
+    for (int f = 0; f < 6; f++) f0[f] = ld<V>(cell + at_f<S>(f + 1, nc, 0));
 #pragma unroll
     for (int m = 0; m < 5; m++) {
         V x[7], w4[4], w3[3], g4[4], g3[3];
@@ -313,7 +313,7 @@ __device__ __forceinline__ void sweep_flux(const typename Lanes<V>::S* __restric
         x[0] = dm;
 #pragma unroll
         for (int f = 0; f < 6; f++) {
-            const V f1 = ld<V>(cell + (SF + 1 + f) * nc + (m + 1) * CS);
+            const V f1 = ld<V>(cell + at_f<S>(f + 1, nc, (m + 1) * CS));
             x[f + 1] = vsub(f1, f0[f]);
             f0[f] = f1;
         }
@@ -378,7 +378,7 @@ __device__ __forceinline__ void sweep_flux(const typename Lanes<V>::S* __restric
     dF[6] = vfma(e.hv2, drho, vsub(dpg, vfma(e.nbm, dbpar, vmul(e.rho, vdv))));
 #pragma unroll
     for (int f = 0; f < 7; f++) {
-        const typename Lanes<V>::S* F = cell + fslot(f) * nc;
+        const S* F = cell + at_f<S>(f, nc, 0);
         const V in = vadd(ld<V>(F + 2 * CS), ld<V>(F + 3 * CS)), ex = vadd(ld<V>(F + CS), ld<V>(F + 4 * CS));
         out[f] = vfma(in, splat<V>(S(7.0 / 12.0)), vfma(ex, splat<V>(S(-1.0 / 12.0)), dF[f]));
     }
@@ -487,7 +487,7 @@ __device__ __forceinline__ void flat_body(const SweepArgs<T>& A, const Tile& til
     T F[7];
 #pragma unroll
     for (int f = 0; f < 7; f++) {
-        const T f2 = sm[fslot(f) * kSweepNT + tid] + sm[fslot(f) * kSweepNT + tid];
+        const T f1 = sm[at_f<T>(f, kSweepNT, tid)], f2 = f1 + f1;
         if constexpr (sizeof(T) == 8) F[f] = fma(f2, 7.0 / 12.0, f2 * (-1.0 / 12.0));
         else F[f] = (T(7) * f2 - f2) * T(1.0 / 12.0);
     }
