@@ -49,6 +49,42 @@ __device__ __forceinline__ long long locate(const PatchDev* __restrict__ patches
     return Q.off + ((long long)k * Q.ny + j) * Q.nx + i;
 }
 
+// The 27 patches round the patch of a block, in shared memory: a block that
+// looks up many cells of one patch loads its links and their patch records once
+// (two dependent loads) instead of per cell.
+struct LinkTab {
+    long long off[27];
+    int nx[27], ny[27], nz[27];
+    // every thread of the block calls it; tid: its linear index
+    __device__ __forceinline__ void load(const PatchDev* __restrict__ patches, const int* __restrict__ links, int p,
+                                         int tid) {
+        if (tid < 27) {
+            const PatchDev Q = patches[links[27 * p + tid]];
+            off[tid] = Q.off;
+            nx[tid] = Q.nx;
+            ny[tid] = Q.ny;
+            nz[tid] = Q.nz;
+        }
+        __syncthreads();
+    }
+    // locate() from the table; P the block's patch
+    __device__ __forceinline__ long long at(const PatchDev& P, int i, int j, int k) const {
+        const int ox = i < 0 ? -1 : (i >= P.nx ? 1 : 0);
+        const int oy = j < 0 ? -1 : (j >= P.ny ? 1 : 0);
+        const int oz = k < 0 ? -1 : (k >= P.nz ? 1 : 0);
+        const int d = 9 * (oz + 1) + 3 * (oy + 1) + (ox + 1);
+        const int qx = nx[d], qy = ny[d], qz = nz[d];
+        i = ox < 0 ? i + qx : (ox > 0 ? i - P.nx : i);
+        j = oy < 0 ? j + qy : (oy > 0 ? j - P.ny : j);
+        k = oz < 0 ? k + qz : (oz > 0 ? k - P.nz : k);
+        // a patch linked to itself along an axis shorter than the stencil reach
+        if ((unsigned)i >= (unsigned)qx) i = wrap_cell(i, qx);
+        if ((unsigned)j >= (unsigned)qy) j = wrap_cell(j, qy);
+        if ((unsigned)k >= (unsigned)qz) k = wrap_cell(k, qz);
+        return off[d] + ((long long)k * qy + j) * qx + i;
+    }
+};
+
 // Bounds-checked builds (WB_BOUNDS_CHECK=1, the library's "check" variant):
 // each global or shared index the solver kernels form is tested against its
 // array; an index outside it sets kFlagBounds in the grid's status word and

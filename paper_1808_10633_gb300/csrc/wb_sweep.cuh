@@ -343,12 +343,13 @@ __device__ __forceinline__ int tile_cell(const PatchDev& P, int ia, int ip, int 
     return (k * P.ny + j) * P.nx + i;
 }
 
-// Cell (i, j, k) of patch p as a tile meets it: outside the patch along the
-// sweep axis where the stencil reaches past its end.  Most cells lie inside with
+// Cell (i, j, k) of a tile's patch as the tile meets it: outside along the
+// sweep axis where the stencil reaches past the patch's end (tab: its links, of
+// a linked grid).  Most cells lie inside with
 // their three upper neighbours and need no wrap and no link.
 template <class T, int AXIS>
-__device__ __forceinline__ void load_cell_tile(const SweepArgs<T>& A, int p, const PatchDev& P, int i, int j, int k,
-                                               RawCell<T>& r, long long& c) {
+__device__ __forceinline__ void load_cell_tile(const SweepArgs<T>& A, const LinkTab& tab, const PatchDev& P, int i,
+                                               int j, int k, RawCell<T>& r, long long& c) {
     long long cx, cy, cz;
     const int nxy = P.nx * P.ny;
     if ((unsigned)i < (unsigned)(P.nx - 1) && (unsigned)j < (unsigned)(P.ny - 1) && (unsigned)k < (unsigned)(P.nz - 1)) {
@@ -357,10 +358,10 @@ __device__ __forceinline__ void load_cell_tile(const SweepArgs<T>& A, int p, con
         cy = c + P.nx;
         cz = c + nxy;
     } else if (A.links) {
-        c = locate(A.patches, A.links, p, P, i, j, k);
-        cx = locate(A.patches, A.links, p, P, i + 1, j, k);
-        cy = locate(A.patches, A.links, p, P, i, j + 1, k);
-        cz = locate(A.patches, A.links, p, P, i, j, k + 1);
+        c = tab.at(P, i, j, k);
+        cx = tab.at(P, i + 1, j, k);
+        cy = tab.at(P, i, j + 1, k);
+        cz = tab.at(P, i, j, k + 1);
     } else {
         if (AXIS == 0) i = wrap_near(i, P.nx);
         else if (AXIS == 1) j = wrap_near(j, P.ny);

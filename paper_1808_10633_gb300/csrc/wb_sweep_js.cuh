@@ -413,6 +413,9 @@ __device__ __forceinline__ void tile_body(const SweepArgs<T>& A, const Tile& til
     const int na = AXIS == 0 ? P.nx : (AXIS == 1 ? P.ny : P.nz);
     const int np = AXIS == 0 ? P.ny : P.nx, n3 = AXIS == 2 ? P.ny : P.nz;
 
+    __shared__ LinkTab tab;
+    if (A.links) tab.load(A.patches, A.links, tile.x, tid);
+
     // staging: cells tile.y-3 .. tile.y+TA+1 along the axis, TP pencils
     constexpr int NIT = (NC + NT - 1) / NT;
     RawCell<T> raw[NIT];
@@ -434,7 +437,7 @@ __device__ __forceinline__ void tile_body(const SweepArgs<T>& A, const Tile& til
             if (AXIS == 0) { i = raw_a; j = cp; k = w; }
             else if (AXIS == 1) { i = cp; j = raw_a; k = w; }
             else { i = cp; j = w; k = raw_a; }
-            load_cell_tile<T, AXIS>(A, tile.x, P, i, j, k, raw[it], rc[it]);
+            load_cell_tile<T, AXIS>(A, tab, P, i, j, k, raw[it], rc[it]);
         }
     }
 #pragma unroll

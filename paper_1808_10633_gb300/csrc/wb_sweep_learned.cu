@@ -493,6 +493,8 @@ __global__ void __launch_bounds__(kLearnedNT, WB_LEARNED_MINB) sweep_learned_ker
     for (int i = tid; i < kMlpSmemWords; i += TA * TP) Wsm[i] = mlp[i];
 #endif
 
+    __shared__ LinkTab tab;
+    if (A.links) tab.load(A.patches, A.links, tile.x, tid);
     constexpr int NIT = (NC + TA * TP - 1) / (TA * TP);
     RawCell<T> raw[NIT];
     long long rc[NIT];
@@ -515,7 +517,7 @@ __global__ void __launch_bounds__(kLearnedNT, WB_LEARNED_MINB) sweep_learned_ker
             if (AXIS == 0) { i = raw_a; j = cp; k = w; }
             else if (AXIS == 1) { i = cp; j = raw_a; k = w; }
             else { i = cp; j = w; k = raw_a; }
-            load_cell_tile<T, AXIS>(A, tile.x, P, i, j, k, raw[it], rc[it]);
+            load_cell_tile<T, AXIS>(A, tab, P, i, j, k, raw[it], rc[it]);
         }
     }
 #pragma unroll

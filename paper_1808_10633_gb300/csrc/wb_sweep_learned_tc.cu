@@ -399,6 +399,8 @@ __global__ void __launch_bounds__(kTcNT, 2) sweep_learned_tc_kernel(const SweepA
     const PatchDev P = A.patches[tile.x & 0xffffff];
     const int na = AXIS == 0 ? P.nx : (AXIS == 1 ? P.ny : P.nz);
     const int np = AXIS == 0 ? P.ny : P.nx, n3 = AXIS == 2 ? P.ny : P.nz;
+    __shared__ LinkTab tab;
+    if (A.links) tab.load(A.patches, A.links, tile.x & 0xffffff, tid);
     constexpr int NIT = (NC + kTcNT - 1) / kTcNT;
     RawCell<T> raw[NIT];
     long long rc[NIT];
@@ -421,7 +423,7 @@ __global__ void __launch_bounds__(kTcNT, 2) sweep_learned_tc_kernel(const SweepA
             if (AXIS == 0) { i = raw_a; j = cp; k = w; }
             else if (AXIS == 1) { i = cp; j = raw_a; k = w; }
             else { i = cp; j = w; k = raw_a; }
-            load_cell_tile<T, AXIS>(A, tile.x & 0xffffff, P, i, j, k, raw[it], rc[it]);
+            load_cell_tile<T, AXIS>(A, tab, P, i, j, k, raw[it], rc[it]);
         }
     }
 #pragma unroll

@@ -99,18 +99,16 @@ __device__ __forceinline__ T combine_value(int integrator, int stage, T un, T uk
 
 // Cell (i, j, k) of patch p, where an index one step outside the patch
 // wraps round a periodic patch or, with LINKED, reaches the neighbouring
-// patch through the link table.
+// patch through the block's table of links (tab).
 template <class T, bool LINKED>
 struct Geo {
     const PatchDev P;
-    const PatchDev* __restrict__ patches;
-    const int* __restrict__ links;
-    int p;
+    const LinkTab& tab;
     long long N;
     unsigned int* flag;
     __device__ __forceinline__ long long at(int i, int j, int k) const {
         if constexpr (LINKED) {
-            return chk(locate(patches, links, p, P, i, j, k), N, flag);
+            return chk(tab.at(P, i, j, k), N, flag);
         } else {
             i = i < 0 ? i + P.nx : (i >= P.nx ? i - P.nx : i);
             j = j < 0 ? j + P.ny : (j >= P.ny ? j - P.ny : j);
@@ -125,7 +123,9 @@ struct Geo {
 template <class T, bool LINKED>
 __global__ void __launch_bounds__(kCellBlock) emf_kernel(const UpdateArgs<T> A) {
     const CellBlock cb = A.blocks[blockIdx.x];
-    const Geo<T, LINKED> G{A.patches[cb.x], A.patches, A.links, cb.x, A.ncells, A.flag};
+    __shared__ LinkTab tab;
+    if constexpr (LINKED) tab.load(A.patches, A.links, cb.x, threadIdx.x);
+    const Geo<T, LINKED> G{A.patches[cb.x], tab, A.ncells, A.flag};
     const int local = cb.y + threadIdx.x;
     const int nxy = G.P.nx * G.P.ny;
     if (local >= nxy * G.P.nz) return;
@@ -161,7 +161,9 @@ template <class T, bool LINKED>
 __global__ void __launch_bounds__(kCellBlock / 2) emf_kernel2(const UpdateArgs<T> A) {
     constexpr int H = kCellBlock / 2;
     const CellBlock cb = A.blocks[blockIdx.x];
-    const Geo<T, LINKED> G{A.patches[cb.x], A.patches, A.links, cb.x, A.ncells, A.flag};
+    __shared__ LinkTab tab;
+    if constexpr (LINKED) tab.load(A.patches, A.links, cb.x, threadIdx.x);
+    const Geo<T, LINKED> G{A.patches[cb.x], tab, A.ncells, A.flag};
     const int nxy = G.P.nx * G.P.ny, np = nxy * G.P.nz;
     const int local0 = cb.y + threadIdx.x;
     if (local0 >= np) return;
@@ -205,7 +207,9 @@ __global__ void __launch_bounds__(kCellBlock / 2) emf_kernel2(const UpdateArgs<T
 template <class T, bool LINKED>
 __global__ void __launch_bounds__(kCellBlock, 4) update_kernel(const UpdateArgs<T> A) {
     const CellBlock cb = A.blocks[blockIdx.x];
-    const Geo<T, LINKED> G{A.patches[cb.x], A.patches, A.links, cb.x, A.ncells, A.flag};
+    __shared__ LinkTab tab;
+    if constexpr (LINKED) tab.load(A.patches, A.links, cb.x, threadIdx.x);
+    const Geo<T, LINKED> G{A.patches[cb.x], tab, A.ncells, A.flag};
     const int local = cb.y + threadIdx.x;
     const int nxy = G.P.nx * G.P.ny;
     if (local >= nxy * G.P.nz) return;
@@ -255,7 +259,9 @@ template <class T, bool LINKED>
 __global__ void __launch_bounds__(kCellBlock / 2, 6) update_kernel2(const UpdateArgs<T> A) {
     constexpr int H = kCellBlock / 2;
     const CellBlock cb = A.blocks[blockIdx.x];
-    const Geo<T, LINKED> G{A.patches[cb.x], A.patches, A.links, cb.x, A.ncells, A.flag};
+    __shared__ LinkTab tab;
+    if constexpr (LINKED) tab.load(A.patches, A.links, cb.x, threadIdx.x);
+    const Geo<T, LINKED> G{A.patches[cb.x], tab, A.ncells, A.flag};
     const int nxy = G.P.nx * G.P.ny, np = nxy * G.P.nz;
     const int local0 = cb.y + threadIdx.x;
     if (local0 >= np) return;
@@ -327,7 +333,9 @@ __global__ void __launch_bounds__(kCellBlock / 2, 6) update_kernel2(const Update
 template <class T, bool LINKED>
 __global__ void __launch_bounds__(kCellBlock / 2) ct_update_kernel(const UpdateArgs<T> A) {
     const CellBlock cb = A.blocks[blockIdx.x >> 1];
-    const Geo<T, LINKED> G{A.patches[cb.x], A.patches, A.links, cb.x, A.ncells, A.flag};
+    __shared__ LinkTab tab;
+    if constexpr (LINKED) tab.load(A.patches, A.links, cb.x, threadIdx.x);
+    const Geo<T, LINKED> G{A.patches[cb.x], tab, A.ncells, A.flag};
     const int local = cb.y + (blockIdx.x & 1) * (kCellBlock / 2) + threadIdx.x;
     const int nx = G.P.nx, nxy = nx * G.P.ny;
     if (local >= nxy * G.P.nz) return;
