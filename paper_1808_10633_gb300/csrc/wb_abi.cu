@@ -102,7 +102,6 @@ struct wb_grid {
     uint32_t* d_mlp = nullptr;            // learned weights, fragment order
     void* d_mlp_tc = nullptr;             // learned weights, tensor-core shared-memory image
     unsigned long long* d_lstats = nullptr;   // detector firings, decisions (learned grids)
-    int* d_queue = nullptr;               // per-axis tile counters of the persistent sweeps
     int step_totals = 0;                  // 1: every step also takes the totals of its start state
     cudaStream_t side = nullptr;          // stream the per-step totals run on
     cudaEvent_t ev_fork = nullptr, ev_join = nullptr;
@@ -111,9 +110,8 @@ struct wb_grid {
     cudaStream_t branch[3] = {nullptr, nullptr, nullptr};
     cudaEvent_t ev_branch[4] = {nullptr, nullptr, nullptr, nullptr};   // their ends, and the forks
     double kappa = 4.0, pjump = 0.5, smooth = 1.03;   // detector thresholds, smoothness gate
-    int tile_policy[3] = {-2, -2, -2};    // build_tiles policy of each axis' table
-    int tile_split[3][4] = {};            // per axis: tiles of each shape of a table sorted
-                                          // by shape, or all 0 (wb::SweepArgs::split)
+    int tile_policy[3] = {-1, -1, -1};    // build_tiles policy of each axis' table
+    int tile_split[3][4] = {};            // per axis: tiles of each shape (wb::SweepArgs::split)
     wb::PatchDev* d_patches = nullptr;
     std::vector<wb::PatchDev> h_patches;
     bool links = false;                   // the descriptor links patches
@@ -142,20 +140,11 @@ namespace {
 constexpr int kNTileCandidate = WB_NTILE_CANDIDATE;   // tile tables wb_autotune times per axis
 static_assert(WB_NTILE_SHAPE == wb::kNTileShape, "tile shape count");
 
-// Tiles of each shape when the table is sorted by shape (then each shape
-// runs as its own fixed-shape launch), else all 0.
+// Tiles of each shape of a table (sorted by shape: each shape runs as its own
+// fixed-shape launch).
 void tile_split(const std::vector<wb::Tile>& t, int split[4]) {
     split[0] = split[1] = split[2] = split[3] = 0;
-    int prev = 0;
-    for (const wb::Tile& x : t) {
-        const int sh = (int)((unsigned)x.x >> 24);
-        if (sh < prev || sh > wb::kFlatShape) {
-            split[0] = split[1] = split[2] = split[3] = 0;
-            return;
-        }
-        split[sh]++;
-        prev = sh;
-    }
+    for (const wb::Tile& x : t) split[(unsigned)x.x >> 24]++;
 }
 
 template <class T>
@@ -209,7 +198,6 @@ int enqueue_stages(wb_grid* g, Prof* pf) {
             a.zweights = g->weights;
             set_split(a, g->tile_split[axis]);
             a.lstats = g->d_lstats;
-            a.queue = g->d_queue + axis;
             a.flag = g->d_flag;
             const bool forked = axis > 0 && !pf;
             if (axis == 0 && !pf)
@@ -221,9 +209,9 @@ int enqueue_stages(wb_grid* g, Prof* pf) {
                 if (g->precision == WB_FP32_LEARNED)
                     WB_CK(launch_learned(g, axis, a, s));
                 else
-                    WB_CK(wb::launch_sweep<T>(axis, a, g->ntiles[axis], s));
+                    WB_CK(wb::launch_sweep<T>(axis, a, s));
             } else {
-                WB_CK(wb::launch_sweep<T>(axis, a, g->ntiles[axis], s));
+                WB_CK(wb::launch_sweep<T>(axis, a, s));
             }
             if ((rc = prof_end(pf, g->stream, WB_K_SWEEP_X + axis)) != WB_OK) return rc;
         }
@@ -431,7 +419,7 @@ void release(wb_grid* g) {
     if (g->stream) cudaStreamSynchronize(g->stream);
     if (g->graph) cudaGraphExecDestroy(g->graph);
     if (g->side) cudaStreamSynchronize(g->side);
-    void* ptrs[] = {g->un, g->uk, g->acc, g->flux, g->er, g->emf, g->d_mlp, g->d_mlp_tc, g->d_lstats, g->d_queue,
+    void* ptrs[] = {g->un, g->uk, g->acc, g->flux, g->er, g->emf, g->d_mlp, g->d_mlp_tc, g->d_lstats,
                     g->d_patches, g->d_links, g->d_tiles[0], g->d_tiles[1], g->d_tiles[2], g->d_blocks,
                     g->d_vblocks, g->d_scalars, g->d_smax, g->d_flag, g->d_partial, g->d_io};
     for (void* p : ptrs)
@@ -452,7 +440,7 @@ void release(wb_grid* g) {
 // everywhere; policy < 0: per patch the shape needing the fewest thread slots
 // (ragged tiles at the patch edges idle threads), ties to the lower shape
 // (FP64: to the longer tile);
-// policy -2 then orders the table by shape (a fixed-shape launch per shape).
+// the table is ordered by shape (a fixed-shape launch per shape).
 // A periodic patch one cell deep along the axis takes flat tiles under every
 // policy (the learned sweep counts its decisions there as everywhere).
 // The shape goes into the top byte of the tile's patch field.
@@ -517,8 +505,7 @@ std::vector<wb::Tile> build_tiles(const wb_grid* g, int axis, int policy) {
             q = end;
         }
     }
-    if (policy != -1)
-        std::stable_sort(out.begin(), out.end(), [](const wb::Tile& a, const wb::Tile& b) {
+    std::stable_sort(out.begin(), out.end(), [](const wb::Tile& a, const wb::Tile& b) {
             return ((unsigned)a.x >> 24) < ((unsigned)b.x >> 24);
         });
     return out;
@@ -609,10 +596,10 @@ int face_fluxes_impl(wb_grid* g, int axis, double* F_out) {
             if (!g->d_mlp) return fail(WB_EINVAL, "learned grid: install the networks with wb_set_mlp first");
             WB_CK(launch_learned(g, axis, a, g->stream));
         } else {
-            WB_CK(wb::launch_sweep<T>(axis, a, g->ntiles[axis], g->stream));
+            WB_CK(wb::launch_sweep<T>(axis, a, g->stream));
         }
     } else {
-        WB_CK(wb::launch_sweep<T>(axis, a, g->ntiles[axis], g->stream));
+        WB_CK(wb::launch_sweep<T>(axis, a, g->stream));
     }
     // 7 N doubles fit the 11 N staging buffer
     WB_CK(wb::launch_export_flux<T>(flux, g->d_io, g->d_blocks, g->d_patches, N, g->nblocks,
@@ -624,7 +611,7 @@ int face_fluxes_impl(wb_grid* g, int axis, double* F_out) {
 }
 
 template <class T>
-int time_sweep(wb_grid* g, int axis, const wb::Tile* tiles, int ntiles, const int split[4], float* ms) {
+int time_sweep(wb_grid* g, int axis, const wb::Tile* tiles, const int split[4], float* ms) {
     wb::SweepArgs<T> a;
     a.src = static_cast<const T*>(g->un);
     a.flux = static_cast<T*>(g->flux) + (long long)axis * wb::kNFlux * g->N;
@@ -637,15 +624,14 @@ int time_sweep(wb_grid* g, int axis, const wb::Tile* tiles, int ntiles, const in
     a.rg1 = 1.0 / (g->gamma - 1.0);
     a.zweights = g->weights;
     set_split(a, split);
-    a.queue = g->d_queue + axis;
     a.flag = g->d_flag;
     cudaEvent_t e0, e1;
     WB_CK(cudaEventCreate(&e0));
     WB_CK(cudaEventCreate(&e1));
-    WB_CK(wb::launch_sweep<T>(axis, a, ntiles, g->stream));
+    WB_CK(wb::launch_sweep<T>(axis, a, g->stream));
     WB_CK(cudaEventRecord(e0, g->stream));
-    WB_CK(wb::launch_sweep<T>(axis, a, ntiles, g->stream));
-    WB_CK(wb::launch_sweep<T>(axis, a, ntiles, g->stream));
+    WB_CK(wb::launch_sweep<T>(axis, a, g->stream));
+    WB_CK(wb::launch_sweep<T>(axis, a, g->stream));
     WB_CK(cudaEventRecord(e1, g->stream));
     WB_CK(cudaEventSynchronize(e1));
     cudaEventElapsedTime(ms, e0, e1);
@@ -744,7 +730,7 @@ int wb_init_grid(const wb_grid_desc* d, const double* U0, const double* b0, void
     // tiles and cell blocks
     std::vector<wb::Tile> tiles[3];
     std::vector<wb::CellBlock> blocks;
-    for (int a = 0; a < 3; a++) tiles[a] = build_tiles(g, a, g->precision == WB_FP32_LEARNED ? 0 : -2);
+    for (int a = 0; a < 3; a++) tiles[a] = build_tiles(g, a, g->precision == WB_FP32_LEARNED ? 0 : -1);
     for (int p = 0; p < g->npatch; p++) {
         const wb::PatchDev& P = g->h_patches[p];
         const long long np = (long long)P.nx * P.ny * P.nz;
@@ -794,7 +780,6 @@ int wb_init_grid(const wb_grid_desc* d, const double* U0, const double* b0, void
     if ((rc = dmalloc(g, &g->d_io, sizeof(double) * 11 * N))) return bail(rc);
     if (g->precision == WB_FP32_LEARNED &&
         (rc = dmalloc(g, &g->d_lstats, sizeof(unsigned long long) * 2))) return bail(rc);
-    if ((rc = dmalloc(g, &g->d_queue, sizeof(int) * 3))) return bail(rc);
     if (cudaMallocHost(reinterpret_cast<void**>(&g->h_small), 256) != cudaSuccess)
         return bail(fail(WB_ENOMEM, "pinned host allocation failed"));
 
@@ -1154,10 +1139,9 @@ int wb_set_mlp_gate(wb_grid* g, double smooth) {
 
 namespace {
 
-// build_tiles policy of wb_autotune's candidate table c: 0 the per-patch
-// model (one persistent launch), 1..3 each fixed shape, 4 the per-patch
-// model ordered by shape (a launch per shape)
-int candidate_policy(int c) { return c == 0 ? -1 : (c <= wb::kNTileShape ? c - 1 : -2); }
+// build_tiles policy of wb_autotune's candidate table c: 0 and 4 the per-patch
+// model, 1..3 each fixed shape
+int candidate_policy(int c) { return c >= 1 && c <= wb::kNTileShape ? c - 1 : -1; }
 
 // Builds and uploads the tile table of `axis` for `policy` (synchronous).
 int install_tiles(wb_grid* g, int axis, int policy) {
@@ -1194,8 +1178,6 @@ int wb_autotune(wb_grid* g, double* ms_out) {
         float best_ms = -1.f;
         int best = -1;
         for (int c = 0; c < kNTileCandidate; c++) {
-            // 0: per-patch model (one persistent launch), 1..3: each fixed
-            // shape, 4: the per-patch model sorted by shape (a launch per shape)
             const int policy = candidate_policy(c);
             std::vector<wb::Tile> t = build_tiles(g, axis, policy);
             wb::Tile* d = nullptr;
@@ -1207,8 +1189,8 @@ int wb_autotune(wb_grid* g, double* ms_out) {
             int split[4];
             tile_split(t, split);
             if (rc == WB_OK)
-                rc = g->precision == WB_FP64 ? time_sweep<double>(g, axis, d, (int)t.size(), split, &ms)
-                                             : time_sweep<float>(g, axis, d, (int)t.size(), split, &ms);
+                rc = g->precision == WB_FP64 ? time_sweep<double>(g, axis, d, split, &ms)
+                                             : time_sweep<float>(g, axis, d, split, &ms);
             cudaFree(d);
             if (rc != WB_OK) return rc;
             if (ms_out) ms_out[axis * kNTileCandidate + c] = ms;

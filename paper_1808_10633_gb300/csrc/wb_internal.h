@@ -185,11 +185,9 @@ struct SweepArgs {
     double rg1 = 0;                // 1 / (gamma - 1) (the Jiang-Shu and WENO-Z sweeps)
     int zweights = 0;              // 1: WENO-Z weights instead of Jiang-Shu
     unsigned long long* lstats = nullptr;   // learned sweep: detector firings, decisions
-    int* queue = nullptr;          // persistent sweep: tile counter of this launch (or fixed stride)
-    int split[4] = {0, 0, 0, 0};   // tiles of shape 0, 1, 2 and flat ones of a table
-                                   // sorted by shape (one fixed launch per shape, a
-                                   // tile per block);
-                                   // all 0: the persistent runtime-shape launch
+    int split[4] = {0, 0, 0, 0};   // tiles of shape 0, 1, 2 and flat ones of the table,
+                                   // which is sorted by shape (a launch per shape, a
+                                   // tile per block; not the learned sweeps')
     unsigned int* flag = nullptr;  // status word (bounds-checked builds)
 };
 
@@ -221,7 +219,7 @@ int set_last_error(int code, const char* msg);
 
 // ---- launchers (one per translation unit) ---------------------------------
 template <class T>
-cudaError_t launch_sweep(int axis, const SweepArgs<T>& a, int ntiles, cudaStream_t s);
+cudaError_t launch_sweep(int axis, const SweepArgs<T>& a, cudaStream_t s);
 template <class T>
 cudaError_t prepare_sweep_kernels();
 // Tile shape s (0 = default, kNTileShape alternatives) of the sweep along

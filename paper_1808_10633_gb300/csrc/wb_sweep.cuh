@@ -739,11 +739,6 @@ __host__ __device__ constexpr int shape_ta(int axis, int s) {
 }
 constexpr int kNShape = 3;
 __host__ __device__ constexpr int nc_of(int ta) { return (ta + 5) * (kSweepNT / ta); }
-__host__ __device__ constexpr int max_nc(int axis) {
-    return nc_of(shape_ta(axis, 0)) > nc_of(shape_ta(axis, 1))
-               ? (nc_of(shape_ta(axis, 0)) > nc_of(shape_ta(axis, 2)) ? nc_of(shape_ta(axis, 0)) : nc_of(shape_ta(axis, 2)))
-               : (nc_of(shape_ta(axis, 1)) > nc_of(shape_ta(axis, 2)) ? nc_of(shape_ta(axis, 1)) : nc_of(shape_ta(axis, 2)));
-}
 
 }  // namespace
 }  // namespace wb

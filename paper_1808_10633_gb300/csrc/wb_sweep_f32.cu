@@ -3,5 +3,5 @@
 
 namespace wb {
 template cudaError_t prepare_sweep_kernels<float>();
-template cudaError_t launch_sweep<float>(int, const SweepArgs<float>&, int, cudaStream_t);
+template cudaError_t launch_sweep<float>(int, const SweepArgs<float>&, cudaStream_t);
 }  // namespace wb

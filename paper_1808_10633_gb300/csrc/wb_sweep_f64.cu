@@ -10,7 +10,7 @@ void sweep_shape(int axis, int s, int* ta, int* tp) {
 }
 
 template cudaError_t prepare_sweep_kernels<double>();
-template cudaError_t launch_sweep<double>(int, const SweepArgs<double>&, int, cudaStream_t);
+template cudaError_t launch_sweep<double>(int, const SweepArgs<double>&, cudaStream_t);
 template cudaError_t launch_harvest<double>(const double*, long long, const PatchDev&, int,
                                             const long long*, long long, const double*,
                                             const double*, double, double, double, float*,

@@ -506,45 +506,11 @@ __global__ void __launch_bounds__(kSweepNT) sweep_flat_kernel(const SweepArgs<T>
     flat_body<T, AXIS>(A, tile, P, reinterpret_cast<T*>(smem_raw), threadIdx.x);
 }
 
-// Persistent sweep: a grid of (SMs x resident blocks) takes tiles of any
-// shape from a work counter, so patches of uneven sizes share one launch;
-// each tile runs the body compiled for its shape (a block-uniform switch).
-// Serves tile tables that are not ordered by shape.
-template <class T, int AXIS, bool Z>
-__global__ void __launch_bounds__(kSweepNT, kMinBlocks<T>) sweep_kernel(const SweepArgs<T> A, int ntiles) {
-    constexpr int NCMAX = max_nc(AXIS);
-    extern __shared__ __align__(16) unsigned char smem_raw[];
-    T* sm = reinterpret_cast<T*>(smem_raw);
-    const int tid = threadIdx.x;
-    __shared__ int next_tile;
-    // work queue: each block starts on tile blockIdx.x and then takes the next
-    // unclaimed tile from the launch's counter (zeroed before the launch), so
-    // uneven tiles balance across SMs; without a counter, a fixed stride
-    for (int t = blockIdx.x; t < ntiles;) {
-        Tile tile = A.tiles[t];
-        const int shape = (unsigned)tile.x >> 24;
-        tile.x &= 0xffffff;
-        const PatchDev P = A.patches[tile.x];
-        if (shape == 0) tile_body<T, AXIS, shape_ta(AXIS, 0), NCMAX, Z>(A, tile, P, sm, tid);
-        else if (shape == 1) tile_body<T, AXIS, shape_ta(AXIS, 1), NCMAX, Z>(A, tile, P, sm, tid);
-        else if (shape == 2) tile_body<T, AXIS, shape_ta(AXIS, 2), NCMAX, Z>(A, tile, P, sm, tid);
-        else flat_body<T, AXIS>(A, tile, P, sm, tid);
-        __syncthreads();
-        if (A.queue) {
-            if (tid == 0) next_tile = gridDim.x + atomicAdd(A.queue, 1);
-            __syncthreads();
-            t = next_tile;
-        } else {
-            t += gridDim.x;
-        }
-    }
-}
-
-// One tile per block of one shape S: the launch for tile tables that use one
-// shape throughout (a single grid, or patches tuned to it), and for each
-// shape's range of a table sorted by shape, with either weights.  (WENO-Z on
-// the persistent kernel, whose three bodies share one register allocation and
-// spill 800 bytes, took 1.55 ms per 128^3 FP32 step's sweeps against 1.13.)
+// One tile per block of one shape S, a launch for each shape's range of a tile
+// table.  (One persistent launch over tiles of all shapes, its three bodies in
+// one register allocation with 800 bytes of spills, took 18 ms per axis of 4 096
+// patches against 13, and 1.55 ms for a 128^3 FP32 WENO-Z step's sweeps against
+// 1.13; separately compiled, it also rounded differently.)
 template <class T, int AXIS, int S, bool Z>
 __global__ void __launch_bounds__(kSweepNT, kMinBlocks<T>) sweep_kernel_fixed(const SweepArgs<T> A) {
     constexpr int NC0 = nc_of(shape_ta(AXIS, S));
@@ -562,8 +528,6 @@ constexpr size_t tile_smem(int nc) {
 }
 template <class T, int AXIS, int S>
 constexpr size_t smem_bytes_fixed() { return tile_smem<T>(nc_of(shape_ta(AXIS, S))); }
-template <class T, int AXIS>
-constexpr size_t smem_bytes_persistent() { return tile_smem<T>(max_nc(AXIS)); }
 
 // f(axis, shape, z) over every fixed kernel
 template <class T, int AX, int S, bool Z>
@@ -576,26 +540,8 @@ cudaError_t prepare_axis() {
     cudaError_t e = prepare_fixed<T, AX, 0, Z>();
     if (e == cudaSuccess) e = prepare_fixed<T, AX, 1, Z>();
     if (e == cudaSuccess) e = prepare_fixed<T, AX, 2, Z>();
-    if (e == cudaSuccess)
-        e = cudaFuncSetAttribute(sweep_kernel<T, AX, Z>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                 (int)smem_bytes_persistent<T, AX>());
     return e;
 }
-template <class T, int AX, bool Z>
-int persistent_blocks_per_sm() {
-    int nb = 0;
-    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, sweep_kernel<T, AX, Z>, kSweepNT,
-                                                  smem_bytes_persistent<T, AX>());
-    return nb > 0 ? nb : 1;
-}
-
-// Persistent grid sizes per axis, set by prepare_sweep_kernels (outside any
-// stream capture).
-template <class T>
-struct PersistGrid {
-    static inline int g[3] = {0, 0, 0};
-};
-
 template <class T, bool Z, int S>
 void launch_fixed_shape(int axis, const SweepArgs<T>& a, int ntiles, cudaStream_t s) {
     if (axis == 0) sweep_kernel_fixed<T, 0, S, Z><<<ntiles, kSweepNT, smem_bytes_fixed<T, 0, S>(), s>>>(a);
@@ -613,28 +559,15 @@ void launch_flat(int axis, const SweepArgs<T>& a, int ntiles, cudaStream_t s) {
 }
 
 template <class T, bool Z>
-cudaError_t launch_sweep_w(int axis, const SweepArgs<T>& a, int ntiles, cudaStream_t s) {
-    if (a.split[0] | a.split[1] | a.split[2] | a.split[3]) {
-        // a table sorted by shape: one launch of the fixed kernel per shape
-        SweepArgs<T> b = a;
-        if (a.split[0]) launch_fixed_shape<T, Z, 0>(axis, b, a.split[0], s);
-        b.tiles = a.tiles + a.split[0];
-        if (a.split[1]) launch_fixed_shape<T, Z, 1>(axis, b, a.split[1], s);
-        b.tiles = a.tiles + a.split[0] + a.split[1];
-        if (a.split[2]) launch_fixed_shape<T, Z, 2>(axis, b, a.split[2], s);
-        b.tiles = a.tiles + a.split[0] + a.split[1] + a.split[2];
-        if (a.split[3]) launch_flat<T>(axis, b, a.split[3], s);
-        return cudaGetLastError();
-    }
-    const int grid = PersistGrid<T>::g[axis] > 0 ? PersistGrid<T>::g[axis] : 152;
-    const int nb = ntiles < grid ? ntiles : grid;
-    if (a.queue) {
-        const cudaError_t e = cudaMemsetAsync(a.queue, 0, sizeof(int), s);
-        if (e != cudaSuccess) return e;
-    }
-    if (axis == 0) sweep_kernel<T, 0, Z><<<nb, kSweepNT, smem_bytes_persistent<T, 0>(), s>>>(a, ntiles);
-    else if (axis == 1) sweep_kernel<T, 1, Z><<<nb, kSweepNT, smem_bytes_persistent<T, 1>(), s>>>(a, ntiles);
-    else sweep_kernel<T, 2, Z><<<nb, kSweepNT, smem_bytes_persistent<T, 2>(), s>>>(a, ntiles);
+cudaError_t launch_sweep_w(int axis, const SweepArgs<T>& a, cudaStream_t s) {
+    SweepArgs<T> b = a;
+    if (a.split[0]) launch_fixed_shape<T, Z, 0>(axis, b, a.split[0], s);
+    b.tiles += a.split[0];
+    if (a.split[1]) launch_fixed_shape<T, Z, 1>(axis, b, a.split[1], s);
+    b.tiles += a.split[1];
+    if (a.split[2]) launch_fixed_shape<T, Z, 2>(axis, b, a.split[2], s);
+    b.tiles += a.split[2];
+    if (a.split[3]) launch_flat<T>(axis, b, a.split[3], s);
     return cudaGetLastError();
 }
 
@@ -648,20 +581,12 @@ cudaError_t prepare_sweep_kernels() {
     if (e == cudaSuccess) e = prepare_axis<T, 0, true>();
     if (e == cudaSuccess) e = prepare_axis<T, 1, true>();
     if (e == cudaSuccess) e = prepare_axis<T, 2, true>();
-    if (e != cudaSuccess) return e;
-    int dev = 0, nsm = 0;
-    if ((e = cudaGetDevice(&dev)) != cudaSuccess) return e;
-    if ((e = cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev)) != cudaSuccess) return e;
-    PersistGrid<T>::g[0] = nsm * persistent_blocks_per_sm<T, 0, false>();
-    PersistGrid<T>::g[1] = nsm * persistent_blocks_per_sm<T, 1, false>();
-    PersistGrid<T>::g[2] = nsm * persistent_blocks_per_sm<T, 2, false>();
-    return cudaGetLastError();
+    return e;
 }
 
 template <class T>
-cudaError_t launch_sweep(int axis, const SweepArgs<T>& a, int ntiles, cudaStream_t s) {
-    if (ntiles <= 0) return cudaSuccess;
-    return a.zweights ? launch_sweep_w<T, true>(axis, a, ntiles, s) : launch_sweep_w<T, false>(axis, a, ntiles, s);
+cudaError_t launch_sweep(int axis, const SweepArgs<T>& a, cudaStream_t s) {
+    return a.zweights ? launch_sweep_w<T, true>(axis, a, s) : launch_sweep_w<T, false>(axis, a, s);
 }
 
 }  // namespace wb

@@ -59,10 +59,8 @@ def test_flat_axis_fluxes_and_step(precision, weights, axis, na, nb):
 
 
 def test_flat_patches_among_others_in_every_tile_table():
-    """Patches with and without flat axes in one grid: each ordered tile table
-    gives the bits of the patches run on their own; the unordered one (0) runs
-    another kernel, whose x sweep contracts differently (a flux differs by an
-    ulp or two): the bound of the test above on the state."""
+    """Patches with and without flat axes in one grid: each tile table gives
+    the bits of the patches run on their own."""
     from paper_1808_10633_gb300 import inputs
     from paper_1808_10633_gb300 import wombat as wb
 
@@ -81,8 +79,4 @@ def test_flat_patches_among_others_in_every_tile_table():
             g.set_tiles(c)
             g.set_state(*first)
             g.step(1e-3, 2)
-            got, ref = g.get_state()[0], np.concatenate(alone)
-            if c > 0:
-                assert np.array_equal(got, ref), c
-            else:
-                assert np.abs(got - ref).max() <= 8 * EPS["fp32"] * np.abs(ref).max()
+            assert np.array_equal(g.get_state()[0], np.concatenate(alone)), c
