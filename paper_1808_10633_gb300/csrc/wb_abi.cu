@@ -233,9 +233,9 @@ int enqueue_stages(wb_grid* g, Prof* pf) {
         u.flag = g->d_flag;
         u.dt = g->d_scalars;
         u.ncells = N;
-        u.idx = 1.0 / g->dx;
-        u.idy = 1.0 / g->dy;
-        u.idz = 1.0 / g->dz;
+        u.idx = T(1.0 / g->dx);
+        u.idy = T(1.0 / g->dy);
+        u.idz = T(1.0 / g->dz);
         u.stage = st;
         u.integrator = g->integrator;
         u.emf_mode = g->emf_mode;

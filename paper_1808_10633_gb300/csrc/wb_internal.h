@@ -207,7 +207,8 @@ struct UpdateArgs {
     const int* __restrict__ links; // patch links (see locate) or nullptr
     const double* __restrict__ dt; // device scalar
     long long ncells;
-    double idx, idy, idz;
+    T idx, idy, idz;               // in the grid's precision (a conversion in the kernel
+                                   // would take each warp 64 cycles of the FP64 pipe)
     int stage;                     // SSP-RK3: 0,1,2; RK4: 0..3
     int integrator;
     int emf_mode;

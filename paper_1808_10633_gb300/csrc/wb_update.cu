@@ -155,10 +155,52 @@ __global__ void __launch_bounds__(kCellBlock) emf_kernel(const UpdateArgs<T> A) 
                                 m0 ? Er[2 * N + cim] : T(0), m0 ? Er[2 * N + c] : T(0), A.emf_mode);
 }
 
+// The cells one step back along each axis and each pair of axes.  In a linked
+// patch a neighbour inside the patch is a fixed distance away and only the
+// lanes at its lower faces look links up (six lookups per cell before); a
+// periodic one's wraps are cheaper than the choice.
+template <class T, bool LINKED>
+struct Back {
+    long long x, y, z, yz, xz, xy;
+    __device__ __forceinline__ Back(const Geo<T, LINKED>& G, long long c, int i, int j, int k) {
+        if constexpr (LINKED) {
+            const int nx = G.P.nx, nxy = nx * G.P.ny;
+            x = c - 1; y = c - nx; z = c - nxy;
+            yz = y - nxy; xz = x - nxy; xy = y - 1;
+            if (i == 0) {
+                x = G.at(-1, j, k);
+                xy = G.at(-1, j - 1, k);
+                xz = G.at(-1, j, k - 1);
+            }
+            if (j == 0) {
+                y = G.at(i, -1, k);
+                xy = G.at(i - 1, -1, k);
+                yz = G.at(i, -1, k - 1);
+            }
+            if (k == 0) {
+                z = G.at(i, j, -1);
+                xz = G.at(i - 1, j, -1);
+                yz = G.at(i, j - 1, -1);
+            }
+            x = chk(x, G.N, G.flag); y = chk(y, G.N, G.flag); z = chk(z, G.N, G.flag);
+            yz = chk(yz, G.N, G.flag); xz = chk(xz, G.N, G.flag); xy = chk(xy, G.N, G.flag);
+        } else {
+            x = G.at(i - 1, j, k); y = G.at(i, j - 1, k); z = G.at(i, j, k - 1);
+            yz = G.at(i, j - 1, k - 1); xz = G.at(i - 1, j, k - 1); xy = G.at(i - 1, j - 1, k);
+        }
+    }
+};
+
 // Two cells per thread (t and t + 128 of a 256-cell block), the loads of
 // both issued before the first store; the same arithmetic as emf_kernel.
+// Bound by the latency of its 27 loads per cell: warps in flight count for more
+// than loads per warp.  160^3 in 64 linked bricks, EMFs of a step: 291 us with
+// six lookups per cell (64 registers, 8 blocks per SM), with the fixed distances
+// 215, at 10 / 12 / 16 blocks per SM 210 / 197 / 185 (48 / 40 / 32 registers).
+// 320 periodic patches, 14.7 M cells: 603 us at 8 blocks, 584 at 10 and 12, 654
+// at 14 (32 registers spill its six wraps).
 template <class T, bool LINKED>
-__global__ void __launch_bounds__(kCellBlock / 2) emf_kernel2(const UpdateArgs<T> A) {
+__global__ void __launch_bounds__(kCellBlock / 2, LINKED ? 16 : 10) emf_kernel2(const UpdateArgs<T> A) {
     constexpr int H = kCellBlock / 2;
     const CellBlock cb = A.blocks[blockIdx.x];
     __shared__ LinkTab tab;
@@ -185,15 +227,16 @@ __global__ void __launch_bounds__(kCellBlock / 2) emf_kernel2(const UpdateArgs<T
         const int i = rem - j * G.P.nx;
         c[u] = chk(G.P.off + local, N, A.flag);
         const long long cc = c[u];
-        const long long cim = G.at(i - 1, j, k), cjm = G.at(i, j - 1, k), ckm = G.at(i, j, k - 1);
+        const Back<T, LINKED> B(G, cc, i, j, k);
+        const long long cim = B.x, cjm = B.y, ckm = B.z;
         e[u][0] = edge_emf(-Fy[5 * N + ckm], -Fy[5 * N + cc], Fz[6 * N + cjm], Fz[6 * N + cc],
-                           m0 ? Er[G.at(i, j - 1, k - 1)] : T(0), m0 ? Er[ckm] : T(0),
+                           m0 ? Er[B.yz] : T(0), m0 ? Er[ckm] : T(0),
                            m0 ? Er[cjm] : T(0), m0 ? Er[cc] : T(0), A.emf_mode);
         e[u][1] = edge_emf(Fx[6 * N + ckm], Fx[6 * N + cc], -Fz[5 * N + cim], -Fz[5 * N + cc],
-                           m0 ? Er[N + G.at(i - 1, j, k - 1)] : T(0), m0 ? Er[N + ckm] : T(0),
+                           m0 ? Er[N + B.xz] : T(0), m0 ? Er[N + ckm] : T(0),
                            m0 ? Er[N + cim] : T(0), m0 ? Er[N + cc] : T(0), A.emf_mode);
         e[u][2] = edge_emf(-Fx[5 * N + cjm], -Fx[5 * N + cc], Fy[6 * N + cim], Fy[6 * N + cc],
-                           m0 ? Er[2 * N + G.at(i - 1, j - 1, k)] : T(0), m0 ? Er[2 * N + cjm] : T(0),
+                           m0 ? Er[2 * N + B.xy] : T(0), m0 ? Er[2 * N + cjm] : T(0),
                            m0 ? Er[2 * N + cim] : T(0), m0 ? Er[2 * N + cc] : T(0), A.emf_mode);
     }
 #pragma unroll
@@ -223,7 +266,7 @@ __global__ void __launch_bounds__(kCellBlock, 4) update_kernel(const UpdateArgs<
     const long long cy = G.at(i, j + 1, k);
     const long long cz = G.at(i, j, k + 1);
     const T dt = T(*A.dt);
-    const T idx = T(A.idx), idy = T(A.idy), idz = T(A.idz);
+    const T idx = A.idx, idy = A.idy, idz = A.idz;
     const T* __restrict__ Fx = A.flux;
     const T* __restrict__ Fy = A.flux + 7 * N;
     const T* __restrict__ Fz = A.flux + 14 * N;
@@ -281,7 +324,7 @@ __global__ void __launch_bounds__(kCellBlock / 2, 6) update_kernel2(const Update
         cz[u] = G.at(i, j, k + 1);
     }
     const T dt = T(*A.dt);
-    const T idx = T(A.idx), idy = T(A.idy), idz = T(A.idz);
+    const T idx = A.idx, idy = A.idy, idz = A.idz;
     const T* __restrict__ Fx = A.flux;
     const T* __restrict__ Fy = A.flux + 7 * N;
     const T* __restrict__ Fz = A.flux + 14 * N;
@@ -357,7 +400,7 @@ __global__ void __launch_bounds__(kCellBlock / 2) ct_update_kernel(const UpdateA
     const T* __restrict__ Fy = A.flux + 7 * N;
     const T* __restrict__ Fz = A.flux + 14 * N;
     T Lq[8];
-    const T idx = T(A.idx), idy = T(A.idy), idz = T(A.idz);
+    const T idx = A.idx, idy = A.idy, idz = A.idz;
 #pragma unroll
     for (int q = 0; q < 5; q++) {
         const long long o = q * N;
@@ -555,7 +598,7 @@ __global__ void __launch_bounds__(kCellBlock, 4) update_kernel_vec(const UpdateA
     if (!vrow<V>(cb, P, threadIdx.x, r, A.ncells, A.flag)) return;
     const long long N = A.ncells;
     const T dt = T(*A.dt);
-    const T idx = T(A.idx), idy = T(A.idy), idz = T(A.idz);
+    const T idx = A.idx, idy = A.idy, idz = A.idz;
     const T* __restrict__ Fx = A.flux;
     const T* __restrict__ Fy = A.flux + 7 * N;
     const T* __restrict__ Fz = A.flux + 14 * N;
