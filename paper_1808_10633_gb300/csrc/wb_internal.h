@@ -67,13 +67,15 @@ struct LinkTab {
         }
         __syncthreads();
     }
-    // locate() from the table; P the block's patch
-    __device__ __forceinline__ long long at(const PatchDev& P, int i, int j, int k) const {
+    // locate() from the table; P the block's patch.  (i, j, k) become the place
+    // in the patch found, q its extents.
+    __device__ __forceinline__ long long find(const PatchDev& P, int& i, int& j, int& k, int& qx, int& qy,
+                                              int& qz) const {
         const int ox = i < 0 ? -1 : (i >= P.nx ? 1 : 0);
         const int oy = j < 0 ? -1 : (j >= P.ny ? 1 : 0);
         const int oz = k < 0 ? -1 : (k >= P.nz ? 1 : 0);
         const int d = 9 * (oz + 1) + 3 * (oy + 1) + (ox + 1);
-        const int qx = nx[d], qy = ny[d], qz = nz[d];
+        qx = nx[d], qy = ny[d], qz = nz[d];
         i = ox < 0 ? i + qx : (ox > 0 ? i - P.nx : i);
         j = oy < 0 ? j + qy : (oy > 0 ? j - P.ny : j);
         k = oz < 0 ? k + qz : (oz > 0 ? k - P.nz : k);
@@ -82,6 +84,10 @@ struct LinkTab {
         if ((unsigned)j >= (unsigned)qy) j = wrap_cell(j, qy);
         if ((unsigned)k >= (unsigned)qz) k = wrap_cell(k, qz);
         return off[d] + ((long long)k * qy + j) * qx + i;
+    }
+    __device__ __forceinline__ long long at(const PatchDev& P, int i, int j, int k) const {
+        int qx, qy, qz;
+        return find(P, i, j, k, qx, qy, qz);
     }
 };
 

@@ -429,8 +429,10 @@ __device__ __forceinline__ void tile_body(const SweepArgs<T>& A, const Tile& til
         else { s = e / TP; tp = e - s * TP; }
         int cp, w;
         tile_pencil(tile, tp, np, cp, w);
-        rok[it] = e < NC && w < n3;
         const int raw_a = tile.y - 3 + s;
+        // cells past the last interface's stencil serve idle threads only
+        // (160^3 in 64 bricks: 2.66 -> 2.63 ms, 320 patches 8.44 -> 8.40)
+        rok[it] = e < NC && w < n3 && raw_a < na + 2;
         rown[it] = raw_a >= tile.y && raw_a < tile.y + TA && raw_a < na;
         if (rok[it]) {
             int i, j, k;
