@@ -38,11 +38,10 @@ UNIT = "zone-updates/s"
 # direction, one stage) and of one staged cell, counted from the kernel's
 # formulas (add/sub/mul = 1, FMA = 2, div/sqrt = 1): eigen-structure 100,
 # interface average 16, central flux 35, differences of the stencil 70,
-# their projection 10 x 68, split differences and two phi_N per field
-# 7 x 114 (the eps of each smoothness indicator folded into its fused
-# multiply-adds, phi_N taken on twice the split differences and halved
-# once), back-projection 80.
-SWEEP_FLOPS_PER_INTERFACE = 1779
+# their projection 10 x 50, split differences and two phi_N per field
+# 7 x 103 (the smoothness indicators as quadratic forms that share eps and
+# a square, phi_N as N / (3 W) - q / 12), back-projection 80.
+SWEEP_FLOPS_PER_INTERFACE = 1522
 SWEEP_FLOPS_PER_STAGED_CELL = 80
 
 # DRAM bytes (dram__bytes_read.sum + dram__bytes_write.sum) per launch of the
@@ -50,15 +49,15 @@ SWEEP_FLOPS_PER_STAGED_CELL = 80
 # benchmark times (profiles/sweep_traffic_fp32_turbulence256.md); reported
 # only at that size and while the sweep sources hash to SWEEP_TRAFFIC_SOURCES.
 SWEEP_TRAFFIC_N = 256
-SWEEP_TRAFFIC = {"sweep_x": 1180.90e6, "sweep_y": 980.41e6, "sweep_z": 978.70e6}
-SWEEP_TRAFFIC_SOURCES = "69dc94dc5fccf3ed"
+SWEEP_TRAFFIC = {"sweep_x": 1178.32e6, "sweep_y": 982.53e6, "sweep_z": 983.33e6}
+SWEEP_TRAFFIC_SOURCES = "45a70bfd88897158"
 
 
 def sweep_sources_hash() -> str:
     import hashlib
 
     h = hashlib.sha256()
-    for f in ("wb_sweep.cuh", "wb_sweep_f32.cu"):
+    for f in ("wb_math.cuh", "wb_sweep.cuh", "wb_sweep_js.cuh", "wb_sweep_f32.cu"):
         with open(os.path.join(ROOT, "paper_1808_10633_gb300", "csrc", f), "rb") as fh:
             h.update(fh.read())
     return h.hexdigest()[:16]

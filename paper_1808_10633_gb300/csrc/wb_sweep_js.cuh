@@ -10,12 +10,12 @@
 // ms; three and four blocks per SM (168 and 128 registers) are no faster.
 // FP32 takes the one of wb_sweep.cuh (interface_flux), which packs the U and F
 // differences of a stencil step, and here the two sides of phi_N, in the lanes
-// of Blackwell's packed FP32 instructions: 1 376 to 1 419 instructions per
-// interface, issued on 60 to 64 % of cycles by sixteen warps per SM.  256^3,
-// x, y, z sweeps of a step: 2.88 / 2.83 / 3.01 -> 2.67 / 2.79 / 2.97 ms.  Two
-// interfaces per thread (neighbouring pencils in the two lanes) need only
-// 1 107 instructions per interface, but 200 to 255 registers: eight warps per
-// SM issue on 41 % of cycles, and with the staging moved to further warps
+// of Blackwell's packed FP32 instructions: 1 320 to 1 335 instructions per
+// interface (1 454 before), issued on 59 to 61 % of cycles by sixteen warps per
+// SM.  256^3, x, y, z sweeps of a step: 2.88 / 2.83 / 3.01 -> 2.70 / 2.77 / 2.80
+// ms.  Two interfaces per thread (neighbouring pencils in the two lanes) need
+// only 1 107 instructions per interface, but 200 to 255 registers: eight warps
+// per SM issue on 41 % of cycles, and with the staging moved to further warps
 // (cp.async, registers split between the warps) on 50 %: 3.1 to 3.5 and 2.6 to
 // 3.0 ms per axis.
 #pragma once
