@@ -3,8 +3,8 @@
 //
 // One interface per thread.  FP64 takes the interface arithmetic below
 // (sweep_flux), which counts operations of the FP64 pipe (two per clock and SM
-// on this GPU, 87 % busy, everything else hidden behind it): quadratic-form
-// smoothness indicators and one reciprocal for the two phi_N of a field (60
+// on this GPU, 87 % busy, everything else hidden behind it): smoothness
+// indicators of ten operations and one reciprocal for the two phi_N of a field (60
 // instead of 83 operations), three-operation reciprocals, Alfven rows that act
 // on the differences directly.  96^3, x + y + z sweep of a step: 21.3 -> 17.6
 // ms; three and four blocks per SM (168 and 128 registers) are no faster.
@@ -39,19 +39,25 @@ constexpr int kSlotsV = kNBackV + 24;
 template <class T> constexpr int kSlots = sizeof(T) == 4 ? thread_slots(4) : kSlotsV;
 
 // ---- phi_N (Sec. 2.1) ------------------------------------------------------------
-// With a, b, c, d four successive differences, IS_k as printed are quadratic
-// forms: IS_0 / 16 = a (a - 11/4 b) + 5/2 b^2, IS_1 / 16 = b (b - 5/4 c) + c^2,
-// IS_2 / 16 = d (d - 11/4 c) + 5/2 c^2 (smallest eigenvalues 0.18, 0.38,
-// 0.18: no cancellation to speak of).  The weights depend on the ratios of
-// the eps + IS_k only, so e_k = (eps + IS_k) / 16, ten operations, serve.
+// With a, b, c, d four successive differences, the IS_k as printed are quadratic
+// forms; completed squares keep them sums of non-negative terms,
+//   IS_0 / 16 = (a - 11/8 b)^2 + 39/64 b^2, IS_1 / 16 = (b - 5/8 c)^2 + 39/64 c^2,
+//   IS_2 / 16 = (d - 11/8 c)^2 + 39/64 c^2,
+// each good to three roundings.  The weights depend on the ratios of the
+// eps + IS_k only, so e_k = (eps + IS_k) / 16, ten operations, serve.  (The forms
+// multiplied out, a (a - 11/4 b) + 5/2 b^2 and so on, also take ten, but lose
+// four bits where a = 11/8 b, and round IS_0 and IS_2 of a symmetric stencil
+// differently: WENO-Z divides their difference, then a rounding error, by the
+// smallest eps + IS_k.)
 template <class V>
 __device__ __forceinline__ void smoothness(V a, V b, V c, V d, typename Lanes<V>::S eps16, V& e0, V& e1, V& e2) {
     using S = typename Lanes<V>::S;
-    const V eps = splat<V>(eps16), k11 = splat<V>(S(-2.75)), k5 = splat<V>(S(-1.25)), k52 = splat<V>(S(2.5));
-    e0 = vfma(a, vfma(b, k11, a), vfma(vmul(b, k52), b, eps));
-    const V cc = vfma(c, c, eps);
-    e1 = vfma(b, vfma(c, k5, b), cc);
-    e2 = vfma(d, vfma(c, k11, d), vfma(cc, k52, splat<V>(S(-1.5) * eps16)));
+    const V eps = splat<V>(eps16), k39 = splat<V>(S(39.0 / 64.0)), k11 = splat<V>(S(-1.375)), k5 = splat<V>(S(-0.625));
+    const V sb = vfma(vmul(b, k39), b, eps), sc = vfma(vmul(c, k39), c, eps);
+    const V t0 = vfma(b, k11, a), t1 = vfma(c, k5, b), t2 = vfma(c, k11, d);
+    e0 = vfma(t0, t0, sb);
+    e1 = vfma(t1, t1, sc);
+    e2 = vfma(t2, t2, sc);
 }
 
 // p = a - 2b + c
