@@ -68,11 +68,16 @@ __device__ __forceinline__ double vfma(double a, double b, double c) { return fm
 __device__ __forceinline__ double vmul(double a, double b) { return a * b; }
 __device__ __forceinline__ double vadd(double a, double b) { return a + b; }
 __device__ __forceinline__ double vsub(double a, double b) { return a - b; }
+__device__ __forceinline__ double vfms(double a, double b, double c) { return fma(a, b, -c); }
+__device__ __forceinline__ double vrcp(double a) { return recip(a); }
 __device__ __forceinline__ double vneg(double a) { return -a; }
 __device__ __forceinline__ float2 vfma(float2 a, float2 b, float2 c) { return __ffma2_rn(a, b, c); }
 __device__ __forceinline__ float2 vmul(float2 a, float2 b) { return __fmul2_rn(a, b); }
 __device__ __forceinline__ float2 vadd(float2 a, float2 b) { return __fadd2_rn(a, b); }
 __device__ __forceinline__ float2 vsub(float2 a, float2 b) { return __ffma2_rn(b, make_float2(-1.f, -1.f), a); }
+__device__ __forceinline__ float2 vfms(float2 a, float2 b, float2 c) {      // a b - c
+    return make_float2(fmaf(a.x, b.x, -c.x), fmaf(a.y, b.y, -c.y));
+}
 __device__ __forceinline__ float2 vneg(float2 a) { return make_float2(-a.x, -a.y); }
 __device__ __forceinline__ float2 vrcp(float2 a) { return make_float2(recip(a.x), recip(a.y)); }
 __device__ __forceinline__ double vabs(double a) { return fabs(a); }

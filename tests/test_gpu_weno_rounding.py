@@ -144,3 +144,23 @@ def test_weno_z_on_symmetric_stencils(lib, dtype, size):
     err = np.abs(z.astype(np.longdouble) - (_phi(x[:4], "z") - _phi(x[4:], "z")))
     m = np.abs(x).max(axis=0)
     assert float((err / m).max()) <= 16 * U[dtype], float((err / m).max()) / U[dtype]
+
+
+@pytest.mark.parametrize("weights", ["js", "z"])
+@pytest.mark.parametrize("dtype", [np.float32, np.float64])
+def test_corrections_at_a_jump(lib, dtype, weights):
+    """A jump J seen by both sides where neither takes it into its stencil: each side
+    is J / 12 with all but saturated weights and the correction their small difference.  Four
+    roundings a side (the numerator's two, the quotient's two) at u / sqrt(3) each are
+    1.25 u J rms at most, two sides, over 24 for the halved differences."""
+    rng = np.random.default_rng(6)
+    j = 10.0 ** rng.uniform(1.5, 3, N)
+    x = np.zeros((8, N))
+    x[1] = -j * (1 + 1e-3 * rng.standard_normal(N))     # minus side: b
+    x[7] = j                                            # plus side: d
+    x = x.astype(dtype)
+    got = _run(lib, x, weights)[1]
+    want = _phi(x[:4], weights) - _phi(x[4:], weights)
+    err = (got.astype(np.longdouble) - want) / np.abs(x[7])
+    rms = float(np.sqrt((err ** 2).mean()))
+    assert rms <= 2 ** 0.5 * 1.25 / 24 * U[dtype], rms / U[dtype]
