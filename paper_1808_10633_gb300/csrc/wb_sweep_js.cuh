@@ -376,7 +376,7 @@ __device__ __forceinline__ void sweep_flux(const typename Lanes<V>::S* __restric
     for (int f = 0; f < 7; f++) {
         const S* F = cell + at_f<S>(f, nc, 0);
         const V in = vadd(ld<V>(F + 2 * CS), ld<V>(F + 3 * CS)), ex = vadd(ld<V>(F + CS), ld<V>(F + 4 * CS));
-        out[f] = vfma(in, splat<V>(S(7.0 / 12.0)), vfma(ex, splat<V>(S(-1.0 / 12.0)), dF[f]));
+        out[f] = vfma(vfms(in, splat<V>(S(7)), ex), splat<V>(S(1.0 / 12.0)), dF[f]);
     }
 }
 
@@ -489,8 +489,7 @@ __device__ __forceinline__ void flat_body(const SweepArgs<T>& A, const Tile& til
 #pragma unroll
     for (int f = 0; f < 7; f++) {
         const T f1 = sm[at_f<T>(f, kSweepNT, tid)], f2 = f1 + f1;
-        if constexpr (sizeof(T) == 8) F[f] = fma(f2, 7.0 / 12.0, f2 * (-1.0 / 12.0));
-        else F[f] = (T(7) * f2 - f2) * T(1.0 / 12.0);
+        F[f] = (T(7) * f2 - f2) * T(1.0 / 12.0);
     }
     store_flux<T, AXIS>(A, c, F);
 }

@@ -164,3 +164,28 @@ def test_corrections_at_a_jump(lib, dtype, weights):
     err = (got.astype(np.longdouble) - want) / np.abs(x[7])
     rms = float(np.sqrt((err ** 2).mean()))
     assert rms <= 2 ** 0.5 * 1.25 / 24 * U[dtype], rms / U[dtype]
+
+
+@pytest.mark.parametrize("precision,dtype", [("fp32", np.float32), ("fp64", np.float64)])
+@pytest.mark.parametrize("dims", [(2, 3, 2), (2, 3, 1)])
+def test_central_flux_of_uniform_states(precision, dtype, dims):
+    """The mass flux of a uniform state is its momentum: the central combination
+    (7 (F + F) - (F + F)) / 12 is off by the constant's half u, and no bias else."""
+    from paper_1808_10633_gb300 import inputs
+    from paper_1808_10633_gb300 import wombat as wb
+
+    rng = np.random.default_rng(7)
+    sts, m = [], []
+    for _ in range(400):
+        st = inputs.uniform(*dims)
+        mom = np.exp2(rng.uniform(-2, 0, 3)).astype(dtype).astype(np.float64)
+        st.U[0] = 1.0
+        st.U[1:4] = mom[:, None, None, None]
+        st.U[7] = 10.0
+        sts.append(st)
+        m.append(mom)
+    n, m = dims[0] * dims[1] * dims[2], np.array(m)
+    with wb.Grid.from_patches(sts, precision=precision) as g:
+        F = [g.face_fluxes(a).reshape(400, 7, n)[:, 0, 0] for a in range(3)]      # patch by patch
+    err = np.concatenate([(F[a] - m[:, a]) / m[:, a] for a in range(3)]) / U[dtype]
+    assert np.abs(err).max() <= 2.5 and abs(err.mean()) <= 0.6, (err.min(), err.max(), err.mean())
