@@ -55,6 +55,32 @@ __device__ __forceinline__ float recip(float x) { return 1.0f / x; }
 __device__ __forceinline__ float rsq_root(float x) { return rsqrtf(x); }
 __device__ __forceinline__ float sq_root(float x) { return sqrtf(x); }
 
+// The FP64 value of an FP32 number, formed from its bits with integer
+// operations (IEEE 754 binary32 -> binary64 is exact: sign kept, exponent
+// rebiased by 1023 - 127, mantissa widened by 29 zero bits; subnormals
+// normalised, zero, infinities and NaN mapped to their binary64 forms).  The
+// conversion instruction would run on the FP64 pipe, which is narrow on this
+// GPU; with this only the sums do.
+__device__ __forceinline__ double widen(float x) {
+    const unsigned int u = __float_as_uint(x);
+    const unsigned long long sign = (unsigned long long)(u >> 31) << 63;
+    const unsigned int e = (u >> 23) & 0xffu;
+    unsigned int m = u & 0x7fffffu;
+    unsigned long long bits;
+    if (e == 0xffu) {                       // infinity or NaN
+        bits = sign | (0x7ffull << 52) | ((unsigned long long)m << 29);
+    } else if (e != 0u) {                   // normal
+        bits = sign | ((unsigned long long)(e + 896u) << 52) | ((unsigned long long)m << 29);
+    } else if (m == 0u) {                   // signed zero
+        bits = sign;
+    } else {                                // subnormal: value m 2^-149
+        const int sh = __clz(m) - 8;        // shifts that bring the top bit to bit 23
+        m = (m << sh) & 0x7fffffu;
+        bits = sign | ((unsigned long long)(897 - sh) << 52) | ((unsigned long long)m << 29);
+    }
+    return __longlong_as_double((long long)bits);
+}
+
 // ---- one FP64 value or two FP32 lanes -------------------------------------------
 template <class V> struct Lanes;
 template <> struct Lanes<double> { using S = double; static constexpr int N = 1; };

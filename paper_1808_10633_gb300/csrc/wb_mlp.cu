@@ -15,12 +15,13 @@
 //                    entries, record by record in a fixed order;
 //   apply_kernel     one thread per entry: the blocks' sums in a fixed order,
 //                    the mean, and the Adam step of its parameter.
-// Every sum over records is exact to twice the FP32 mantissa (see add_prod),
-// so the gradient is bitwise repeatable and rounds once, at the end.
+// Every sum over records has at least the bits and the range of an FP64 one, in
+// a fixed order, so the gradient is bitwise repeatable.
 // Minibatch indices come from a counter-based generator (splitmix64 of seed,
 // step, field, slot), so a run is reproducible.
 #include "../../include/wombat_gb300.h"
 #include "wb_internal.h"
+#include "wb_math.cuh"
 
 #include <algorithm>
 #include <vector>
@@ -75,24 +76,39 @@ __device__ __forceinline__ long long pick(const long long* off, const long long*
     return off[f] + (long long)(h % (unsigned long long)cnt[f]);
 }
 
-// Two entries' sums at once, in the lanes of the packed FP32 instructions: each
-// an unevaluated pair hi + lo, += a b (nb = -b).  The product and the sum are
-// both split into their rounded value and its exact error (Dekker's and Knuth's
-// error-free transformations), the errors collecting in lo.  The sum keeps 48
-// bits for 10 FP32 operations; an FP64 accumulator would cost a fused
-// multiply-add and two conversions on a pipe 64 times narrower.
-struct Sum2 {
-    float2 hi = {0.f, 0.f}, lo = {0.f, 0.f};
+// Two entries' sums over one chunk, in the lanes of the packed FP32 instructions:
+// each an unevaluated hi + mid + lo, += a b (nb = -b).  The product and every sum
+// but lo's are split into their rounded value and its exact error (Dekker's and
+// Knuth's error-free transformations), so a chunk's sum is good to 2^-72 of its
+// magnitudes (errors of products below 2^-102 vanish: under half of the least
+// FP32 number in a mean).  22 FP32 operations for two entries, 5.7 ms in
+// the case below; FP64 fused multiply-adds on their 64 times narrower pipe take
+// 8.5, and a pair hi + lo of ten operations takes 4.2 but loses four of
+// FP64's bits.
+struct Sum3 {
+    float2 hi = {0.f, 0.f}, mid = {0.f, 0.f}, lo = {0.f, 0.f};
+    static __device__ __forceinline__ float2 minus(float2 a, float2 b) {          // a - b
+        return __ffma2_rn(b, make_float2(-1.f, -1.f), a);
+    }
+    // s += x, returns the rounding error
+    static __device__ __forceinline__ float2 add_exact(float2& s, float2 x) {
+        const float2 t = __fadd2_rn(s, x), z = minus(t, s), back = minus(s, minus(t, z));
+        s = t;
+        return __fadd2_rn(back, minus(x, z));
+    }
     __device__ __forceinline__ void add(float2 a, float2 b, float2 nb) {
-        const float2 m1 = make_float2(-1.f, -1.f);
         const float2 n = __fmul2_rn(a, nb), e = __ffma2_rn(a, b, n);              // -p, a b - p
-        const float2 t = __ffma2_rn(n, m1, hi), z = __ffma2_rn(hi, m1, t);        // hi + p
-        const float2 back = __ffma2_rn(__ffma2_rn(z, m1, t), m1, hi);             // hi - (t - z)
-        const float2 err = __ffma2_rn(__fadd2_rn(n, z), m1, back);                // + (p - z)
+        const float2 t = minus(hi, n), z = minus(t, hi), back = minus(hi, minus(t, z));
+        const float2 err = minus(back, __fadd2_rn(n, z));                         // + (p - z)
         hi = t;
-        lo = __fadd2_rn(lo, __fadd2_rn(err, e));
+        const float2 r = add_exact(mid, err);
+        lo = __fadd2_rn(lo, __fadd2_rn(r, add_exact(mid, e)));
     }
 };
+// A lane of a chunk's sum in FP64; NaN where it left the FP32 range.
+__device__ __forceinline__ double joined(float hi, float mid, float lo) {
+    return wb::widen(hi) + (wb::widen(mid) + wb::widen(lo));
+}
 
 // The two factors of gradient entry j in a record's row.
 __device__ __forceinline__ void entry_factors(int j, int& ga, int& gb) {
@@ -112,15 +128,14 @@ __device__ __forceinline__ void entry_factors(int j, int& ga, int& gb) {
 // padded so that rows and columns of W2 are both read without bank
 // conflicts); then the block adds the chunk's outer products, a 2 x 2 tile of
 // dW2 per thread and the 356 other entries one or two per thread.  Bound by
-// the FP32 pipe: 10 of the 13 operations per entry and record are the exact
-// sums.  60 steps of 4 096 records per field and one full-batch gradient, host
-// side included: 83.5 -> 4.2 ms (33 us per step here, 7 in apply_kernel) against
-// a serial loop over the records per
-// entry with FP64 accumulators (and a loss copied to the host every step).
+// the FP32 pipe: the exact sums are 22 of the 25 operations per two entries and
+// record.  60 steps of 4 096 records per field and one full-batch gradient, host
+// side included: 83.5 -> 5.7 ms against a serial loop over the records per entry
+// with FP64 accumulators (and a loss copied to the host every step).
 __global__ void __launch_bounds__(kGradThreads, 2)
 grad_kernel(const float* __restrict__ rec, const long long* __restrict__ perm, const long long* __restrict__ off,
             const long long* __restrict__ cnt, const float* __restrict__ params, int batch, int full,
-            unsigned long long seed, long long step, float lam, float2* __restrict__ part) {
+            unsigned long long seed, long long step, float lam, double* __restrict__ part) {
     __shared__ __align__(16) float row[kChunk][SROW];
     __shared__ __align__(16) float W1[NIN][NH], W2[NH][NH + 1], W3[NOUT][NH];
     __shared__ float B1[NH], B2[NH], B3[NOUT + 1];
@@ -149,7 +164,7 @@ grad_kernel(const float* __restrict__ rec, const long long* __restrict__ perm, c
     int ga0, gb0, ga1, gb1;
     entry_factors(e0, ga0, gb0);
     entry_factors(two ? e1 : e0, ga1, gb1);
-    Sum2 top, bot, rest;           // the tile's two rows, and e0 with e1
+    double acc[6] = {0, 0, 0, 0, 0, 0};    // the chunks' sums: the tile by rows, e0, e1
     __syncthreads();
     for (long long c = (long long)g * kChunk; c < n; c += (long long)kGradBlocks * kChunk) {
         // forward and backward, four records per warp, lane = hidden unit
@@ -277,6 +292,7 @@ grad_kernel(const float* __restrict__ rec, const long long* __restrict__ perm, c
         }
         __syncthreads();
         const int m = n - c < kChunk ? (int)(n - c) : kChunk;
+        Sum3 top, bot, rest;       // the tile's two rows, and e0 with e1
 #pragma unroll 2
         for (int q = 0; q < m; q++) {
             const float* w = row[q];
@@ -288,42 +304,46 @@ grad_kernel(const float* __restrict__ rec, const long long* __restrict__ perm, c
             const float2 f = make_float2(w[gb0], w[gb1]);
             rest.add(make_float2(w[ga0], w[ga1]), f, make_float2(-f.x, -f.y));
         }
+        double sum[6] = {joined(top.hi.x, top.mid.x, top.lo.x),    joined(top.hi.y, top.mid.y, top.lo.y),
+                         joined(bot.hi.x, bot.mid.x, bot.lo.x),    joined(bot.hi.y, bot.mid.y, bot.lo.y),
+                         joined(rest.hi.x, rest.mid.x, rest.lo.x), joined(rest.hi.y, rest.mid.y, rest.lo.y)};
+#pragma unroll
+        for (int k = 0; k < 6; k++) {
+            if (!isfinite(sum[k])) {                   // out of the FP32 range, infinite or NaN
+                const int ga = k < 4 ? S_DA2 + 2 * ti + (k >> 1) : (k == 4 ? ga0 : ga1);
+                const int gb = k < 4 ? S_H1 + 2 * tk + (k & 1) : (k == 4 ? gb0 : gb1);
+                sum[k] = 0.0;
+                for (int q = 0; q < m; q++) sum[k] = fma(double(row[q][ga]), double(row[q][gb]), sum[k]);
+            }
+            acc[k] += sum[k];
+        }
         __syncthreads();
     }
-    float2* o = part + (long long)blockIdx.x * NE;
+    double* o = part + (long long)blockIdx.x * NE;
     const int j = O_W2 + 2 * ti * NH + 2 * tk;
-    o[j] = make_float2(top.hi.x, top.lo.x);
-    o[j + 1] = make_float2(top.hi.y, top.lo.y);
-    o[j + NH] = make_float2(bot.hi.x, bot.lo.x);
-    o[j + NH + 1] = make_float2(bot.hi.y, bot.lo.y);
-    o[e0] = make_float2(rest.hi.x, rest.lo.x);
-    if (two) o[e1] = make_float2(rest.hi.y, rest.lo.y);
+    o[j] = acc[0];
+    o[j + 1] = acc[1];
+    o[j + NH] = acc[2];
+    o[j + NH + 1] = acc[3];
+    o[e0] = acc[4];
+    if (two) o[e1] = acc[5];
 }
 
 // Gradient entry j of field f: the blocks' sums added in FP64 in the order of
 // the blocks, over the number of records; entry NP is the loss.  With m given
 // also the parameter's Adam step.
 __global__ void __launch_bounds__(64)
-apply_kernel(const float2* __restrict__ part, const long long* __restrict__ cnt, int batch, int full,
+apply_kernel(const double* __restrict__ part, const long long* __restrict__ cnt, int batch, int full,
              float* __restrict__ grad, float* __restrict__ loss, float* __restrict__ params, float* __restrict__ m,
              float* __restrict__ v, float lr, float b1, float b2, float eps, float c1, float c2) {
     const int gid = blockIdx.x * blockDim.x + threadIdx.x;
     const int f = gid / NE, j = gid - f * NE;
     if (f >= NF) return;
     const long long n = cnt[f] == 0 ? 0 : (full ? cnt[f] : (long long)batch);
-    const float2* s = part + (long long)f * kGradBlocks * NE + j;
-    // the same pair sums as in the blocks (FP64 additions would run on the
-    // narrow pipe: 13 us instead of 7)
-    float hi = 0.f, lo = 0.f;
+    const double* s = part + (long long)f * kGradBlocks * NE + j;
+    double sum = 0.0;
 #pragma unroll
-    for (int b = 0; b < kGradBlocks; b++) {
-        const float2 a = s[(long long)b * NE];
-        const float t = __fadd_rn(hi, a.x), z = __fsub_rn(t, hi);
-        lo = __fadd_rn(lo, __fadd_rn(a.y, __fadd_rn(__fsub_rn(hi, __fsub_rn(t, z)), __fsub_rn(a.x, z))));
-        hi = t;
-    }
-    // an infinite sum leaves NaN in the errors: it stands by itself
-    const double sum = isfinite(hi) ? double(hi) + double(lo) : double(hi);
+    for (int b = 0; b < kGradBlocks; b++) sum += s[(long long)b * NE];
     const float g = float(n > 0 ? sum / double(n) : 0.0);
     if (j == NP) {
         loss[f] = g;
@@ -350,7 +370,7 @@ struct Dev {
     float* grad = nullptr;
     float* m = nullptr;            // Adam's moments, m then v
     float* v = nullptr;
-    float2* part = nullptr;        // the blocks' sums
+    double* part = nullptr;        // the blocks' sums
     float* loss = nullptr;         // 7 per step
     ~Dev() {
         if (all) cudaFree(all);
@@ -387,7 +407,7 @@ int setup(Dev& D, const float* records, long long n, const float* params, long l
     const size_t np = sizeof(float) * NF * NP;
     const size_t rec = place(sizeof(float) * n * REC), prm = place(sizeof(long long) * perm.size()),
                  tab = place(sizeof(long long) * 2 * NF), par = place(np), grd = place(np), mom = place(2 * np),
-                 prt = place(sizeof(float2) * NE * NF * kGradBlocks),
+                 prt = place(sizeof(double) * NE * NF * kGradBlocks),
                  los = place(sizeof(float) * NF * std::max<long long>(steps, 1));
     if (cudaMalloc(&D.all, used) != cudaSuccess) {
         cudaGetLastError();
@@ -401,7 +421,7 @@ int setup(Dev& D, const float* records, long long n, const float* params, long l
     D.grad = reinterpret_cast<float*>(D.all + grd);
     D.m = reinterpret_cast<float*>(D.all + mom);
     D.v = D.m + NF * NP;
-    D.part = reinterpret_cast<float2*>(D.all + prt);
+    D.part = reinterpret_cast<double*>(D.all + prt);
     D.loss = reinterpret_cast<float*>(D.all + los);
     long long table[2 * NF];
     for (int f = 0; f < NF; f++) {

@@ -2,6 +2,7 @@
 // deterministic FP64 conserved totals, and the FP64 <-> state conversions
 // used at the ABI.
 #include "wb_internal.h"
+#include "wb_math.cuh"
 
 #include <cfloat>
 #include <limits>
@@ -169,32 +170,6 @@ cfl_kernel_vec(const T* __restrict__ q, const CellBlock* __restrict__ vblocks, i
         }
     }
     block_max_out<T>(s, smax_bits);
-}
-
-// The FP64 value of an FP32 number, formed from its bits with integer
-// operations (IEEE 754 binary32 -> binary64 is exact: sign kept, exponent
-// rebiased by 1023 - 127, mantissa widened by 29 zero bits; subnormals
-// normalised, zero, infinities and NaN mapped to their binary64 forms).  The
-// conversion instruction would run on the FP64 pipe, which is narrow on this
-// GPU; here only the sums do.
-__device__ __forceinline__ double widen(float x) {
-    const unsigned int u = __float_as_uint(x);
-    const unsigned long long sign = (unsigned long long)(u >> 31) << 63;
-    const unsigned int e = (u >> 23) & 0xffu;
-    unsigned int m = u & 0x7fffffu;
-    unsigned long long bits;
-    if (e == 0xffu) {                       // infinity or NaN
-        bits = sign | (0x7ffull << 52) | ((unsigned long long)m << 29);
-    } else if (e != 0u) {                   // normal
-        bits = sign | ((unsigned long long)(e + 896u) << 52) | ((unsigned long long)m << 29);
-    } else if (m == 0u) {                   // signed zero
-        bits = sign;
-    } else {                                // subnormal: value m 2^-149
-        const int sh = __clz(m) - 8;        // shifts that bring the top bit to bit 23
-        m = (m << sh) & 0x7fffffu;
-        bits = sign | ((unsigned long long)(897 - sh) << 52) | ((unsigned long long)m << 29);
-    }
-    return __longlong_as_double((long long)bits);
 }
 
 // s + e = a + b exactly, s rounded (Knuth's two-sum); e is NaN where s overflows.
