@@ -358,7 +358,7 @@ totals_pass1(const T* __restrict__ q, long long N, long long chunk, double* __re
 #pragma unroll
         for (int f = 0; f < 8; f++) {
             if (fabsf(s[f]) <= 3.4e38f && fabsf(eh[f]) <= 3.4e38f) {
-                acc[f] = widen(s[f]) + widen(eh[f] + el[f]);
+                acc[f] = widen(s[f]) + (widen(eh[f]) + widen(el[f]));
             } else {                           // out of the FP32 range, infinite or NaN
                 for (long long c = beg + threadIdx.x; c < end; c += 256) acc[f] += widen(q[f * N + c]);
             }
