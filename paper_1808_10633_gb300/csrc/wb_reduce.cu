@@ -186,7 +186,8 @@ __device__ __forceinline__ double face_div(double xp, double x, double yp, doubl
 }
 // FP32 faces: an upper bound of its magnitude, and whether that is below
 // `least`, from pairs of FP32 values (differences exact, products and sums to
-// 2^-42 of the terms' magnitudes; ih + il = 1 / dx to 2^-48).
+// 2^-42 of the terms' magnitudes; ih + il = 1 / dx to 2^-48, for 1 / dx from
+// 1e-30 on).
 __device__ __forceinline__ bool face_div_below(float xp, float x, float yp, float y, float zp, float z, float2 ix,
                                                float2 iy, float2 iz, float least) {
     float hi = 0.f, lo = 0.f, mag = 0.f;
@@ -227,6 +228,8 @@ divb_kernel(const T* __restrict__ q, const CellBlock* __restrict__ blocks, int n
     float least = 0.f;
     auto pair = [](double v) { const float h = float(v); return make_float2(h, float(v - double(h))); };
     const float2 ix = pair(idx), iy = pair(idy), iz = pair(idz);
+    // below 1e-30 the pairs lose bits to the subnormal numbers
+    const bool pairs = sizeof(T) == 4 && fminf(ix.x, fminf(iy.x, iz.x)) >= 1e-30f;
     for (int b = blockIdx.x; b < nblocks; b += gridDim.x) {
         const CellBlock cb = blocks[b];
         const PatchDev P = patches[cb.x];
@@ -249,7 +252,7 @@ divb_kernel(const T* __restrict__ q, const CellBlock* __restrict__ blocks, int n
         }
         bool need = in;
         if constexpr (sizeof(T) == 4) {
-            need = in && !face_div_below(xp, bx, yp, by, zp, bz, ix, iy, iz, least);
+            need = in && !(pairs && face_div_below(xp, bx, yp, by, zp, bz, ix, iy, iz, least));
             if (!__any_sync(0xffffffffu, need)) continue;
         }
         if (need) {
