@@ -395,10 +395,10 @@ int upload(wb_grid* g, const double* U, const double* b) {
     if (mapped(g, U) && mapped(g, b)) {      // the import kernel reads the host arrays in place
         if (g->precision == WB_FP64)
             WB_CK((wb::launch_import<double, double>(U, b, static_cast<double*>(g->un), g->d_blocks,
-                                                     g->d_patches, N, g->nblocks, g->stream)));
+                                                     g->d_patches, N, g->nblocks, true, g->stream)));
         else
             WB_CK((wb::launch_import<float, double>(U, b, static_cast<float*>(g->un), g->d_blocks,
-                                                    g->d_patches, N, g->nblocks, g->stream)));
+                                                    g->d_patches, N, g->nblocks, true, g->stream)));
         return WB_OK;
     }
     WB_CK(cudaMemcpyAsync(g->d_io, U, sizeof(double) * 8 * N, cudaMemcpyHostToDevice, g->stream));
@@ -406,10 +406,10 @@ int upload(wb_grid* g, const double* U, const double* b) {
                           g->stream));
     if (g->precision == WB_FP64)
         WB_CK((wb::launch_import<double, double>(g->d_io, g->d_io + 8 * N, static_cast<double*>(g->un),
-                                        g->d_blocks, g->d_patches, N, g->nblocks, g->stream)));
+                                        g->d_blocks, g->d_patches, N, g->nblocks, false, g->stream)));
     else
         WB_CK((wb::launch_import<float, double>(g->d_io, g->d_io + 8 * N, static_cast<float*>(g->un),
-                                       g->d_blocks, g->d_patches, N, g->nblocks, g->stream)));
+                                       g->d_blocks, g->d_patches, N, g->nblocks, false, g->stream)));
     return WB_OK;
 }
 
@@ -969,14 +969,14 @@ int wb_set_state_f32(wb_grid* g, const float* U, const float* b) {
     const long long N = g->N;
     if (mapped(g, U) && mapped(g, b)) {      // the import kernel reads the host arrays in place
         WB_CK((wb::launch_import<float, float>(U, b, static_cast<float*>(g->un), g->d_blocks,
-                                              g->d_patches, N, g->nblocks, g->stream)));
+                                              g->d_patches, N, g->nblocks, true, g->stream)));
         return WB_OK;
     }
     float* io = reinterpret_cast<float*>(g->d_io);
     WB_CK(cudaMemcpyAsync(io, U, sizeof(float) * 8 * N, cudaMemcpyHostToDevice, g->stream));
     WB_CK(cudaMemcpyAsync(io + 8 * N, b, sizeof(float) * 3 * N, cudaMemcpyHostToDevice, g->stream));
     WB_CK((wb::launch_import<float, float>(io, io + 8 * N, static_cast<float*>(g->un), g->d_blocks,
-                                          g->d_patches, N, g->nblocks, g->stream)));
+                                          g->d_patches, N, g->nblocks, false, g->stream)));
     return WB_OK;
 }
 
@@ -989,14 +989,14 @@ int wb_get_state_f32(wb_grid* g, float* U_out, float* b_out) {
     if ((!U_out || mapped(g, U_out)) && (!b_out || mapped(g, b_out))) {
         // the export kernel writes the host arrays in place
         WB_CK((wb::launch_export<float, float>(static_cast<const float*>(g->un), U_out, b_out, g->d_blocks,
-                                              g->d_patches, g->d_links, N, g->nblocks, g->stream)));
+                                              g->d_patches, g->d_links, N, g->nblocks, true, g->stream)));
         return check_flag(g);
     }
     float* io = reinterpret_cast<float*>(g->d_io);
     float* dU = U_out ? io : nullptr;
     float* db = b_out ? io + 8 * N : nullptr;
     WB_CK((wb::launch_export<float, float>(static_cast<const float*>(g->un), dU, db, g->d_blocks,
-                                          g->d_patches, g->d_links, N, g->nblocks, g->stream)));
+                                          g->d_patches, g->d_links, N, g->nblocks, false, g->stream)));
     if (U_out)
         WB_CK(cudaMemcpyAsync(U_out, dU, sizeof(float) * 8 * N, cudaMemcpyDeviceToHost, g->stream));
     if (b_out)
@@ -1014,10 +1014,10 @@ int wb_get_state(wb_grid* g, double* U_out, double* b_out) {
     double* db = b_out ? (in_place ? b_out : g->d_io + 8 * N) : nullptr;
     if (g->precision == WB_FP64)
         WB_CK((wb::launch_export<double, double>(static_cast<const double*>(g->un), dU, db, g->d_blocks,
-                                        g->d_patches, g->d_links, N, g->nblocks, g->stream)));
+                                        g->d_patches, g->d_links, N, g->nblocks, in_place, g->stream)));
     else
         WB_CK((wb::launch_export<float, double>(static_cast<const float*>(g->un), dU, db, g->d_blocks,
-                                       g->d_patches, g->d_links, N, g->nblocks, g->stream)));
+                                       g->d_patches, g->d_links, N, g->nblocks, in_place, g->stream)));
     if (U_out && !in_place)
         WB_CK(cudaMemcpyAsync(U_out, dU, sizeof(double) * 8 * N, cudaMemcpyDeviceToHost, g->stream));
     if (b_out && !in_place)

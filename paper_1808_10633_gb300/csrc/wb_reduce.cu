@@ -396,12 +396,16 @@ totals_pass2(const double* __restrict__ partial, int npartial, double dV, double
 // with (rho, mx, my, mz, Bx, By, Bz, E), b[patch][3][cells]; state layout:
 // field-major over all patches.
 //
-// Both copies are bound by the host link, which moves whole 128-byte lines: each
-// field's threads are shifted so that a warp covers one line of its host array
+// To and from page-locked host arrays (HOST) both copies are bound by the link, which
+// moves whole 128-byte lines: each field's threads are shifted so that a warp covers
+// one line of its host array
 // (the fields of a patch of odd size start at odd places), and the ragged
 // accesses fall on device memory.  FP32 state in and out, GB/s over the link:
 // 320 uneven patches 190 / 142 -> 210 / 192, 64 uneven bricks 187 / 127 -> 205 /
-// 188; 192^3, aligned as it is, 207 / 190 -> 208 / 190.
+// 188; 192^3, aligned as it is, 207 / 190 -> 208 / 190.  From device staging
+// (pageable arrays) they are bound by the latency of the loads: one cell per thread,
+// all its loads before the first store (192^3, FP64 arrays and an FP32 state, in and
+// out: 190 / 347 us with the shifted threads' field by field, 98 / 253 so).
 template <class H>
 __device__ __forceinline__ int line_offset(const H* p) {
     return (int)((reinterpret_cast<unsigned long long>(p) / sizeof(H)) % (128 / sizeof(H)));
@@ -416,7 +420,7 @@ __device__ __forceinline__ void line_cells(const H* p, int first, int np, F&& f)
     if (first + kCellBlock >= np && l + kCellBlock < np) f(l + kCellBlock);
 }
 
-template <class T, class H>
+template <class T, class H, bool HOST>
 __global__ void __launch_bounds__(kCellBlock)
 import_kernel(const H* __restrict__ U, const H* __restrict__ b, T* __restrict__ q,
               const CellBlock* __restrict__ blocks, const PatchDev* __restrict__ patches,
@@ -424,15 +428,27 @@ import_kernel(const H* __restrict__ U, const H* __restrict__ b, T* __restrict__ 
     const CellBlock cb = blocks[blockIdx.x];
     const PatchDev P = patches[cb.x];
     const int np = P.nx * P.ny * P.nz;
+    auto from = [&](int f) {
+        return f < 5 ? U + 8 * P.off + (long long)(f == 4 ? 7 : f) * np : b + 3 * P.off + (long long)(f - 5) * np;
+    };
+    if constexpr (HOST) {
 #pragma unroll
-    for (int f = 0; f < 8; f++) {
-        const H* from = f < 5 ? U + 8 * P.off + (long long)(f == 4 ? 7 : f) * np : b + 3 * P.off + (long long)(f - 5) * np;
-        T* to = q + f * N + P.off;
-        line_cells(from, cb.y, np, [&](int l) { to[l] = T(from[l]); });
+        for (int f = 0; f < 8; f++) {
+            T* to = q + f * N + P.off;
+            line_cells(from(f), cb.y, np, [&](int l) { to[l] = T(from(f)[l]); });
+        }
+    } else {
+        const int l = cb.y + threadIdx.x;
+        if (l >= np) return;
+        H v[8];
+#pragma unroll
+        for (int f = 0; f < 8; f++) v[f] = from(f)[l];
+#pragma unroll
+        for (int f = 0; f < 8; f++) q[f * N + P.off + l] = T(v[f]);
     }
 }
 
-template <class T, class H, bool LINKED>
+template <class T, class H, bool LINKED, bool HOST>
 __global__ void __launch_bounds__(kCellBlock)
 export_kernel(const T* __restrict__ q, H* __restrict__ U, H* __restrict__ b,
               const CellBlock* __restrict__ blocks, const PatchDev* __restrict__ patches,
@@ -440,6 +456,37 @@ export_kernel(const T* __restrict__ q, H* __restrict__ U, H* __restrict__ b,
     const CellBlock cb = blocks[blockIdx.x];
     const PatchDev P = patches[cb.x];
     const int nxy = P.nx * P.ny, np = nxy * P.nz;
+    if constexpr (!HOST) {
+        const int l = cb.y + threadIdx.x;
+        if (l >= np) return;
+        const int k = l / nxy;
+        const int rem = l - k * nxy;
+        const int j = rem / P.nx;
+        const int i = rem - j * P.nx;
+        const long long c = P.off + l;
+        T v[5], face[3], up[3];
+#pragma unroll
+        for (int f = 0; f < 3; f++) face[f] = q[(5 + f) * N + c];
+        if (U) {
+#pragma unroll
+            for (int f = 0; f < 5; f++) v[f] = q[f * N + c];
+            up[0] = q[5 * N + upper<LINKED>(patches, links, cb.x, P, i + 1, j, k)];
+            up[1] = q[6 * N + upper<LINKED>(patches, links, cb.x, P, i, j + 1, k)];
+            up[2] = q[7 * N + upper<LINKED>(patches, links, cb.x, P, i, j, k + 1)];
+            H* u = U + 8 * P.off + l;
+#pragma unroll
+            for (int f = 0; f < 4; f++) u[(long long)f * np] = H(double(v[f]));
+#pragma unroll
+            for (int f = 0; f < 3; f++) u[(long long)(4 + f) * np] = H(0.5 * (double(face[f]) + double(up[f])));
+            u[7LL * np] = H(double(v[4]));
+        }
+        if (b) {
+            H* o = b + 3 * P.off + l;
+#pragma unroll
+            for (int f = 0; f < 3; f++) o[(long long)f * np] = H(double(face[f]));
+        }
+        return;
+    }
     if (U) {
 #pragma unroll
         for (int f = 0; f < 8; f++) {
@@ -566,19 +613,27 @@ cudaError_t launch_totals(const T* state, const PatchDev*, int, long long ncells
 
 template <class T, class H>
 cudaError_t launch_import(const H* U, const H* b, T* state, const CellBlock* blocks,
-                          const PatchDev* patches, long long ncells, int nblocks, cudaStream_t s) {
-    import_kernel<T, H><<<nblocks, kCellBlock, 0, s>>>(U, b, state, blocks, patches, ncells);
+                          const PatchDev* patches, long long ncells, int nblocks, bool host, cudaStream_t s) {
+    if (host) import_kernel<T, H, true><<<nblocks, kCellBlock, 0, s>>>(U, b, state, blocks, patches, ncells);
+    else import_kernel<T, H, false><<<nblocks, kCellBlock, 0, s>>>(U, b, state, blocks, patches, ncells);
     return cudaGetLastError();
+}
+
+template <class T, class H, bool LINKED>
+void launch_export_links(const T* state, H* U, H* b, const CellBlock* blocks, const PatchDev* patches,
+                         const int* links, long long ncells, int nblocks, bool host, cudaStream_t s) {
+    if (host)
+        export_kernel<T, H, LINKED, true><<<nblocks, kCellBlock, 0, s>>>(state, U, b, blocks, patches, links, ncells);
+    else
+        export_kernel<T, H, LINKED, false><<<nblocks, kCellBlock, 0, s>>>(state, U, b, blocks, patches, links, ncells);
 }
 
 template <class T, class H>
 cudaError_t launch_export(const T* state, H* U, H* b, const CellBlock* blocks,
                           const PatchDev* patches, const int* links, long long ncells, int nblocks,
-                          cudaStream_t s) {
-    if (links)
-        export_kernel<T, H, true><<<nblocks, kCellBlock, 0, s>>>(state, U, b, blocks, patches, links, ncells);
-    else
-        export_kernel<T, H, false><<<nblocks, kCellBlock, 0, s>>>(state, U, b, blocks, patches, links, ncells);
+                          bool host, cudaStream_t s) {
+    if (links) launch_export_links<T, H, true>(state, U, b, blocks, patches, links, ncells, nblocks, host, s);
+    else launch_export_links<T, H, false>(state, U, b, blocks, patches, links, ncells, nblocks, host, s);
     return cudaGetLastError();
 }
 
@@ -594,17 +649,17 @@ cudaError_t launch_export(const T* state, H* U, H* b, const CellBlock* blocks,
                                           int, double, double*, cudaStream_t);                \
     template cudaError_t launch_import<T, double>(const double*, const double*, T*,          \
                                                   const CellBlock*, const PatchDev*, long long, \
-                                                  int, cudaStream_t);                          \
+                                                  int, bool, cudaStream_t);                    \
     template cudaError_t launch_export<T, double>(const T*, double*, double*, const CellBlock*, \
                                                   const PatchDev*, const int*, long long, int,  \
-                                                  cudaStream_t);                                \
+                                                  bool, cudaStream_t);                         \
     template cudaError_t launch_export_flux<T>(const T*, double*, const CellBlock*,           \
                                                const PatchDev*, long long, int, cudaStream_t);
 WB_INST(float)
 template cudaError_t launch_import<float, float>(const float*, const float*, float*, const CellBlock*,
-                                                 const PatchDev*, long long, int, cudaStream_t);
+                                                 const PatchDev*, long long, int, bool, cudaStream_t);
 template cudaError_t launch_export<float, float>(const float*, float*, float*, const CellBlock*,
-                                                 const PatchDev*, const int*, long long, int, cudaStream_t);
+                                                 const PatchDev*, const int*, long long, int, bool, cudaStream_t);
 WB_INST(double)
 #undef WB_INST
 
