@@ -21,6 +21,8 @@
 #pragma once
 #include "wb_sweep.cuh"
 
+#include <cmath>
+
 namespace wb {
 namespace {
 
@@ -471,7 +473,8 @@ __device__ __forceinline__ void tile_body(const SweepArgs<T>& A, const Tile& til
 // ---- an axis of one cell ----------------------------------------------------------------
 // A periodic patch one cell deep along the axis (2-D and 1-D runs): all six
 // stencil cells of an interface are its one cell, every projected difference
-// is zero, and the flux is the central combination of four equal fluxes.  One
+// is zero, and the flux is the central combination of four equal fluxes (or NaN,
+// where the cell's state has no eigen-structure).  One
 // thread per cell; tile.y is the first of kSweepNT cells.  As ordinary tiles
 // these sweeps ran one warp per block at half its lanes through the whole
 // interface arithmetic (64^2 x 1, RK4, FP64, four steps: 2.24 -> 1.24 ms).
@@ -485,11 +488,20 @@ __device__ __forceinline__ void flat_body(const SweepArgs<T>& A, const Tile& til
     long long c;
     load_cell<T>(A, P, i, j, k, r, c);
     derive_cell<T, AXIS>(A, r, c, sm, kSweepNT, tid, A.er != nullptr);
+    // a state without an eigen-structure gives NaN, as the interface arithmetic does
+    // (the zero differences times its infinite or NaN coefficients)
+    const T p = sm[SP_P * kSweepNT + tid];
+    bool sound = r.rho > T(0) && p > T(0) && isfinite(r.rho) && isfinite(p);
     T F[7];
 #pragma unroll
     for (int f = 0; f < 7; f++) {
         const T f1 = sm[at_f<T>(f, kSweepNT, tid)], f2 = f1 + f1;
         F[f] = (T(7) * f2 - f2) * T(1.0 / 12.0);
+        sound = sound && isfinite(f1);
+    }
+    if (!sound) {
+#pragma unroll
+        for (int f = 0; f < 7; f++) F[f] = T(NAN);
     }
     store_flux<T, AXIS>(A, c, F);
 }
