@@ -206,10 +206,10 @@ int wb_face_fluxes(wb_grid *g, int axis, double *F_out);
  * shape, so that each shape runs as its own launch of one tile per block.
  * wb_autotune measures, for each axis, one sweep of the current state with
  * WB_NTILE_CANDIDATE tables (CUDA events, mean of the second and third of three
- * launches): the cost-model table, each fixed shape everywhere, and the
- * cost-model table again (the same one; the candidate's number is kept), and
- * keeps the fastest.  ms_out (host, 3 * WB_NTILE_CANDIDATE, may be NULL): the
- * times, per axis [model, shape 0, shape 1, shape 2, model].  Not for
+ * launches): the cost-model table and each fixed shape everywhere, and keeps the
+ * fastest.  ms_out (host, 3 * WB_NTILE_CANDIDATE, may be NULL): the times, per
+ * axis [model, shape 0, shape 1, shape 2, model]; the last candidate is the first
+ * one's table under another number, measured once.  Not for
  * WB_FP32_LEARNED grids.  Synchronises. */
 #define WB_NTILE_SHAPE 3
 #define WB_NTILE_CANDIDATE (WB_NTILE_SHAPE + 2)

@@ -31,6 +31,7 @@ EXPORTS = ("wb_init_grid", "wb_set_state", "wb_step", "wb_step_cfl", "wb_cfl_dt"
            "wb_learned_stats", "wb_div_b", "wb_set_step_totals", "wb_step_totals",
            "wb_set_state_f32", "wb_get_state_f32")
 MLP_NFIELD, MLP_NPARAM, MLP_RECORD = 7, 1379, 12
+# every table is ordered by shape: the last one is the first
 TILE_CANDIDATES = ("per-patch model", "shape 0", "shape 1", "shape 2", "per-patch model by shape")
 KERNEL_CLASSES = ("sweep_x", "sweep_y", "sweep_z", "update", "cfl", "dt", "totals", "emf")
 
@@ -274,7 +275,7 @@ class Grid:
     def autotune(self) -> np.ndarray:
         """Measure and keep the fastest sweep tile tables; times (3, 5) in ms
         per axis for TILE_CANDIDATES (per-patch model, shape 0, shape 1,
-        shape 2, per-patch model ordered by shape)."""
+        shape 2, and the first again)."""
         ms = np.empty(3 * len(TILE_CANDIDATES))
         _check(self._lib.wb_autotune(self._h, ms.ctypes.data))
         return ms.reshape(3, len(TILE_CANDIDATES))
