@@ -83,8 +83,8 @@ __device__ __forceinline__ double widen(float x) {
 
 // ---- one FP64 value or two FP32 lanes -------------------------------------------
 template <class V> struct Lanes;
-template <> struct Lanes<double> { using S = double; static constexpr int N = 1; };
-template <> struct Lanes<float2> { using S = float; static constexpr int N = 2; };
+template <> struct Lanes<double> { using S = double; };
+template <> struct Lanes<float2> { using S = float; };
 
 template <class V> __device__ __forceinline__ V splat(typename Lanes<V>::S v);
 template <> __device__ __forceinline__ double splat<double>(double v) { return v; }
@@ -96,7 +96,6 @@ __device__ __forceinline__ double vadd(double a, double b) { return a + b; }
 __device__ __forceinline__ double vsub(double a, double b) { return a - b; }
 __device__ __forceinline__ double vfms(double a, double b, double c) { return fma(a, b, -c); }
 __device__ __forceinline__ double vrcp(double a) { return recip(a); }
-__device__ __forceinline__ double vneg(double a) { return -a; }
 __device__ __forceinline__ float2 vfma(float2 a, float2 b, float2 c) { return __ffma2_rn(a, b, c); }
 __device__ __forceinline__ float2 vmul(float2 a, float2 b) { return __fmul2_rn(a, b); }
 __device__ __forceinline__ float2 vadd(float2 a, float2 b) { return __fadd2_rn(a, b); }
@@ -104,21 +103,8 @@ __device__ __forceinline__ float2 vsub(float2 a, float2 b) { return __ffma2_rn(b
 __device__ __forceinline__ float2 vfms(float2 a, float2 b, float2 c) {      // a b - c
     return make_float2(fmaf(a.x, b.x, -c.x), fmaf(a.y, b.y, -c.y));
 }
-__device__ __forceinline__ float2 vneg(float2 a) { return make_float2(-a.x, -a.y); }
 __device__ __forceinline__ float2 vrcp(float2 a) { return make_float2(recip(a.x), recip(a.y)); }
 __device__ __forceinline__ double vabs(double a) { return fabs(a); }
 __device__ __forceinline__ float2 vabs(float2 a) { return make_float2(fabsf(a.x), fabsf(a.y)); }
-// max of values >= 0: their bit patterns order like the values, so FP64 takes
-// an integer max, off the FP64 pipe
-__device__ __forceinline__ double vmax0(double a, double b) {
-    return __longlong_as_double(max(__double_as_longlong(a), __double_as_longlong(b)));
-}
-__device__ __forceinline__ float2 vmax0(float2 a, float2 b) { return make_float2(fmaxf(a.x, b.x), fmaxf(a.y, b.y)); }
-
-// lane l of v
-__device__ __forceinline__ double lane(double v, int) { return v; }
-__device__ __forceinline__ float lane(float2 v, int l) { return l == 0 ? v.x : v.y; }
-__device__ __forceinline__ void set_lane(double& v, int, double s) { v = s; }
-__device__ __forceinline__ void set_lane(float2& v, int l, float s) { (l == 0 ? v.x : v.y) = s; }
 
 }  // namespace wb

@@ -16,10 +16,12 @@
 // Per interface (cells i-2..i+3 of the stencil):
 //   1. interface state = mean of the primitives of cells i, i+1;
 //   2. closed-form 7-wave eigensystem (Roe-Balsara normalisation) at it;
-//   3. projection of U_k, F_k on the left eigenvectors, done as
-//      (dW/dU) x followed by the sparse left vectors, in two groups of
-//      characteristic fields (fast+slow, then Alfven+entropy) so that the
-//      projected stencil fits in registers in FP64 too;
+//   3. projection of the stencil's five U and F differences on the left
+//      eigenvectors, done as (dW/dU) x followed by the sparse left vectors; the
+//      Alfven and entropy fields wait in shared memory while the fast and slow
+//      ones are reconstructed (FP32 here, U and F in one packed pair; FP64 in
+//      wb_sweep_js.cuh; the tensor-core learned sweep projects the six cells,
+//      in two groups of fields);
 //   4. local Lax-Friedrichs splitting, alpha_s = max |lambda_s| over the
 //      stencil and the interface state;
 //   5. WENO5-JS weights and phi_N for both split fluxes;

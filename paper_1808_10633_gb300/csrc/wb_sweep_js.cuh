@@ -141,13 +141,13 @@ __device__ __forceinline__ V z_phi12(V a, V b, V c, V d, typename Lanes<V>::S ep
 // phi_N(D-_{i+5/2} ..), from the split differences taken twice over, p_m = 2 D+
 // of steps m = 0..3 and n_m = 2 D- of steps m = 1..4 of the stencil: phi_N with
 // 4 eps on them, halved (exact).
-template <class V, bool Z>
-__device__ __forceinline__ V weno_corr(const V (&p)[4], const V (&n)[4]) {
-    using S = typename Lanes<V>::S;
-    constexpr S eps16 = S(4.0 * 1e-6 / 16.0);
+template <bool Z>
+__device__ __forceinline__ double weno_corr(const double (&p)[4], const double (&n)[4]) {
+    constexpr double eps16 = 4.0 * 1e-6 / 16.0;
     if constexpr (Z) {
-        const V rm = z_phi12<V>(n[3], n[2], n[1], n[0], eps16), rp = z_phi12<V>(p[0], p[1], p[2], p[3], eps16);
-        return vmul(vsub(rm, rp), splat<V>(S(1.0 / 24.0)));
+        const double rm = z_phi12<double>(n[3], n[2], n[1], n[0], eps16);
+        const double rp = z_phi12<double>(p[0], p[1], p[2], p[3], eps16);
+        return (rm - rp) * (1.0 / 24.0);
     } else {
         return half_phi_diff(n[3], n[2], n[1], n[0], p[0], p[1], p[2], p[3], eps16);
     }
@@ -167,175 +167,161 @@ struct JsWeights {
     }
 };
 
-// ---- eigen-structure over V ---------------------------------------------------------
+// ---- one interface in FP64 --------------------------------------------------------------
 // Left-vector coefficients (negated where the projection subtracts), the
 // speeds and what the back-projection needs.
-template <class V>
-struct EigV {
-    V rho, nu, nv1, nv2, nbm, hv2, be1, be2, nbe2;
-    V cf, cs, ca;
-    V Af, Bf, Cf, Df, As, Bs, Cs, Ds, nEe;
-    V nvb;                       // -(be1 v1 + be2 v2)
-    V q1, q2, q0, r1, r2;        // Alfven rows: q1 x3 + q2 x2 + q0 x0 +- (r1 x5 + r2 x4)
+struct Eig64 {
+    double rho, nu, nv1, nv2, nbm, hv2, be1, be2, nbe2;
+    double cf, cs, ca;
+    double Af, Bf, Cf, Df, As, Bs, Cs, Ds, nEe;
+    double nvb;                       // -(be1 v1 + be2 v2)
+    double q1, q2, q0, r1, r2;        // Alfven rows: q1 x3 + q2 x2 + q0 x0 +- (r1 x5 + r2 x4)
 };
 
-template <class V, class S = typename Lanes<V>::S>
-__device__ __forceinline__ void eigen_lane(int l, V rho_, V u_, V v1_, V v2_, V bn_, V b1_, V b2_, V p_, S gamma,
-                                           S rg1, EigV<V>& e, V (&back)[kNBackV]) {
-    Eig<S> s;
-    S bp[kNBack];
-    eigen<S>(lane(rho_, l), lane(u_, l), lane(v1_, l), lane(v2_, l), lane(bn_, l), lane(b1_, l), lane(b2_, l),
-             lane(p_, l), gamma, s, bp, 1);
-    set_lane(e.rho, l, s.rho);
-    set_lane(e.nu, l, -s.u);
-    set_lane(e.nv1, l, -s.v1);
-    set_lane(e.nv2, l, -s.v2);
-    set_lane(e.nbm, l, -s.bm);
-    set_lane(e.hv2, l, s.hv2);
-    set_lane(e.be1, l, s.be1);
-    set_lane(e.be2, l, s.be2);
-    set_lane(e.nbe2, l, -s.be2);
-    set_lane(e.cf, l, s.cf);
-    set_lane(e.cs, l, s.cs);
-    set_lane(e.ca, l, s.ca);
-    set_lane(e.Af, l, s.Af);
-    set_lane(e.Bf, l, s.Bf);
-    set_lane(e.Cf, l, s.Cf);
-    set_lane(e.Df, l, s.Df);
-    set_lane(e.As, l, s.As);
-    set_lane(e.Bs, l, s.Bs);
-    set_lane(e.Cs, l, s.Cs);
-    set_lane(e.Ds, l, s.Ds);
-    set_lane(e.nEe, l, -s.Ee);
-    set_lane(e.nvb, l, -(s.be1 * s.v1 + s.be2 * s.v2));
-    const S q1 = s.Aa * s.be1, q2 = -s.Aa * s.be2;
-    set_lane(e.q1, l, q1);
-    set_lane(e.q2, l, q2);
-    set_lane(e.q0, l, -(q1 * s.v2 + q2 * s.v1));
-    set_lane(e.r1, l, s.Ba * s.be1);
-    set_lane(e.r2, l, -s.Ba * s.be2);
-    set_lane(back[B_ALF], l, bp[BP_ALF]);
-    set_lane(back[B_ALS], l, bp[BP_ALS]);
-    set_lane(back[B_AFCF], l, bp[BP_AFCF]);
-    set_lane(back[B_ASCS], l, bp[BP_ASCS]);
-    set_lane(back[B_ASR], l, bp[BP_ASR]);
-    set_lane(back[B_SSR], l, bp[BP_SSR]);
-    set_lane(back[B_RAG], l, bp[BP_RA2] * rg1);
+__device__ __forceinline__ void eigen64(double rho, double u, double v1, double v2, double bn, double b1, double b2,
+                                        double p, double gamma, double rg1, Eig64& e, double (&back)[kNBackV]) {
+    Eig<double> s;
+    double bp[kNBack];
+    eigen<double>(rho, u, v1, v2, bn, b1, b2, p, gamma, s, bp, 1);
+    e.rho = s.rho;
+    e.nu = -s.u;
+    e.nv1 = -s.v1;
+    e.nv2 = -s.v2;
+    e.nbm = -s.bm;
+    e.hv2 = s.hv2;
+    e.be1 = s.be1;
+    e.be2 = s.be2;
+    e.nbe2 = -s.be2;
+    e.cf = s.cf;
+    e.cs = s.cs;
+    e.ca = s.ca;
+    e.Af = s.Af;
+    e.Bf = s.Bf;
+    e.Cf = s.Cf;
+    e.Df = s.Df;
+    e.As = s.As;
+    e.Bs = s.Bs;
+    e.Cs = s.Cs;
+    e.Ds = s.Ds;
+    e.nEe = -s.Ee;
+    e.nvb = -(s.be1 * s.v1 + s.be2 * s.v2);
+    e.q1 = s.Aa * s.be1;
+    e.q2 = -s.Aa * s.be2;
+    e.q0 = -(e.q1 * s.v2 + e.q2 * s.v1);
+    e.r1 = s.Ba * s.be1;
+    e.r2 = -s.Ba * s.be2;
+    back[B_ALF] = bp[BP_ALF];
+    back[B_ALS] = bp[BP_ALS];
+    back[B_AFCF] = bp[BP_AFCF];
+    back[B_ASCS] = bp[BP_ASCS];
+    back[B_ASR] = bp[BP_ASR];
+    back[B_SSR] = bp[BP_SSR];
+    back[B_RAG] = bp[BP_RA2] * rg1;
 }
 
 // One difference vector on all seven left eigenvectors: fast-, slow-, slow+,
 // fast+ into o4, Alfven-, entropy, Alfven+ into o3.
-template <class V>
-__device__ __forceinline__ void project(const EigV<V>& e, const V (&x)[7], V (&o4)[4], V (&o3)[3]) {
-    const V du = vfma(e.nu, x[0], x[1]);
-    const V vpar = vfma(e.be1, x[2], vfma(e.be2, x[3], vmul(e.nvb, x[0])));
-    const V bpar = vfma(e.be1, x[4], vmul(e.be2, x[5]));
-    V P = vfma(e.hv2, x[0], x[6]);
-    P = vfma(e.nu, x[1], P);
-    P = vfma(e.nv1, x[2], P);
-    P = vfma(e.nv2, x[3], P);
-    P = vfma(e.nbm, bpar, P);
-    const V tf1 = vfma(e.Af, du, vmul(e.Bf, vpar)), tf2 = vfma(e.Cf, bpar, vmul(e.Df, P));
-    const V ts1 = vfma(e.As, du, vmul(e.Bs, vpar)), ts2 = vfma(e.Cs, bpar, vmul(e.Ds, P));
-    o4[0] = vsub(tf2, tf1);
-    o4[1] = vsub(ts2, ts1);
-    o4[2] = vadd(ts2, ts1);
-    o4[3] = vadd(tf2, tf1);
-    const V t1 = vfma(e.q1, x[3], vfma(e.q2, x[2], vmul(e.q0, x[0])));
-    const V t2 = vfma(e.r1, x[5], vmul(e.r2, x[4]));
-    o3[0] = vadd(t1, t2);
-    o3[1] = vfma(e.nEe, P, x[0]);
-    o3[2] = vsub(t1, t2);
-}
-
-template <class V>
-__device__ __forceinline__ V ld(const typename Lanes<V>::S* __restrict__ p) {
-    return *reinterpret_cast<const V*>(p);
+__device__ __forceinline__ void project(const Eig64& e, const double (&x)[7], double (&o4)[4], double (&o3)[3]) {
+    const double du = fma(e.nu, x[0], x[1]);
+    const double vpar = fma(e.be1, x[2], fma(e.be2, x[3], e.nvb * x[0]));
+    const double bpar = fma(e.be1, x[4], e.be2 * x[5]);
+    double P = fma(e.hv2, x[0], x[6]);
+    P = fma(e.nu, x[1], P);
+    P = fma(e.nv1, x[2], P);
+    P = fma(e.nv2, x[3], P);
+    P = fma(e.nbm, bpar, P);
+    const double tf1 = fma(e.Af, du, e.Bf * vpar), tf2 = fma(e.Cf, bpar, e.Df * P);
+    const double ts1 = fma(e.As, du, e.Bs * vpar), ts2 = fma(e.Cs, bpar, e.Ds * P);
+    o4[0] = tf2 - tf1;
+    o4[1] = ts2 - ts1;
+    o4[2] = ts2 + ts1;
+    o4[3] = tf2 + tf1;
+    const double t1 = fma(e.q1, x[3], fma(e.q2, x[2], e.q0 * x[0]));
+    const double t2 = fma(e.r1, x[5], e.r2 * x[4]);
+    o3[0] = t1 + t2;
+    o3[1] = fma(e.nEe, P, x[0]);
+    o3[2] = t1 - t2;
 }
 
 // Largest |lambda_s| over the six cells and the interface state.
-template <class V, int CS>
-__device__ __forceinline__ V lf_speed_v(const typename Lanes<V>::S* __restrict__ cell, int nc, int s, const EigV<V>& e) {
-    const V nc_s = (s == 0 || s == 6) ? e.cf : ((s == 1 || s == 5) ? e.ca : e.cs);
-    V al = s == 3 ? vabs(e.nu) : (s < 3 ? vabs(vadd(e.nu, nc_s)) : vabs(vsub(e.nu, nc_s)));
+template <int CS>
+__device__ __forceinline__ double lf_speed64(const double* __restrict__ cell, int nc, int s, const Eig64& e) {
+    const double nc_s = (s == 0 || s == 6) ? e.cf : ((s == 1 || s == 5) ? e.ca : e.cs);
+    double al = s == 3 ? fabs(e.nu) : (s < 3 ? fabs(e.nu + nc_s) : fabs(e.nu - nc_s));
 #pragma unroll
-    for (int m = 0; m < 6; m++) al = vmax0(al, ld<V>(cell + (SL + s) * nc + m * CS));
+    for (int m = 0; m < 6; m++) al = tmax_nonneg(al, cell[(SL + s) * nc + m * CS]);
     return al;
 }
 
-// Flux through one interface (one per lane): cell points at stencil cell 0,
-// the six cells are CS values apart.
-template <class V, bool Z, int CS>
-__device__ __forceinline__ void sweep_flux(const typename Lanes<V>::S* __restrict__ cell, int nc,
-                                           typename Lanes<V>::S gamma, typename Lanes<V>::S rg1, V* __restrict__ slot,
-                                           int sstride, V (&out)[7]) {
-    using S = typename Lanes<V>::S;
+// Flux through one interface: cell points at stencil cell 0, the six cells are
+// CS values apart.
+template <bool Z, int CS>
+__device__ __forceinline__ void sweep_flux(const double* __restrict__ cell, int nc, double gamma, double rg1,
+                                           double* __restrict__ slot, int sstride, double (&out)[7]) {
     // 1-2. interface state and eigen-structure
-    EigV<V> e;
+    Eig64 e;
     {
-        const V h = splat<V>(S(0.5));
-        auto mean = [&](int s) { return vmul(h, vadd(ld<V>(cell + s * nc + 2 * CS), ld<V>(cell + s * nc + 3 * CS))); };
-        const V rho = mean(SU), u = mean(SP_U), v1 = mean(SP_V1), v2 = mean(SP_V2), bn = mean(SP_BN),
-                b1 = mean(SU + 4), b2 = mean(SU + 5), p = mean(SP_P);
-        V back[kNBackV];
-#pragma unroll
-        for (int l = 0; l < Lanes<V>::N; l++) eigen_lane<V>(l, rho, u, v1, v2, bn, b1, b2, p, gamma, rg1, e, back);
+        auto mean = [&](int s) { return 0.5 * (cell[s * nc + 2 * CS] + cell[s * nc + 3 * CS]); };
+        const double rho = mean(SU), u = mean(SP_U), v1 = mean(SP_V1), v2 = mean(SP_V2), bn = mean(SP_BN),
+                     b1 = mean(SU + 4), b2 = mean(SU + 5), p = mean(SP_P);
+        double back[kNBackV];
+        eigen64(rho, u, v1, v2, bn, b1, b2, p, gamma, rg1, e, back);
 #pragma unroll
         for (int k = 0; k < kNBackV; k++) slot[k * sstride] = back[k];
     }
     // 4. Lax-Friedrichs speeds
-    V al[7];
+    double al[7];
 #pragma unroll
-    for (int s = 0; s < 7; s++) al[s] = lf_speed_v<V, CS>(cell, nc, s, e);
+    for (int s = 0; s < 7; s++) al[s] = lf_speed64<CS>(cell, nc, s, e);
     // 3-4. the five differences of the stencil's U and F on all seven fields,
     // split: 2 D+- = l dF +- alpha l dU (eight values per field; those of the
     // Alfven and entropy fields wait in this thread's slots)
-    V* park = slot + kNBackV * sstride;
-    V dp[7][4], dn[7][4];
-    V u0[7], f0[6];
+    double* park = slot + kNBackV * sstride;
+    double dp[7][4], dn[7][4];
+    double u0[7], f0[6];
 #pragma unroll
-    for (int f = 0; f < 7; f++) u0[f] = ld<V>(cell + (SU + f) * nc);
+    for (int f = 0; f < 7; f++) u0[f] = cell[(SU + f) * nc];
 #pragma unroll
-    for (int f = 0; f < 6; f++) f0[f] = ld<V>(cell + at_f<S>(f + 1, nc, 0));
+    for (int f = 0; f < 6; f++) f0[f] = cell[at_f<double>(f + 1, nc, 0)];
 #pragma unroll
     for (int m = 0; m < 5; m++) {
-        V x[7], w4[4], w3[3], g4[4], g3[3];
+        double x[7], w4[4], w3[3], g4[4], g3[3];
 #pragma unroll
         for (int f = 0; f < 7; f++) {
-            const V u1 = ld<V>(cell + (SU + f) * nc + (m + 1) * CS);
-            x[f] = vsub(u1, u0[f]);
+            const double u1 = cell[(SU + f) * nc + (m + 1) * CS];
+            x[f] = u1 - u0[f];
             u0[f] = u1;
         }
-        const V dm = x[1];                   // the mass flux is the normal momentum
+        const double dm = x[1];                   // the mass flux is the normal momentum
         project(e, x, w4, w3);
         x[0] = dm;
 #pragma unroll
         for (int f = 0; f < 6; f++) {
-            const V f1 = ld<V>(cell + at_f<S>(f + 1, nc, (m + 1) * CS));
-            x[f + 1] = vsub(f1, f0[f]);
+            const double f1 = cell[at_f<double>(f + 1, nc, (m + 1) * CS)];
+            x[f + 1] = f1 - f0[f];
             f0[f] = f1;
         }
         project(e, x, g4, g3);
 #pragma unroll
         for (int s = 0; s < 7; s++) {
-            const V w = s & 1 ? w3[s >> 1] : w4[s >> 1], g = s & 1 ? g3[s >> 1] : g4[s >> 1];
-            V* mine = park + (s >> 1) * 8 * sstride;
+            const double w = s & 1 ? w3[s >> 1] : w4[s >> 1], g = s & 1 ? g3[s >> 1] : g4[s >> 1];
+            double* mine = park + (s >> 1) * 8 * sstride;
             if (m < 4) {
-                const V d = vfma(al[s], w, g);
+                const double d = fma(al[s], w, g);
                 if (s & 1) mine[m * sstride] = d;
                 else dp[s][m] = d;
             }
             if (m > 0) {
-                const V d = vfma(vneg(al[s]), w, g);
+                const double d = fma(-al[s], w, g);
                 if (s & 1) mine[(3 + m) * sstride] = d;
                 else dn[s][m - 1] = d;
             }
         }
     }
     // 5. weights, fast and slow fields, then Alfven and entropy
-    V corr[7];
+    double corr[7];
 #pragma unroll
-    for (int s = 0; s < 7; s += 2) corr[s] = weno_corr<V, Z>(dp[s], dn[s]);
+    for (int s = 0; s < 7; s += 2) corr[s] = weno_corr<Z>(dp[s], dn[s]);
 #pragma unroll
     for (int s = 1; s < 7; s += 2) {
 #pragma unroll
@@ -343,42 +329,40 @@ __device__ __forceinline__ void sweep_flux(const typename Lanes<V>::S* __restric
             dp[s][m] = park[((s >> 1) * 8 + m) * sstride];
             dn[s][m] = park[((s >> 1) * 8 + 4 + m) * sstride];
         }
-        corr[s] = weno_corr<V, Z>(dp[s], dn[s]);
+        corr[s] = weno_corr<Z>(dp[s], dn[s]);
     }
     // 6. back-projection: sum_s r_s corr_s in primitive variables, then dU/dW,
     // and the central flux (7 (F_i + F_{i+1}) - (F_{i-1} + F_{i+2})) / 12
-    const V alf = slot[B_ALF * sstride], als = slot[B_ALS * sstride];
-    const V afcf = slot[B_AFCF * sstride], ascs = slot[B_ASCS * sstride];
-    const V ssr = slot[B_SSR * sstride];
-    const V Fp = vadd(corr[6], corr[0]), Fm = vsub(corr[6], corr[0]);
-    const V Sp = vadd(corr[4], corr[2]), Sm = vsub(corr[4], corr[2]);
-    const V Ap = vadd(corr[5], corr[1]), nAm = vsub(corr[1], corr[5]);
-    const V fs = vfma(alf, Fp, vmul(als, Sp));
-    const V drho = vfma(e.rho, fs, corr[3]);
-    const V du = vfma(afcf, Fm, vmul(ascs, Sm));
-    V sg;                                         // sgn(B_n)
-#pragma unroll
-    for (int l = 0; l < Lanes<V>::N; l++) set_lane(sg, l, lane(ssr, l) < S(0) ? S(-1) : S(1));
-    const V dvpar = vmul(sg, vsub(vmul(afcf, Sm), vmul(ascs, Fm)));
-    const V dbpar = vmul(slot[B_ASR * sstride], vsub(vmul(als, Fp), vmul(alf, Sp)));
-    const V dbper = vmul(ssr, nAm);
-    const V dpg = vmul(slot[B_RAG * sstride], fs);             // dp / (gamma - 1)
-    const V dv1 = vfma(e.be1, dvpar, vmul(e.nbe2, Ap)), dv2 = vfma(e.be2, dvpar, vmul(e.be1, Ap));
-    V dF[7];
+    const double alf = slot[B_ALF * sstride], als = slot[B_ALS * sstride];
+    const double afcf = slot[B_AFCF * sstride], ascs = slot[B_ASCS * sstride];
+    const double ssr = slot[B_SSR * sstride];
+    const double Fp = corr[6] + corr[0], Fm = corr[6] - corr[0];
+    const double Sp = corr[4] + corr[2], Sm = corr[4] - corr[2];
+    const double Ap = corr[5] + corr[1], nAm = corr[1] - corr[5];
+    const double fs = fma(alf, Fp, als * Sp);
+    const double drho = fma(e.rho, fs, corr[3]);
+    const double du = fma(afcf, Fm, ascs * Sm);
+    const double sg = ssr < 0.0 ? -1.0 : 1.0;          // sgn(B_n)
+    const double dvpar = sg * (afcf * Sm - ascs * Fm);
+    const double dbpar = slot[B_ASR * sstride] * (als * Fp - alf * Sp);
+    const double dbper = ssr * nAm;
+    const double dpg = slot[B_RAG * sstride] * fs;             // dp / (gamma - 1)
+    const double dv1 = fma(e.be1, dvpar, e.nbe2 * Ap), dv2 = fma(e.be2, dvpar, e.be1 * Ap);
+    double dF[7];
     dF[0] = drho;
-    dF[4] = vfma(e.be1, dbpar, vmul(e.nbe2, dbper));
-    dF[5] = vfma(e.be2, dbpar, vmul(e.be1, dbper));
-    const V nd = vneg(drho);
-    dF[1] = vfma(e.nu, nd, vmul(e.rho, du));
-    dF[2] = vfma(e.nv1, nd, vmul(e.rho, dv1));
-    dF[3] = vfma(e.nv2, nd, vmul(e.rho, dv2));
-    const V vdv = vfma(e.nu, du, vfma(e.nv1, dv1, vmul(e.nv2, dv2)));       // -v dv
-    dF[6] = vfma(e.hv2, drho, vsub(dpg, vfma(e.nbm, dbpar, vmul(e.rho, vdv))));
+    dF[4] = fma(e.be1, dbpar, e.nbe2 * dbper);
+    dF[5] = fma(e.be2, dbpar, e.be1 * dbper);
+    const double nd = -drho;
+    dF[1] = fma(e.nu, nd, e.rho * du);
+    dF[2] = fma(e.nv1, nd, e.rho * dv1);
+    dF[3] = fma(e.nv2, nd, e.rho * dv2);
+    const double vdv = fma(e.nu, du, fma(e.nv1, dv1, e.nv2 * dv2));       // -v dv
+    dF[6] = fma(e.hv2, drho, dpg - fma(e.nbm, dbpar, e.rho * vdv));
 #pragma unroll
     for (int f = 0; f < 7; f++) {
-        const S* F = cell + at_f<S>(f, nc, 0);
-        const V in = vadd(ld<V>(F + 2 * CS), ld<V>(F + 3 * CS)), ex = vadd(ld<V>(F + CS), ld<V>(F + 4 * CS));
-        out[f] = vfma(vfms(in, splat<V>(S(7)), ex), splat<V>(S(1.0 / 12.0)), dF[f]);
+        const double* F = cell + at_f<double>(f, nc, 0);
+        const double in = F[2 * CS] + F[3 * CS], ex = F[CS] + F[4 * CS];
+        out[f] = fma(fma(in, 7.0, -ex), 1.0 / 12.0, dF[f]);
     }
 }
 
@@ -458,7 +442,7 @@ __device__ __forceinline__ void tile_body(const SweepArgs<T>& A, const Tile& til
     T F[7];
     T* slot = sm + kNSlot * NCMAX + tid;
     if constexpr (sizeof(T) == 8) {
-        sweep_flux<T, Z, CS>(sm + i0, NC, T(A.gamma), T(A.rg1), slot, NT, F);
+        sweep_flux<Z, CS>(sm + i0, NC, T(A.gamma), T(A.rg1), slot, NT, F);
     } else {
         int id[6];
 #pragma unroll

@@ -44,8 +44,8 @@ __global__ void kd(const double* x, double* e, double* z, int n) {
         smoothness<double>(v[4 * s], v[4 * s + 1], v[4 * s + 2], v[4 * s + 3], eps16, e[3 * s * n + i],
                            e[(3 * s + 1) * n + i], e[(3 * s + 2) * n + i]);
     const double m[4] = {v[3], v[2], v[1], v[0]}, p[4] = {v[4], v[5], v[6], v[7]};
-    z[i] = weno_corr<double, false>(p, m);
-    z[n + i] = weno_corr<double, true>(p, m);
+    z[i] = weno_corr<false>(p, m);
+    z[n + i] = weno_corr<true>(p, m);
 }
 template <class T, class K> int go(K k, const T* x, T* o, int n) {
     T* d = nullptr;
