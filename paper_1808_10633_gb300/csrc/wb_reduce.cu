@@ -361,7 +361,13 @@ totals_pass1(const T* __restrict__ q, long long N, long long chunk, double* __re
 #pragma unroll
         for (int f = 0; f < 8; f++) {
             if (fabsf(s[f]) <= 3.4e38f && fabsf(eh[f]) <= 3.4e38f) {
-                acc[f] = widen(s[f]) + (widen(eh[f]) + widen(el[f]));
+                // s + eh + el without FP64 additions of zeros (a thread of a small grid
+                // has a value or two, and every block pays the narrow pipe for them)
+                float e, r;
+                two_sum(eh[f], el[f], e, r);
+                acc[f] = widen(s[f]);
+                if (r != 0.f) acc[f] += widen(e) + widen(r);
+                else if (e != 0.f) acc[f] += widen(e);
             } else {                           // out of the FP32 range, infinite or NaN
                 for (long long c = beg + threadIdx.x; c < end; c += 256) acc[f] += widen(q[f * N + c]);
             }
