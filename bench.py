@@ -39,9 +39,9 @@ UNIT = "zone-updates/s"
 # formulas (add/sub/mul = 1, FMA = 2, div/sqrt = 1): eigen-structure 100,
 # interface average 16, central flux 35, differences of the stencil 70,
 # their projection 10 x 50, split differences and two phi_N per field
-# 7 x 103 (the smoothness indicators as quadratic forms that share eps and
-# a square, phi_N as N / (3 W) - q / 12), back-projection 80.
-SWEEP_FLOPS_PER_INTERFACE = 1522
+# 7 x 102 (the smoothness indicators as completed squares that share one with
+# eps, 12 phi_N of a side as one sum over W), back-projection 80.
+SWEEP_FLOPS_PER_INTERFACE = 1515
 SWEEP_FLOPS_PER_STAGED_CELL = 80
 
 # DRAM bytes (dram__bytes_read.sum + dram__bytes_write.sum) per launch of the
@@ -49,8 +49,8 @@ SWEEP_FLOPS_PER_STAGED_CELL = 80
 # benchmark times (profiles/sweep_traffic_fp32_turbulence256.md); reported
 # only at that size and while the sweep sources hash to SWEEP_TRAFFIC_SOURCES.
 SWEEP_TRAFFIC_N = 256
-SWEEP_TRAFFIC = {"sweep_x": 1178.32e6, "sweep_y": 982.53e6, "sweep_z": 983.33e6}
-SWEEP_TRAFFIC_SOURCES = "45a70bfd88897158"
+SWEEP_TRAFFIC = {"sweep_x": 1181.32e6, "sweep_y": 983.98e6, "sweep_z": 985.41e6}
+SWEEP_TRAFFIC_SOURCES = "2c15e783d94b8a42"
 
 
 def sweep_sources_hash() -> str:

@@ -231,7 +231,8 @@ enum {
     WB_K_CFL = 4,         /* CFL max reduction                                */
     WB_K_DT = 5,          /* dt from the reduced speed                        */
     WB_K_TOTALS = 6,      /* conserved totals (two kernels)                   */
-    WB_K_EMF = 7,         /* edge EMFs of constrained transport               */
+    WB_K_EMF = 7,         /* edge EMFs of constrained transport (no launch of
+                             its own on small grids: part of the update)      */
     WB_NKERNEL = 8
 };
 

@@ -336,7 +336,7 @@ totals_pass1(const T* __restrict__ q, long long N, long long chunk, double* __re
     if constexpr (sizeof(T) == 4) {
         // FP32 values are added in FP32 with every rounding error kept: s the
         // running sum, eh + el the sum of its errors (two-sum at both levels,
-        // el rounds at 2^-72 of the sum), joined in FP64 at the end.  An FP64
+        // el rounds at 2^-72 of the sum), added in FP64 at the end.  An FP64
         // addition per value was the bound (the pipe 79 % busy): 192^3, totals
         // of a state 153 -> 91 us with the host's part.
         float s[8] = {0, 0, 0, 0, 0, 0, 0, 0}, eh[8] = {0, 0, 0, 0, 0, 0, 0, 0}, el[8] = {0, 0, 0, 0, 0, 0, 0, 0};

@@ -4,15 +4,15 @@
 // One interface per thread.  FP64 takes the interface arithmetic below
 // (sweep_flux), which counts operations of the FP64 pipe (two per clock and SM
 // on this GPU, 87 % busy, everything else hidden behind it): smoothness
-// indicators of ten operations and one reciprocal for the two phi_N of a field (60
-// instead of 83 operations), three-operation reciprocals, Alfven rows that act
+// indicators of ten operations and one reciprocal for the two phi_N of a field
+// (60 instead of 83 operations), three-operation reciprocals, Alfven rows that act
 // on the differences directly.  96^3, x + y + z sweep of a step: 21.3 -> 17.6
 // ms; three and four blocks per SM (168 and 128 registers) are no faster.
 // FP32 takes the one of wb_sweep.cuh (interface_flux), which packs the U and F
 // differences of a stencil step, and here the two sides of phi_N, in the lanes
-// of Blackwell's packed FP32 instructions: 1 320 to 1 335 instructions per
-// interface (1 454 before), issued on 59 to 61 % of cycles by sixteen warps per
-// SM.  256^3, x, y, z sweeps of a step: 2.88 / 2.83 / 3.01 -> 2.70 / 2.77 / 2.80
+// of Blackwell's packed FP32 instructions: 1 333 to 1 348 instructions per
+// interface (1 454 before), issued on 60 to 62 % of cycles by sixteen warps per
+// SM.  256^3, x, y, z sweeps of a step: 2.88 / 2.83 / 3.01 -> 2.71 / 2.77 / 2.79
 // ms.  Two interfaces per thread (neighbouring pencils in the two lanes) need
 // only 1 107 instructions per interface, but 200 to 255 registers: eight warps
 // per SM issue on 41 % of cycles, and with the staging moved to further warps
